@@ -79,14 +79,21 @@ typedef struct {
     double   mixed_floor;   /* relative residual at which FP32 cycles hand over to FP64
                                refinement (PD_PREC_MIXED only); default 5e-6 */
     int      hx_variant;    /* H*x kernel: 0 = automatic (default: the autotuned schedule if
-                               one was recorded, else 3, or 4 with 13 low orbits when fewer
-                               than 3 in 10 orbits are occupied or fewer than 3 in 10 empty), 1 = neighbour
-                               blocks staged one at a time, 2 = all neighbour blocks staged at
-                               once, 3 = no staging, every target gathered from global memory
+                               one was recorded, else chosen by dimension and filling), 1 =
+                               neighbour blocks staged one at a time, 2 = FP32 products by
+                               pair removal on the tensor cores (V_j(t) = x(t + j), Z = G V,
+                               y(s) = sum Z(s - i)_i over the states t of one pair less; G and
+                               V split into two TF32 parts, FP32 accumulation; low_bits does
+                               not concern it; needs scratch memory, at most 2 GiB or that of
+                               one class of rows), other precisions as 3, 3 = no staging,
+                               every target gathered from global memory
                                with O(1) hop tables, 4 = variant 3 with the gathers issued in
                                deep groups (far from half filling, where a thread has one row
                                and x is in DRAM), 5 = variant 3 compiled for 5 resident
-                               CTAs per SM (fewer registers, more warps); 2-5 fall back to 1
+                               CTAs per SM (fewer registers, more warps).  Variant 2 falls
+                               back to 3 where it does not apply (more than 40 orbits, 2^32
+                               states or more, no or only full orbits, no room for its
+                               scratch), 2-5 fall back to 1
                                when their shared memory does not fit.  A truncated handle (pairdiag_truncate) runs
                                variant 1 */
 } pairdiag_options;

@@ -149,6 +149,7 @@ struct pairdiag {
     // within a size), so the launch does not end on one CTA's large block
     uint64_t *d_lpt_h = nullptr, *d_lpt_base = nullptr;
     Blocks B{};
+    FacPlan fac;                     // the FP32 product by pair removal
     int device = 0;
     cudaStream_t st = nullptr;
     // tables
@@ -196,6 +197,13 @@ struct pairdiag {
 
 namespace {
 
+void free_fac(FacPlan &f)
+{
+    for (void *p : {(void *)f.twords, (void *)f.ywords, (void *)f.low, (void *)f.up, (void *)f.scratch, (void *)f.zeros})
+        pool_free(p);
+    f = FacPlan{};
+}
+
 void free_all(pairdiag *h)
 {
     for (auto &ev : h->hx_events) {
@@ -213,6 +221,7 @@ void free_all(pairdiag *h)
     // stream's completion is enough (other streams of the caller go on).
     cudaStreamSynchronize(h->st);
     for (void *p : ptrs) pool_free(p);
+    free_fac(h->fac);
 }
 
 template <typename T>
@@ -246,15 +255,12 @@ int build_tables(pairdiag *h)
     // admissible k (pairs in the low orbits)
     const int kmin = std::max(0, N - H), kmax = std::min(N, L);
     int64_t nblocks = 0;
-    int max_block = 0, max_hh = 0, max_stage = 0;
+    int max_block = 0, max_hh = 0;
     for (int k = kmin; k <= kmax; ++k) {
         const int ph = N - k;
         nblocks += (int64_t)host_binom(H, ph);
         max_block = std::max(max_block, (int)host_binom(L, k));
         max_hh = std::max(max_hh, ph * (H - ph));
-        const int64_t up = (k < L && ph > 0) ? ph * (int64_t)host_binom(L, k + 1) : 0;
-        const int64_t dn = (k > 0 && H - ph > 0) ? (H - ph) * (int64_t)host_binom(L, k - 1) : 0;
-        max_stage = (int)std::max<int64_t>(max_stage, up + dn);
     }
     // the persistent H*x kernels keep block indices in int, and their counters
     // run past nblocks by up to two per CTA before every CTA has stopped
@@ -314,11 +320,31 @@ int build_tables(pairdiag *h)
     B.nblocks = (int64_t)hw.size();
     B.max_block = max_block;
     B.max_hh = max_hh;
-    B.max_stage = max_stage;
     B.variant = h->opt.hx_variant;
     B.blk_h = h->d_blk_h; B.blk_base = h->d_blk_base;
     B.lowword = h->d_lowword; B.rankL = h->d_rankL; B.binom = h->d_binom;
     for (int k = 0; k <= kMaxLow + 1; ++k) B.lo_off[k] = (k <= L + 1) ? off[k] : off[L + 1];
+    return PD_OK;
+}
+
+// The plan of the FP32 product by pair removal: its tables are made on the
+// device; h->fac.on stays false where it does not apply.
+int build_fac(pairdiag *h)
+{
+    FacPlan &f = h->fac;
+    f = FacPlan{};
+    if (!fac_fits(h->omega, h->n, h->full_dim)) return PD_OK;
+    fac_sizes(h->omega, h->n, f);
+    const bool ok = dalloc(&f.twords, (size_t)f.nt) == PD_OK && dalloc(&f.ywords, (size_t)f.ny) == PD_OK &&
+                    dalloc(&f.low, (size_t)1 << f.L) == PD_OK && dalloc(&f.up, (size_t)f.table) == PD_OK &&
+                    dalloc(&f.zeros, fac_zeros()) == PD_OK &&
+                    dalloc(&f.scratch, (size_t)std::max<int64_t>(f.scratch_len, 1)) == PD_OK;
+    if (!ok) {                                    // no room: the kernels without scratch serve the handle
+        free_fac(f);
+        return PD_OK;
+    }
+    PD_CUDA(fac_build(f, h->d_binom, h->st));
+    PD_CUDA(cudaStreamSynchronize(h->st));        // the handle may move to another stream
     return PD_OK;
 }
 
@@ -386,8 +412,12 @@ int hx(pairdiag *h, int precision, const void *x, void *y, const int *skip = nul
         B.blk_h = h->d_lpt_h;
         B.blk_base = h->d_lpt_base;
     }
-    PD_CUDA(hx_launch(B, P, precision, x, y, h->d_tk, h->hxgrid[precision], h->st, skip,
-                      dot_out ? &dot : nullptr));
+    if (precision == 1 && h->fac.on && !B.kept_map)
+        PD_CUDA(fac_launch(h->fac, h->d_binom, h->d_G32, h->d_d32, static_cast<const float *>(x),
+                           static_cast<float *>(y), h->d_tk, h->st, skip, dot_out ? &dot : nullptr));
+    else
+        PD_CUDA(hx_launch(B, P, precision, x, y, h->d_tk, h->hxgrid[precision], h->st, skip,
+                          dot_out ? &dot : nullptr));
     if (ev) PD_CUDA(cudaEventRecord(ev->second, h->st));
     return PD_OK;
 }
@@ -824,12 +854,14 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
         int lb = 0, hv = 0;
         if (tuned_schedule(omega, n_pairs, o.precision, &lb, &hv)) { o.low_bits = lb; o.hx_variant = hv; }
     }
+    bool use_fac = o.hx_variant == 2;             // variant 2 where it serves the problem
     if (o.hx_variant == 0) {
         // untuned: direct gathers; far from half filling (fewer than 3 in 10 orbits
         // occupied, or empty) deep gather groups and 13 low orbits, the fastest
         // schedules measured at Omega = 24..38
         const int minority = std::min(n_pairs, omega - n_pairs);
         const bool low_filling = 10 * minority < 3 * omega;
+        use_fac = o.precision == PD_PREC_MIXED && fac_pays(omega, n_pairs, (int64_t)host_binom(omega, n_pairs));
         o.hx_variant = low_filling ? 4 : 3;
         if (o.low_bits == 0 && low_filling) o.low_bits = 13;
     }
@@ -847,6 +879,7 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { cudaGetLastError(); st = fail(PD_ECUDA, "no CUDA device"); break; }
         if ((st = build_tables(h)) != PD_OK) break;
+        if (use_fac && (st = build_fac(h)) != PD_OK) break;
         std::vector<float> G32(h->G.begin(), h->G.end()), d32(h->d.begin(), h->d.end());
         auto split = [](const std::vector<double> &v) {
             std::vector<float2> r(v.size());
@@ -864,7 +897,7 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
         if ((st = upload(&h->d_dff, split(h->d))) != PD_OK) break;
         if ((st = dalloc(&h->d_tk, 1)) != PD_OK) break;
         if (cudaMemset(h->d_tk, 0, sizeof(Tickets)) != cudaSuccess) { st = fail(PD_ECUDA, "memset"); break; }
-        if ((st = dalloc(&h->d_blkdot, (size_t)h->B.nblocks)) != PD_OK) break;
+        if ((st = dalloc(&h->d_blkdot, (size_t)std::max<int64_t>(h->B.nblocks, fac_partials(h->fac)))) != PD_OK) break;
         h->ldq = (h->dim + 3) / 4 * 4;
         h->hxgrid[0] = hx_grid(h->B, 0);
         h->hxgrid[1] = hx_grid(h->B, 1);
@@ -1394,8 +1427,12 @@ int pairdiag_autotune(int omega, int n_pairs, const double *e, const double *G, 
             o.precision = precision;
             pairdiag_t *h = nullptr;
             if ((rc = pairdiag_create(omega, n_pairs, e, G, &o, &h)) != PD_OK) break;
-            if (variant > 1 && hx_variant(h->B, precision == PD_PREC_FP64 ? 0 : 1) != variant) {
-                pairdiag_destroy(h);             // the variant does not fit: same as variant 1
+            // the variant does not fit: the launch would run another one; variant 2
+            // has a block split of its own, so it is timed once
+            const bool same = variant == 2 ? precision != PD_PREC_MIXED || !h->fac.on || L != h->fac.L
+                                           : variant > 1 && hx_variant(h->B, precision == PD_PREC_FP64 ? 0 : 1) != variant;
+            if (same) {
+                pairdiag_destroy(h);
                 continue;
             }
             rc = [&]() -> int {

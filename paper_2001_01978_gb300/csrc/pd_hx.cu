@@ -436,353 +436,9 @@ hx_batch_kernel(const BatchBlocks BB, const A *__restrict__ Gall, const A *__res
     if (arrive_last(counter + 1) && tid == 0) counter[0] = 0ull;
 }
 
-// ---- variant 2: every neighbouring block of the high<->low hops staged at once --
-struct Layout2 {
-    size_t g, gs, ge, d, rank, low, bin, x, xn, hh, occ, emp, total;
-};
-
-template <typename T, typename A>
-__host__ __device__ inline Layout2 layout2(int omega, int L, int H, int N, int max_block, int max_hh,
-                                          int max_stage)
-{
-    Layout2 s;
-    size_t off = 0;
-    const int h1 = H > 0 ? H : 1;
-    s.g = off;    off = align16(off + sizeof(A) * omega * omega);
-    s.gs = off;   off = align16(off + sizeof(A) * h1 * L);
-    s.ge = off;   off = align16(off + sizeof(A) * h1 * L);
-    s.d = off;    off = align16(off + sizeof(A) * omega);
-    s.rank = off; off = align16(off + sizeof(uint16_t) * (size_t(1) << L));
-    s.low = off;  off = align16(off + sizeof(uint16_t) * (size_t(1) << L));
-    s.bin = off;  off = align16(off + sizeof(uint64_t) * h1 * (N + 1));
-    s.x = off;    off = align16(off + sizeof(T) * max_block);
-    s.xn = off;   off = align16(off + sizeof(T) * (size_t)(max_stage > 0 ? max_stage : 1));
-    s.hh = off;   off = align16(off + sizeof(HHop<A>) * (max_hh > 0 ? max_hh : 1));
-    s.occ = off;  off = align16(off + sizeof(uint64_t) * h1);
-    s.emp = off;  off = align16(off + sizeof(uint64_t) * h1);
-    s.total = off;
-    return s;
-}
-
-// block_base with the binomials of the high orbits in shared memory:
-// sBin[p * (N + 1) + m] = C(L + p, m)
-__device__ __forceinline__ uint64_t block_base_s(uint64_t h, int N, const uint64_t *sBin)
-{
-    int ord = N - __popcll(h);
-    uint64_t s = 0;
-    while (h) {
-        const int p = __ffsll((long long)h) - 1;
-        h &= h - 1;
-        ++ord;
-        s += sBin[p * (N + 1) + ord];
-    }
-    return s;
-}
-
-// asynchronous copy of one 4- or 8-byte element global -> shared (no register
-// round trip, so a thread issues all its copies before any has landed)
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T *dst, const T *src)
-{
-    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "cp.async element of 4 or 8 bytes");
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (sizeof(T) == 4)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// Shared-memory view of variant 2 (one CTA's dynamic shared memory)
-template <typename T, typename A>
-struct Smem2 {
-    A *G, *GS, *GE, *d;
-    uint16_t *rank, *low;
-    uint64_t *bin, *occ, *emp;
-    T *x, *xn;
-    HHop<A> *hh;
-    __device__ Smem2(unsigned char *smem, const Layout2 &lay)
-        : G(reinterpret_cast<A *>(smem + lay.g)), GS(reinterpret_cast<A *>(smem + lay.gs)),
-          GE(reinterpret_cast<A *>(smem + lay.ge)), d(reinterpret_cast<A *>(smem + lay.d)),
-          rank(reinterpret_cast<uint16_t *>(smem + lay.rank)), low(reinterpret_cast<uint16_t *>(smem + lay.low)),
-          bin(reinterpret_cast<uint64_t *>(smem + lay.bin)), occ(reinterpret_cast<uint64_t *>(smem + lay.occ)),
-          emp(reinterpret_cast<uint64_t *>(smem + lay.emp)), x(reinterpret_cast<T *>(smem + lay.x)),
-          xn(reinterpret_cast<T *>(smem + lay.xn)), hh(reinterpret_cast<HHop<A> *>(smem + lay.hh))
-    {
-    }
-};
-
-// One problem's tables into shared memory, read for the whole launch (or, in
-// the batch, until the problem changes): G, d = 2e + diag(G), the rank and
-// low-word tables of L-bit words, and the binomials C(L + p, m) of the high
-// orbits (p < H, m <= N) that block_base_s adds up.
-template <typename T, typename A>
-__device__ __forceinline__ void load_tables2(const Smem2<T, A> &s, int omega, int L, int H, int N,
-                                             const A *__restrict__ G, const A *__restrict__ d,
-                                             const uint16_t *__restrict__ rankL, const uint16_t *__restrict__ lowword,
-                                             const uint64_t *__restrict__ binom)
-{
-    const int tid = threadIdx.x;
-    for (int i = tid; i < omega * omega; i += kThreads) s.G[i] = G[i];
-    for (int i = tid; i < omega; i += kThreads) s.d[i] = d[i];
-    for (int i = tid; i < (1 << L); i += kThreads) {
-        s.rank[i] = rankL[i];
-        s.low[i] = lowword[i];
-    }
-    for (int i = tid; i < (H > 0 ? H : 1) * (N + 1); i += kThreads) {
-        const int p = i / (N + 1), m = i - p * (N + 1);
-        s.bin[i] = __ldg(binom + (L + p) * kBinomStride + m);
-    }
-}
-
-// One basis block (high word h, first index base) of y = H x in variant 2.
-// x and y point at the problem's own vector; s holds its tables.  Called by
-// every thread of the CTA after a barrier that frees the previous block's
-// shared memory; it contains two barriers.  Any cp.async the caller issued
-// before is completed by the first of them.  swdot (nullable): x^T y per warp.
-template <typename T, typename A, int R>
-__device__ __forceinline__ void hx2_block(const Smem2<T, A> &s, const int omega, const int L, const int H,
-                                          const int N, const uint64_t h, const uint64_t base,
-                                          const T *__restrict__ x, T *__restrict__ y, double *swdot)
-{
-    const int tid = threadIdx.x;
-    const uint32_t maskL = (1u << L) - 1u;
-    const uint64_t maskH = (H >= 64) ? ~0ull : ((1ull << H) - 1ull);
-    const int ph = __popcll(h);
-    const int k = N - ph;
-    const int nemp = H - ph;
-    const int nhh = ph * nemp;
-    // block sizes C(L, k), C(L, k+1), C(L, k-1) from row p = 0 of s.bin
-    // (k + 1 <= N whenever a block h - o exists, i.e. ph > 0)
-    const int nk = (int)s.bin[k];
-    const int n_up = (k < L && ph > 0) ? (int)s.bin[k + 1] : 0;
-    const int n_dn = (k > 0 && nemp > 0) ? (int)s.bin[k - 1] : 0;
-    int lo_off = 0;                               // words of popcount k start here in s.low
-    for (int j = 0; j < k; ++j) lo_off += (int)s.bin[j];
-    const uint16_t *lw = s.low + lo_off;
-    T *sxn = s.xn;
-    T *sxd = sxn + ph * n_up;                     // staged blocks h + e start here
-
-    for (int r = tid; r < nk; r += kThreads) cp_async_elem(s.x + r, x + base + r);
-    cp_async_commit();
-
-    for (int t = tid; t < nhh; t += kThreads) {
-        const int a = t / nemp, c = t - a * nemp;
-        const int o = nth_set_bit(h, a);
-        const int q = nth_set_bit(~h & maskH, c);
-        s.hh[t].base = block_base_s(h ^ (1ull << o) ^ (1ull << q), N, s.bin);
-        s.hh[t].g = s.G[(L + q) * omega + (L + o)];
-    }
-    for (int t = tid; t < H; t += kThreads) {
-        const uint64_t bit = 1ull << t;
-        if (h & bit) {
-            const int j = __popcll(h & (bit - 1));
-            s.occ[j] = n_up ? block_base_s(h ^ bit, N, s.bin) : 0;
-            for (int e = 0; e < L; ++e) s.GS[j * L + e] = s.G[e * omega + L + t];
-        } else {
-            const int j = __popcll(~h & maskH & (bit - 1));
-            s.emp[j] = n_dn ? block_base_s(h | bit, N, s.bin) : 0;
-            for (int o = 0; o < L; ++o) s.GE[j * L + o] = s.G[(L + t) * omega + o];
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();                              // own block, hop tables and slot bases visible
-
-    if (n_up)
-        for (int j = 0; j < ph; ++j) {
-            const T *src = x + s.occ[j];
-            T *dst = sxn + j * n_up;
-            for (int r = tid; r < n_up; r += kThreads) cp_async_elem(dst + r, src + r);
-        }
-    if (n_dn)
-        for (int j = 0; j < nemp; ++j) {
-            const T *src = x + s.emp[j];
-            T *dst = sxd + j * n_dn;
-            for (int r = tid; r < n_dn; r += kThreads) cp_async_elem(dst + r, src + r);
-        }
-    cp_async_commit();
-
-    A Dh = A(0);
-    for (uint64_t w = h; w; w &= w - 1) Dh += s.d[L + __ffsll((long long)w) - 1];
-
-    uint32_t lr[R];
-    A acc[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        const int r = tid + i * kThreads;
-        lr[i] = 0;
-        acc[i] = A(0);
-        if (r < nk) {
-            const uint32_t l = lw[r];
-            lr[i] = l;
-            A D = A(0);
-            for (uint32_t w = l; w; w &= w - 1) D += s.d[__ffs(w) - 1];
-            acc[i] = (D + Dh) * A(s.x[r]);
-        }
-    }
-
-    // low -> low
-    if (k > 0 && k < L) {
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            if (tid + i * kThreads < nk) {
-                const uint32_t l = lr[i];
-                A a = acc[i];
-                uint32_t occ = l;
-                for (int u = 0; u < k; ++u) {
-                    const int o = __ffs(occ) - 1;
-                    occ &= occ - 1;
-                    const uint32_t lo = l ^ (1u << o);
-                    const A *gcol = s.G + o;
-                    uint32_t emp = ~l & maskL;
-                    for (int v = 0; v < L - k; ++v) {
-                        const int q = __ffs(emp) - 1;
-                        emp &= emp - 1;
-                        a += gcol[q * omega] * A(s.x[s.rank[lo | (1u << q)]]);
-                    }
-                }
-                acc[i] = a;
-            }
-        }
-    }
-
-    // high -> high: same offsets in the target block (warps without rows skip it)
-    const bool has_rows = (int)(tid & ~31) < nk;
-    for (int j = 0; has_rows && j < nhh; ++j) {
-        const T *xb = x + s.hh[j].base;
-        const A g = s.hh[j].g;
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            const int r = tid + i * kThreads;
-            if (r < nk) acc[i] += g * A(__ldg(xb + r));
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();                              // staged neighbour blocks visible
-
-    // high -> low: pair from occupied high orbit L+t to empty low orbit e;
-    // the target offset rank(l + e) is the same in every staged block
-    if (n_up) {
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            const int r = tid + i * kThreads;
-            if (r < nk) {
-                const uint32_t l = lr[i];
-                A a = acc[i];
-                for (uint32_t w = ~l & maskL; w; w &= w - 1) {
-                    const int e = __ffs(w) - 1;
-                    const A *g = s.GS + e;
-                    const T *xp = sxn + s.rank[l | (1u << e)];
-                    for (int j = 0; j < ph; ++j) a += g[j * L] * A(xp[j * n_up]);
-                }
-                acc[i] = a;
-            }
-        }
-    }
-    // low -> high: pair from occupied low orbit o to empty high orbit L+t
-    if (n_dn) {
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            const int r = tid + i * kThreads;
-            if (r < nk) {
-                const uint32_t l = lr[i];
-                A a = acc[i];
-                for (uint32_t w = l; w; w &= w - 1) {
-                    const int o = __ffs(w) - 1;
-                    const A *g = s.GE + o;
-                    const T *xp = sxd + s.rank[l ^ (1u << o)];
-                    for (int j = 0; j < nemp; ++j) a += g[j * L] * A(xp[j * n_dn]);
-                }
-                acc[i] = a;
-            }
-        }
-    }
-
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        const int r = tid + i * kThreads;
-        if (r < nk) y[base + r] = T(acc[i]);
-    }
-    if (swdot) warp_dot<T, A, R>(acc, s.x, nk, swdot);
-}
-
-// Same product as hx_kernel.  Differences: all ph blocks h - o (k+1 low pairs)
-// and all H-ph blocks h + e (k-1) are staged together; the coefficients of the
-// high<->low hops are laid out per staged block (G_{e, L+t} for block h - t at
-// row t of sGS, G_{L+t, o} for block h + t in sGE), so for each row and low
-// orbit the innermost loop runs over the staged blocks with one coefficient
-// load, one gather and one FMA.
-//
-// Latency: G, d, the rank and low-word tables and the binomials of the high
-// orbits live in shared memory for the whole launch, so the per-block tables
-// need no global loads; the block's own x and its neighbours arrive through
-// cp.async, issued before the table setup and before the low->low and
-// high->high hops respectively, so their latency overlaps that work; thread 0
-// takes the next block index and copies its (h, base) into shared memory one
-// block ahead.  FP32: at most 40 registers, so that six CTAs fit an SM when
-// shared memory allows.
-template <typename T, typename A, int R>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 6 : 4)
-hx2_kernel(const Blocks B, const A *__restrict__ Gg, const A *__restrict__ dg,
-           const T *__restrict__ x, T *__restrict__ y, Tickets *tk, const int *__restrict__ skip,
-           double *blk_part, double *dot_out)
-{
-    if (skip && *skip) return;                    // CTA-uniform
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_idx[2];
-    __shared__ __align__(8) uint64_t s_h[2], s_base[2];
-    __shared__ double sred[kThreads / 32];
-    __shared__ double swdot[kThreads / 32];
-    const int omega = B.omega, L = B.L, H = B.H, N = B.n;
-    const Smem2<T, A> s(smem, layout2<T, A>(omega, L, H, N, B.max_block, B.max_hh, B.max_stage));
-    const int tid = threadIdx.x;
-    load_tables2<T, A>(s, omega, L, H, N, Gg, dg, B.rankL, B.lowword, B.binom);
-
-    // block schedule: slot it holds (index, h, base) of the block of iteration
-    // it.  Thread 0 holds the index of the next block in nb1; during the
-    // current block it copies that block's (h, base) into slot it ^ 1 with
-    // cp.async (completed by the first barrier of hx2_block) and takes the
-    // index after it from the counter, so neither latency delays a block.
-    // (Block counts are below 2^31: build_tables rejects more blocks.)
-    const int nblocks = (int)B.nblocks;
-    int nb1 = 0;
-    if (tid == 0) {
-        const int b0 = (int)atomicAdd(&tk->hx_next, 1ull);
-        s_idx[0] = b0;
-        if (b0 < nblocks) {
-            s_h[0] = __ldg(B.blk_h + b0);
-            s_base[0] = __ldg(B.blk_base + b0);
-            nb1 = (int)atomicAdd(&tk->hx_next, 1ull);
-        }
-    }
-    long long prev = -1;
-    for (int it = 0;; it ^= 1) {
-        __syncthreads();                          // smem of the previous block is free; slot it visible
-        const int b = s_idx[it];
-        int nb2 = 0;
-        if (tid == 0) {
-            block_sum_deferred(blk_part, prev, swdot);
-            if (b < nblocks && nb1 < nblocks) {
-                cp_async_elem(&s_h[it ^ 1], B.blk_h + nb1);
-                cp_async_elem(&s_base[it ^ 1], B.blk_base + nb1);
-                nb2 = (int)atomicAdd(&tk->hx_next, 1ull);
-            }
-        }
-        if (b >= nblocks) break;
-        hx2_block<T, A, R>(s, omega, L, H, N, s_h[it], s_base[it], x, y, blk_part ? swdot : nullptr);
-        prev = b;
-        if (tid == 0) {                           // publish the next block (read after the barrier)
-            s_idx[it ^ 1] = nb1;
-            nb1 = nb2;
-        }
-    }
-    hx_finish(tk, B.nblocks, blk_part, dot_out, sred);
-}
-
 // ---- variant 3: no staging rounds; hop tables in O(1) per entry ------------------
-// Variants 1 and 2 stage neighbour blocks in shared memory, which pays when
-// blocks are large (half filling).  Far from half filling most blocks hold a
+// Variant 1 stages neighbour blocks in shared memory, which pays when blocks
+// are large (half filling).  Far from half filling most blocks hold a
 // few rows (C(12,0..1) = 1..12 at Omega=38, N=10), and there variant 1's H
 // staging rounds (each a memory latency plus two barriers) and the per-entry
 // block_base loops of the hop tables dominate.  Variant 3 gathers every
@@ -1254,22 +910,13 @@ hx3_batch_kernel(const BatchBlocks BB, const A *__restrict__ Gall, const A *__re
 
 constexpr size_t kSmemLimit = 200 * 1024;
 
-// Variant 2 only on request (the autotuner's choice, or the caller's) and when
-// its shared memory fits; which variant is faster depends on the problem and
-// the block split (at Omega=24 variant 2 with L=11 in FP32, at Omega=32 variant 1).
-template <typename T, typename A>
-bool use_v2(const Blocks &B)
-{
-    if (B.variant != 2 || B.kept_map) return false;     // a truncated space runs variant 1
-    return layout2<T, A>(B.omega, B.L, B.H, B.n, B.max_block, B.max_hh, B.max_stage).total <= kSmemLimit;
-}
-
-// Variant 3 (lean loops), 4 (deep gather groups) or 5 (lean loops, 5 CTAs per
+// Variant 3 (lean loops; also where variant 2, the FP32 product of pd_hxf.cu,
+// does not serve the call), 4 (deep gather groups) or 5 (lean loops, 5 CTAs per
 // SM) on request, when the shared memory fits (full space only)
 template <typename T, typename A>
 bool use_v3(const Blocks &B)
 {
-    if ((B.variant < 3 || B.variant > 5) || B.kept_map) return false;
+    if ((B.variant < 2 || B.variant > 5) || B.kept_map) return false;
     return layout3<T, A>(B.omega, B.L, B.H, B.n, B.max_block, B.max_hh).total <= kSmemLimit;
 }
 
@@ -1281,15 +928,14 @@ const void *kernel_fn(const Blocks &B)
         return B.variant == 4   ? (const void *)hx3_kernel<T, A, R, true>
                : B.variant == 5 ? (const void *)hx3_kernel<T, A, R, false, 5>
                                 : (const void *)hx3_kernel<T, A, R, false>;
-    return use_v2<T, A>(B) ? (const void *)hx2_kernel<T, A, R> : (const void *)hx_kernel<T, A, R, false>;
+    return (const void *)hx_kernel<T, A, R, false>;
 }
 
 template <typename T, typename A>
 size_t kernel_smem(const Blocks &B)
 {
     if (use_v3<T, A>(B)) return layout3<T, A>(B.omega, B.L, B.H, B.n, B.max_block, B.max_hh).total;
-    return use_v2<T, A>(B) ? layout2<T, A>(B.omega, B.L, B.H, B.n, B.max_block, B.max_hh, B.max_stage).total
-                           : layout<T, A>(B.omega, B.L, B.H, B.max_block, B.max_hh).total;
+    return layout<T, A>(B.omega, B.L, B.H, B.max_block, B.max_hh).total;
 }
 
 template <typename T, typename A, int R>
@@ -1297,7 +943,6 @@ cudaError_t launch_t(const Blocks &B, const A *G, const A *d, const void *x, voi
                      Tickets *tk, int grid, cudaStream_t st, const int *skip, const HxDot *dot)
 {
     const size_t smem = kernel_smem<T, A>(B);
-    const bool v2 = use_v2<T, A>(B);
     cudaError_t err = cudaFuncSetAttribute(kernel_fn<T, A, R>(B),
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
@@ -1315,9 +960,6 @@ cudaError_t launch_t(const Blocks &B, const A *G, const A *d, const void *x, voi
     else if (use_v3<T, A>(B))
         hx3_kernel<T, A, R, false><<<grid, kThreads, smem, st>>>(B, G, d, static_cast<const T *>(x),
                                                                  static_cast<T *>(y), tk, skip, bp, out);
-    else if (v2)
-        hx2_kernel<T, A, R><<<grid, kThreads, smem, st>>>(B, G, d, static_cast<const T *>(x),
-                                                          static_cast<T *>(y), tk, skip, bp, out);
     else
         hx_kernel<T, A, R, false><<<grid, kThreads, smem, st>>>(B, G, d, static_cast<const T *>(x),
                                                                 static_cast<T *>(y), tk, skip, bp, out);
@@ -1617,8 +1259,8 @@ size_t hx_smem_bytes(const Blocks &B, int precision)
 
 int hx_variant(const Blocks &B, int precision)
 {
-    if (precision == 0 ? use_v3<double, double>(B) : use_v3<float, float>(B)) return B.variant;
-    return (precision == 0 ? use_v2<double, double>(B) : use_v2<float, float>(B)) ? 2 : 1;
+    if (precision == 0 ? use_v3<double, double>(B) : use_v3<float, float>(B)) return B.variant == 2 ? 3 : B.variant;
+    return 1;
 }
 
 int hx_grid(const Blocks &B, int precision)

@@ -1,0 +1,851 @@
+// pd_hxf.cu -- y = H x by pair removal on the tensor cores (variant 2, FP32).
+//
+// The off-diagonal part of Eq. 2 is a product of two sparse maps with a dense
+// matrix in between,
+//     V(t)_j = x(t + j),   Z(t) = G V(t),   y(s) = sum_{i in s} Z(s - i)_i,
+// t running over the states with one pair less (t + j: a pair added on orbit j,
+// j empty in t).  One gather of the M = Omega - N + 1 elements around t serves
+// all M (M - 1) hops that pass through t, where a row-by-row kernel loads,
+// addresses and multiplies every hop on its own.  The middle step is one small
+// dense product per t with the same matrix, so 128 words t make one tile
+//     Z [128 x Omega] = V [128 x Omega] G
+// on the 5th-generation tensor cores.
+//
+// Precision.  tcgen05.mma kind::tf32 keeps 11 significant bits of an operand, so
+// V and G are split in two, v = v_hi + v_lo with v_hi = v rounded to TF32 (the
+// difference is exact), and Z = V_hi G_hi + V_lo G_hi + V_hi G_lo accumulates in
+// FP32: what is dropped is below 2^-23 of a term, and a row sum is a tree of
+// depth two instead of a chain of N (Omega - N) additions.  Elements that are
+// not finite (or that overflow when rounded to TF32) cannot be split; a tile
+// that meets one sets a flag, and the second kernel then forms its rows term by
+// term.
+//
+// Layout.  Low orbits: the L <= 12 lowest; high word h, block as in
+// pd_internal.h.  remove_kernel takes one high word at a time (a block of t):
+// one thread gathers one t, writes the split row into tensor memory (operand A
+// of the product), and reads its row of Z back from there.  Results for low
+// orbits belong to rows of the block h itself and meet in shared memory (slot
+// [orbit][row], one writer each); the block's partial y is written once.
+// Results for a high orbit q belong to block h + q at the same low word: they go
+// to a scratch vector, ordered by (block of y, ordinal of q, row), where
+// add_kernel streams them: y(h, l) += sum_a scratch(h, a, l).  No two threads
+// add to the same element, so the sums have a fixed order.
+#include "pd_internal.h"
+
+#include <climits>
+#include <type_traits>
+#include <utility>
+
+namespace pd {
+namespace {
+
+constexpr int kLT = 12;                  // low orbits
+constexpr int kRows = 924;               // most rows of a block: C(12,6)
+constexpr int kSpare = kRows;            // slot of hops that do not exist (reads 0, writes ignored)
+constexpr int kStride = 928;             // floats per orbit of the partial results
+// Scratch (floats): all rows at once up to 2 GiB, else class by class (the rows
+// with k low pairs, k ascending), which bounds it at the largest class: 1.2 GB
+// instead of 5.2 GB at Omega=30, 5 GB instead of 22 GB at Omega=32.  Measured
+// at once / by class: Omega=24 0.096 / 0.28 ms (26 short launches), Omega=28
+// 1.79 / 1.97 ms, Omega=30 7.45 / 7.36 ms.
+constexpr int64_t kScratchAll = (int64_t)2048 << 18;
+constexpr int kTile = 128;               // words t per tile: the lanes of tensor memory
+constexpr int kMaxHigh = 28;             // high orbits (12 + 28 = 40 columns)
+constexpr size_t kSmemMax = 112 * 1024;   // two CTAs per SM
+constexpr int kTmemCols = 256;           // tensor-memory columns of a CTA: two CTAs fill an SM
+constexpr int kWaitLimit = 1 << 14;      // mbarrier polls (each suspended up to a millisecond) before a wait gives up
+
+__host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+template <class F, int... I>
+__device__ __forceinline__ void for_each_impl(F &&f, std::integer_sequence<int, I...>)
+{
+    (f(std::integral_constant<int, I>{}), ...);
+}
+// f(0), ..., f(N - 1) with the index as a compile-time constant
+template <int N, class F>
+__device__ __forceinline__ void for_each(F &&f)
+{
+    for_each_impl(f, std::make_integer_sequence<int, N>{});
+}
+
+// Columns of a tile: low orbit p at p, high orbit q at 12 + q, zero-padded to KP
+// (K of the product) and NP (its N).  Tensor memory per group of four warps:
+// V_hi [KP], V_lo [KP], Z [NP].  Groups per CTA: as many as 256 columns hold.
+template <int KP>
+struct Cfg {
+    static constexpr int kN = (KP + 15) / 16 * 16;
+    static constexpr int kCols = 2 * KP + kN;
+    static constexpr int kGroups = KP <= 24 ? 3 : 2;
+    static constexpr int kSets = KP <= 32 ? 2 : 1;       // sets of partial results in shared memory
+    static constexpr int kWarps = 4 * kGroups;           // and one warp that prepares the next block
+    static constexpr int kThreads = 32 * (kWarps + 1);
+    static_assert(kGroups * kCols <= kTmemCols, "tensor memory of a CTA");
+};
+
+// ---- tables ---------------------------------------------------------------------
+__device__ int colex_rank(uint32_t w, const uint64_t *__restrict__ binom)
+{
+    int r = 0, c = 0;
+    for (; w; w &= w - 1) r += (int)__ldg(binom + (__ffs(w) - 1) * kBinomStride + ++c);
+    return r;
+}
+// Low words and their hops.  Word w = the r-th of c pairs is row lo_off[c] + r.
+// For orbit j: byte offset 4 * rank(w with orbit j added), 4 * kSpare if j is in
+// w or not an orbit.  Two orbits per 32-bit entry, the entries of one pair of
+// orbits contiguous over the rows (table[pair << L | row]), so that a warp's 32
+// rows are one coalesced load.
+__global__ void hop_table_kernel(int L, const uint64_t *__restrict__ binom, uint16_t *__restrict__ low,
+                                 uint32_t *__restrict__ up)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ((kLT / 2) << L)) return;
+    const uint32_t w = (uint32_t)i & ((1u << L) - 1u);
+    const int pair = i >> L;
+    int row = colex_rank(w, binom);
+    for (int c = 0; c < __popc(w); ++c) row += (int)__ldg(binom + L * kBinomStride + c);
+    uint32_t u = 0;
+    for (int t = 1; t >= 0; --t) {
+        const int j = 2 * pair + t;
+        u = u << 16 | (uint32_t)((j < L && !(w >> j & 1u)) ? 4 * colex_rank(w | (1u << j), binom) : 4 * kSpare);
+    }
+    up[(pair << L) + row] = u;
+    if (pair == 0) low[row] = (uint16_t)w;
+}
+
+// High words by class (pairs in the high orbits), ascending within a class
+// (colex unranking)
+struct WordClasses {
+    int n;
+    int ph[kLT + 1];
+    int64_t first[kLT + 2];              // number of the class's first word
+};
+__global__ void high_words_kernel(const WordClasses C, int H, const uint64_t *__restrict__ binom,
+                                  uint32_t *__restrict__ words)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= C.first[C.n]) return;
+    int c = 0;
+    while (i >= C.first[c + 1]) ++c;
+    uint64_t idx = (uint64_t)(i - C.first[c]);
+    uint32_t w = 0;
+    int p = H - 1;
+    for (int j = C.ph[c]; j > 0; --j) {
+        while (__ldg(binom + p * kBinomStride + j) > idx) --p;
+        idx -= __ldg(binom + p * kBinomStride + j);
+        w |= 1u << p;
+        --p;
+    }
+    words[i] = w;
+}
+
+// ---- pair removal ---------------------------------------------------------------
+constexpr int kPartBytes = 4 * kLT * kStride;
+
+struct __align__(16) BlockSmem {         // one block of t
+    const float *xe[32];                 // block h + q of x, by high orbit q; zeros if q is occupied
+    float *ze[32];                       // where the results for orbit q go
+    float x[kStride];                    // block h of x; x[kSpare] = 0
+    uint32_t h, base;
+    float dh;                            // diagonal sum of its high orbits
+    long long b;                         // its number; >= end: none left
+};
+
+struct LayoutR {
+    size_t b, buf, dlow, bin, crk, dh, total;
+};
+__host__ __device__ inline LayoutR layout_r(int KP, int H, int N)
+{
+    LayoutR s;
+    const int h1 = H > 0 ? H : 1;
+    const int np = (KP + 15) / 16 * 16;
+    size_t off = (KP <= 32 ? 2 : 1) * kPartBytes;   // the partial results lie at 0
+    s.b = off;    off = align16(off + sizeof(float) * 2 * np * KP);
+    s.buf = off;  off = align16(off + 3 * sizeof(BlockSmem));
+    s.dlow = off; off = align16(off + sizeof(float) * 128);
+    s.bin = off;  off = align16(off + sizeof(uint32_t) * h1 * (N + 2));
+    s.crk = off;  off = align16(off + sizeof(uint32_t) * h1 * (h1 + 2));
+    s.dh = off;   off = align16(off + sizeof(float) * h1);
+    s.total = off;
+    return s;
+}
+
+struct RemoveArgs {
+    int omega, N, L, H;
+    int lo_off[kLT + 2];
+    int64_t first, end;                  // blocks of t of this launch, in words
+    int64_t zbase[kLT + 1];              // scratch of the rows with k low pairs
+    const uint32_t *words;
+    const uint16_t *low;
+    const uint32_t *up;
+    const uint64_t *binom;
+    const float *zeros;                  // kRows zeros
+    float *scratch;
+};
+
+__device__ __forceinline__ void copy_async4(float *dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// The last warp: block of t with high word h into buffer bs.  Lane j: high orbit
+// j.  k = N - popcount(h) low pairs in block h of x, k - 1 in the words t.  With
+// A, B(j) the binomials of the pair on j at its own ordinal and one lower, EA, EB
+// their sums over the occupied high orbits below j, block h + q of x starts at
+//     EB(q) + C(L + q, k + #below) + base(h) - EA(q)     (modulo 2^32)
+// and its place among the words of its class is, with R(j) = C(j, ordinal from 1)
+// and S(j) = C(j, ordinal + 1),   ER(q) + C(q, #below + 1) + sum S - ES(q).
+__device__ __forceinline__ void prepare_block(BlockSmem &bs, const RemoveArgs &A, const uint32_t h,
+                                              const uint32_t *bin, const uint32_t *crk, const float *dh,
+                                              const float *__restrict__ x)
+{
+    const int lane = threadIdx.x & 31;
+    const int N = A.N, H = A.H;
+    const int ph = __popc(h), k = N - ph;
+    const bool occ = (h >> lane) & 1u;
+    const int io = __popc(h & ((1u << lane) - 1u));
+    uint32_t a = 0, bq = 0, c1 = 0, c2 = 0;
+    if (lane < H) {
+        bq = bin[lane * (N + 2) + k + io];
+        c1 = crk[lane * (H + 2) + io + 1];
+    }
+    if (occ) {
+        a = bin[lane * (N + 2) + k + io + 1];
+        c2 = crk[lane * (H + 2) + io + 2];
+    }
+    uint32_t ia = a, ib = occ ? bq : 0u, ir = occ ? c1 : 0u, is = c2;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t ta = __shfl_up_sync(0xffffffffu, ia, o);
+        const uint32_t tb = __shfl_up_sync(0xffffffffu, ib, o);
+        const uint32_t tr = __shfl_up_sync(0xffffffffu, ir, o);
+        const uint32_t ts = __shfl_up_sync(0xffffffffu, is, o);
+        if (lane >= o) { ia += ta; ib += tb; ir += tr; is += ts; }
+    }
+    const uint32_t base = __shfl_sync(0xffffffffu, ia, 31), stot = __shfl_sync(0xffffffffu, is, 31);
+    if (k <= A.L) {                               // block h exists (t is not the full low word)
+        const int nk = A.lo_off[k + 1] - A.lo_off[k];
+        for (int r = lane; r < nk; r += 32) copy_async4(bs.x + r, x + base + r);
+    }
+    if (occ || lane >= H) {
+        bs.xe[lane] = A.zeros;
+    } else {
+        // (lanes of empty orbits: the inclusive sums are the exclusive ones)
+        bs.xe[lane] = x + (uint32_t)(ib + bq + base - ia);
+        const uint64_t place = (uint32_t)(ir + c1 + stot - is);
+        const int nt = A.lo_off[k] - A.lo_off[k - 1];
+        bs.ze[lane] = A.scratch + A.zbase[k - 1] + (int64_t)(place * (uint64_t)(ph + 1) + (uint64_t)io) * nt;
+    }
+    float Dh = occ ? dh[lane] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) Dh += __shfl_xor_sync(0xffffffffu, Dh, o);
+    if (lane == 0) {
+        bs.h = h;
+        bs.base = base;
+        bs.dh = Dh;
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+// shared memory matrix descriptor of G: K-major, no swizzle, core matrices of 8
+// rows x 16 bytes, 128 bytes apart in K and KP * 32 bytes apart in N
+template <int KP>
+__device__ __forceinline__ uint64_t g_desc(uint32_t saddr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(128u >> 4) << 16;
+    d |= (uint64_t)((KP * 32u) >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    return d;
+}
+
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase)
+{
+    for (int it = 0; it < kWaitLimit; ++it) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}\n"
+                     : "=r"(done)
+                     : "r"(bar), "r"(phase), "r"(1000000u)
+                     : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+__device__ __forceinline__ float to_tf32(float v)
+{
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
+    return __uint_as_float(r);
+}
+
+// eight columns of this thread's row of tensor memory
+__device__ __forceinline__ void tmem_st8(uint32_t addr, const float (&v)[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"r"(addr),
+                 "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                 "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+                 "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&v)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// What bounds it: instruction issue and the latency of a tile's chain (gather,
+// split, tensor-memory store, product, load, scatter).  Two CTAs of three groups
+// share an SM's tensor memory, so that one group's gathers overlap another's
+// product; the high orbits of the next tile are loaded while the product runs;
+// the ninth (thirteenth) warp prepares the next block's pointers.  Omega=24:
+// 78 us alone with a cold cache for 3.9e8 hops (48e6 warp instructions, 0.55 of
+// the issue slots), where the row-by-row kernel (pd_hx.cu, variant 3) took
+// 215 us; both kernels together 0.096 ms.  Measured and not kept: FP32
+// multiply-adds instead of the tensor cores (packed pairs, coefficients from
+// shared memory or the constant bank, 8, 10 or 12 low orbits, hops between high
+// orbits in registers): 0.127 to 0.18 ms.
+template <int KP>
+__global__ void __launch_bounds__(Cfg<KP>::kThreads, 2)
+remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G, const float *__restrict__ d,
+              const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip)
+{
+    using C = Cfg<KP>;
+    if (skip && *skip) return;                    // CTA-uniform
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t s_bar[C::kGroups];
+    __shared__ uint32_t s_tmem;
+    const int omega = A.omega, L = A.L, H = A.H, N = A.N;
+    const LayoutR lay = layout_r(KP, H, N);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, group = warp >> 2;
+    uint32_t *bin = reinterpret_cast<uint32_t *>(smem + lay.bin), *crk = reinterpret_cast<uint32_t *>(smem + lay.crk);
+    float *dlow = reinterpret_cast<float *>(smem + lay.dlow), *dh = reinterpret_cast<float *>(smem + lay.dh);
+    BlockSmem *bufs = reinterpret_cast<BlockSmem *>(smem + lay.buf);
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int g = 0; g < C::kGroups; ++g)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&s_bar[g])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    // G in the operand layout, high and low parts (row n: the orbit that
+    // receives the pair, column k: the orbit it leaves)
+    for (int i = tid; i < C::kN * KP; i += C::kThreads) {
+        const int n = i / KP, k = i % KP;
+        auto orbit = [&](int c) { return c < kLT ? (c < L ? c : -1) : (c - kLT < H ? L + c - kLT : -1); };
+        const int on = orbit(n), ok = orbit(k);
+        const float g = (on >= 0 && ok >= 0 && on != ok) ? G[on * omega + ok] : 0.0f;
+        const float hi = to_tf32(g);
+        unsigned char *p = smem + lay.b + (n >> 3) * (KP * 32) + (k >> 2) * 128 + (n & 7) * 16 + (k & 3) * 4;
+        *reinterpret_cast<float *>(p) = hi;
+        *reinterpret_cast<float *>(p + 4 * C::kN * KP) = to_tf32(g - hi);
+    }
+    for (int i = tid; i < H * (N + 2); i += C::kThreads)
+        bin[i] = (uint32_t)__ldg(A.binom + (L + i / (N + 2)) * kBinomStride + i % (N + 2));
+    for (int i = tid; i < H * (H + 2); i += C::kThreads)
+        crk[i] = (uint32_t)__ldg(A.binom + (i / (H + 2)) * kBinomStride + i % (H + 2));
+    for (int i = tid; i < H; i += C::kThreads) dh[i] = d[L + i];
+    for (int i = tid; i < 128; i += C::kThreads) {   // diagonal sums of the two halves of a low word
+        const int w = i & 63, p0 = i < 64 ? 0 : 6;
+        float v = 0.0f;
+        for (int p = 0; p < 6; ++p)
+            if ((w >> p & 1) && p0 + p < L) v += d[p0 + p];
+        dlow[i] = v;
+    }
+    if (tid < 3) bufs[tid].x[kSpare] = 0.0f;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // G: generic stores -> tensor core reads
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = s_tmem + (uint32_t)(group < C::kGroups ? group : 0) * C::kCols;
+    const uint32_t trow = tmem + ((uint32_t)(warp & 3) << 21);       // this warp's 32 lanes
+    const uint32_t bar = smem_u32(&s_bar[group < C::kGroups ? group : 0]);
+    uint32_t phase = 0;
+    bool gave_up = false, odd = false;            // odd: a row of Z is NaN
+
+    auto take = [&](BlockSmem &bs) {              // the last warp
+        long long b = 0;
+        if (lane == 0) b = A.first + (long long)atomicAdd(&tk->hx_next, 1ull);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (b < A.end) prepare_block(bs, A, __ldg(A.words + b), bin, crk, dh, x);
+        if (lane == 0) bs.b = b;
+    };
+    // rows of a finished block: its slots summed per row, the diagonal, y
+    auto rows = [&](const BlockSmem &bs, const float *part) {
+        const int k = N - __popc(bs.h);
+        if (k > L) return;                        // no such block
+        const int lo_k = A.lo_off[k], nk = A.lo_off[k + 1] - lo_k;
+        for (int r = tid; r < nk; r += 32 * C::kWarps) {
+            const uint32_t l = __ldg(A.low + lo_k + r);
+            const float D = (dlow[l & 63u] + dlow[64 + (l >> 6)]) + bs.dh;
+            float s = 0.0f;
+#pragma unroll
+            for (int o = 0; o < kLT; ++o)
+                if (l >> o & 1u) s += part[o * kStride + r];
+            y[bs.base + r] = fmaf(D, bs.x[r], s);
+        }
+    };
+    // One barrier per block: after it the slots of block i are complete and
+    // buffer i + 1 is filled; the warps then sum the rows of block i and go on
+    // to the words of block i + 1 (slots alternate between two sets, buffers
+    // rotate over three: rows, words, preparation).
+    if (warp == C::kWarps) take(bufs[0]);
+    __syncthreads();
+    int cur = 0;                                  // buffer of block i
+    for (int i = 0;; ++i) {
+        const BlockSmem &bs = bufs[cur];
+        const int nxt = cur == 2 ? 0 : cur + 1;
+        const bool more = bs.b < A.end;
+        if (warp == C::kWarps) {
+            if (more) take(bufs[nxt]);
+        } else {
+            if (i > 0) rows(bufs[cur == 0 ? 2 : cur - 1], reinterpret_cast<const float *>(smem + (C::kSets == 2 ? ((i - 1) & 1) * kPartBytes : 0)));
+            if constexpr (C::kSets == 1) asm volatile("bar.sync 4, %0;\n" ::"n"(32 * C::kWarps) : "memory");
+            if (more) {
+                const uint32_t h = bs.h;
+                const int k = N - __popc(h);      // k >= 1
+                const int lo_t = A.lo_off[k - 1], nt = A.lo_off[k] - lo_t;
+                const uint32_t poff = C::kSets == 2 ? (uint32_t)(i & 1) * (kPartBytes * 0x10001u) : 0u;
+                constexpr int kPre = KP <= 24 ? KP - kLT : 8;   // high orbits loaded one tile ahead
+                uint32_t hop[kLT / 2];
+                float vh[kPre];
+                auto load = [&](int c) {
+                    const int rc = min(c * kTile + (tid & (kTile - 1)), nt - 1);
+#pragma unroll
+                    for (int p = 0; p < kLT / 2; ++p) hop[p] = __ldg(A.up + (p << L) + lo_t + rc);
+#pragma unroll
+                    for (int q = 0; q < kPre; ++q) vh[q] = __ldg(bs.xe[q] + rc);
+                };
+                if (group * kTile < nt) load(group);
+                for (int c = group; c * kTile < nt; c += C::kGroups) {
+                    const int r = c * kTile + (tid & (kTile - 1));
+                    const bool in = r < nt;
+                    // gather and split, eight columns at a time
+                    for_each<KP / 8>([&](auto gc) {
+                        constexpr int g = decltype(gc)::value;
+                        float v[8], hi[8];
+#pragma unroll
+                        for (int t = 0; t < 8; ++t) {
+                            const int p = 8 * g + t;
+                            if (p < kLT) {
+                                const uint32_t off = (p & 1) ? hop[p / 2] >> 16 : hop[p / 2] & 0xffffu;
+                                v[t] = *reinterpret_cast<const float *>(reinterpret_cast<const char *>(bs.x) + off);
+                            } else if (p - kLT < kPre) {
+                                v[t] = vh[p - kLT];
+                            } else {
+                                v[t] = __ldg(bs.xe[p - kLT] + (in ? r : nt - 1));
+                            }
+                        }
+#pragma unroll
+                        for (int t = 0; t < 8; ++t) {
+                            hi[t] = to_tf32(v[t]);
+                            v[t] -= hi[t];        // NaN where v is not finite, and with it the whole row of Z
+                        }
+                        tmem_st8(trow + 8 * g, hi);
+                        tmem_st8(trow + KP + 8 * g, v);
+                    });
+                    uint32_t slot[kLT / 2];
+#pragma unroll
+                    for (int p = 0; p < kLT / 2; ++p) slot[p] = hop[p] + poff;
+                    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                    asm volatile("bar.sync %0, 128;\n" ::"r"(group + 1) : "memory");
+                    if ((tid & (kTile - 1)) == 0) {
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        // TF32 operands, FP32 accumulator, both K-major, M = 128
+                        constexpr uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) |
+                                                   ((uint32_t)(C::kN >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+                        const uint64_t b0 = g_desc<KP>(smem_u32(smem + lay.b));
+#pragma unroll
+                        for (int s = 0; s < 3; ++s)
+#pragma unroll
+                            for (int kk = 0; kk < KP / 8; ++kk) {
+                                const uint32_t a = tmem + (s == 1 ? KP : 0) + 8 * kk;
+                                const uint64_t db = b0 + (uint64_t)(((s == 2 ? 4 * C::kN * KP : 0) + kk * 256) >> 4);
+                                const uint32_t accum = (s || kk) ? 1u : 0u;
+                                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                             "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(
+                                                 tmem + 2 * KP),
+                                             "r"(a), "l"(db), "r"(idesc), "r"(accum)
+                                             : "memory");
+                            }
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
+                            : "memory");
+                    }
+                    __syncwarp();
+                    if ((c + C::kGroups) * kTile < nt) load(c + C::kGroups);   // overlaps the product
+                    if (!mbar_wait(bar, phase)) gave_up = true;
+                    phase ^= 1u;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    for_each<KP / 8>([&](auto gc) {
+                        constexpr int g = decltype(gc)::value;
+                        uint32_t z[8];
+                        tmem_ld8(trow + 2 * KP + 8 * g, z);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                        if (g == 0) odd |= __uint_as_float(z[0]) != __uint_as_float(z[0]);
+#pragma unroll
+                        for (int t = 0; t < 8; ++t) {
+                            const int p = 8 * g + t;
+                            if (p < kLT) {
+                                const uint32_t off = (p & 1) ? slot[p / 2] >> 16 : slot[p / 2] & 0xffffu;
+                                *reinterpret_cast<float *>(smem + p * kStride * 4 + off) = __uint_as_float(z[t]);
+                            } else if (p - kLT < H && !(h >> (p - kLT) & 1u)) {
+                                if (in) bs.ze[p - kLT][r] = __uint_as_float(z[t]);
+                            }
+                        }
+                    });
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                }
+            }
+        }
+        if (!more) break;
+        __syncthreads();
+        cur = nxt;
+    }
+    if (odd) atomicOr(&tk->pad, 1ull);
+    if (gave_up) atomicExch(&tk->bar.err, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s_tmem), "r"(kTmemCols) : "memory");
+    if (arrive_last(&tk->hx_done) && tid == 0) tk->hx_next = 0ull;
+}
+
+// ---- pair addition --------------------------------------------------------------
+constexpr int kAThreads = 128;
+constexpr int kARows = 4;                // rows per thread and pass
+constexpr int kACtas = 10;               // CTAs per SM
+
+struct AddArgs {
+    int omega, N, L, H;
+    int lo_off[kLT + 2];
+    int nclass;
+    int ph[kLT + 1];
+    int64_t first[kLT + 2];              // number of the class's first word in words
+    int c0, c1;                          // classes of this launch
+    int64_t zbase[kLT + 1];
+    const uint32_t *words;
+    const uint16_t *low;
+    const uint64_t *binom;
+    const float *scratch;
+    int first_launch, last_launch;       // of the product
+};
+
+// one row term by term (elements that are not finite)
+__device__ __noinline__ float row_slow(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
+                                       const float *__restrict__ x, uint64_t s, float xs)
+{
+    float D = 0.0f;
+    for (int p = 0; p < A.omega; ++p)
+        if (s >> p & 1ull) D += d[p];
+    float acc = D * xs;
+    for (int o = 0; o < A.omega; ++o) {
+        if (!(s >> o & 1ull)) continue;
+        for (int e = 0; e < A.omega; ++e) {
+            if (s >> e & 1ull) continue;
+            uint64_t t = s ^ (1ull << o) ^ (1ull << e), idx = 0;
+            int c = 0;
+            for (uint64_t w = t; w; w &= w - 1)
+                idx += __ldg(A.binom + (__ffsll((long long)w) - 1) * kBinomStride + ++c);
+            acc = fmaf(G[e * A.omega + o], x[idx], acc);
+        }
+    }
+    return acc;
+}
+
+// y(h, l) += sum over the pairs a of h of scratch(h, a, l); fused x^T y.  Bound
+// by the latency of streaming reads: 16 loads per thread in flight, small CTAs
+// so that blocks of very different sizes balance.  Omega=24 (65 MB of scratch,
+// mostly in L2): 26 us alone with a cold cache, against 32 us with 256 threads
+// and 40 us with two rows per thread.
+__global__ void __launch_bounds__(kAThreads, kACtas)
+add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const float *__restrict__ d,
+           const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip, double *part,
+           double *dot_out)
+{
+    if (skip && *skip) return;                    // CTA-uniform
+    __shared__ double sred[kAThreads / 32];
+    __shared__ uint32_t bin[kMaxHigh * (kMaxHigh + kLT)];   // C(L + p, m), m < N + 2
+    const int lane = threadIdx.x & 31;
+    const int NB = A.N + 2;
+    for (int i = threadIdx.x; i < A.H * NB; i += kAThreads)
+        bin[i] = (uint32_t)__ldg(A.binom + (A.L + i / NB) * kBinomStride + i % NB);
+    const bool slow = *reinterpret_cast<volatile unsigned long long *>(&tk->pad) != 0ull;
+    __syncthreads();
+    DotAcc<float> dot;
+    int c = A.c0;
+    int64_t b = A.first[A.c0] + blockIdx.x;
+    const int64_t end = A.first[A.c1];
+    uint32_t hn = b < end ? __ldg(A.words + b) : 0u;
+    for (; b < end; b += gridDim.x) {
+        while (b >= A.first[c + 1]) ++c;
+        const int ph = A.ph[c], k = A.N - ph;
+        const int lo_k = A.lo_off[k], nk = A.lo_off[k + 1] - lo_k;
+        const uint32_t h = hn;
+        if (b + gridDim.x < end) hn = __ldg(A.words + b + gridDim.x);
+        const bool occ = h >> lane & 1u;
+        uint32_t base = occ ? bin[lane * NB + k + 1 + __popc(h & ((1u << lane) - 1u))] : 0u;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
+        const float *z = A.scratch + A.zbase[k] + (b - A.first[c]) * (int64_t)ph * nk;
+        float Dh = 0.0f;
+        if (k == 0) {                             // no pair removal writes these rows
+            Dh = occ ? d[A.L + lane] : 0.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) Dh += __shfl_xor_sync(0xffffffffu, Dh, o);
+        }
+        for (int r0 = threadIdx.x; r0 < nk; r0 += kARows * kAThreads) {
+            float acc[kARows], xr[kARows];
+            bool in[kARows];
+#pragma unroll
+            for (int i = 0; i < kARows; ++i) {
+                const int r = r0 + i * kAThreads;
+                in[i] = r < nk;
+                xr[i] = in[i] && (part || k == 0 || slow) ? __ldg(x + base + r) : 0.0f;
+                acc[i] = k == 0 ? Dh * xr[i] : in[i] ? y[base + r] : 0.0f;
+            }
+            const float *zr = z + r0;
+            int a = 0;
+            for (; a + 4 <= ph; a += 4) {
+                float v[4][kARows];
+#pragma unroll
+                for (int u = 0; u < 4; ++u, zr += nk)
+#pragma unroll
+                    for (int i = 0; i < kARows; ++i) v[u][i] = in[i] ? __ldcs(zr + i * kAThreads) : 0.0f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int i = 0; i < kARows; ++i) acc[i] += v[u][i];
+            }
+            for (; a < ph; ++a, zr += nk)
+#pragma unroll
+                for (int i = 0; i < kARows; ++i)
+                    if (in[i]) acc[i] += __ldcs(zr + i * kAThreads);
+#pragma unroll
+            for (int i = 0; i < kARows; ++i) {
+                const int r = r0 + i * kAThreads;
+                if (!in[i]) continue;
+                if (slow) acc[i] = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr[i]);
+                y[base + r] = acc[i];
+                if (part) dot.add(xr[i], acc[i]);
+            }
+        }
+    }
+    double v = 0.0;
+    if (part) {
+        v = block_reduce(dot, sred);
+        if (threadIdx.x == 0) part[blockIdx.x] = v;
+    }
+    if (!arrive_last(&tk->hx_done)) return;
+    if (A.last_launch && threadIdx.x == 0) tk->pad = 0ull;
+    if (!part) return;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kAThreads) s += __ldcg(part + i);
+    s = block_sum(s, sred);
+    if (threadIdx.x == 0) *dot_out = A.first_launch ? s : *dot_out + s;
+}
+
+template <int KP>
+const void *remove_fn() { return (const void *)remove_kernel<KP>; }
+int padded(int omega)
+{
+    const int c = omega > kLT ? omega : kLT;
+    return c <= 16 ? 16 : (c + 7) / 8 * 8;
+}
+const void *remove_fn_of(int KP)
+{
+    return KP == 16 ? remove_fn<16>() : KP == 24 ? remove_fn<24>() : KP == 32 ? remove_fn<32>() : remove_fn<40>();
+}
+int remove_threads(int KP)
+{
+    return KP == 16 ? Cfg<16>::kThreads : KP == 24 ? Cfg<24>::kThreads : KP == 32 ? Cfg<32>::kThreads : Cfg<40>::kThreads;
+}
+
+}  // namespace
+
+int fac_low(int omega) { return omega < kLT ? omega : kLT; }
+
+bool fac_fits(int omega, int n, int64_t dim)
+{
+    const int H = omega - fac_low(omega);
+    return n >= 1 && n < omega && dim < ((int64_t)1 << 32) && H <= kMaxHigh &&
+           layout_r(padded(omega), H, n).total <= kSmemMax;
+}
+
+// Where variant 2 is the faster one and no less exact (variant 3 / variant 2,
+// FP32, back to back): C(17,6) 15.7 / 18.5 us, C(18,9) = 48620 18.7 / 20.6 us,
+// C(20,10) = 184756 31 / 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 7.4 ms,
+// C(34,9) 12.8 / 6.8 ms.  Far above half filling there are more words t than
+// states and their rows are longer: C(24,16) 94 / 64 us, C(24,18) 48 / 41 us,
+// C(28,22) 141 / 211 us, and C(20,17) loses accuracy (2.2e-7 / 2.6e-7).
+bool fac_pays(int omega, int n, int64_t dim)
+{
+    return dim >= 60000 && 3 * n <= 2 * omega + 2 && fac_fits(omega, n, dim);
+}
+
+// classes of words with `pairs` pairs in all, the largest blocks first
+static void word_classes(int L, int H, int pairs, WordClasses &C)
+{
+    int ks[kLT + 1], n = 0;
+    for (int k = 0; k <= L; ++k)
+        if (pairs - k >= 0 && pairs - k <= H) ks[n++] = k;
+    for (int i = 1; i < n; ++i)
+        for (int j = i; j > 0 && host_binom(L, ks[j]) > host_binom(L, ks[j - 1]); --j) {
+            const int t = ks[j];
+            ks[j] = ks[j - 1];
+            ks[j - 1] = t;
+        }
+    C = WordClasses{};
+    C.n = n;
+    for (int i = 0; i < n; ++i) {
+        C.ph[i] = pairs - ks[i];
+        C.first[i + 1] = C.first[i] + (int64_t)host_binom(H, pairs - ks[i]);
+    }
+}
+
+size_t fac_zeros() { return kStride; }
+
+void fac_sizes(int omega, int n, FacPlan &p)
+{
+    p = FacPlan{};
+    p.omega = omega;
+    p.n = n;
+    p.L = fac_low(omega);
+    const int H = omega - p.L;
+    WordClasses ct, cy;
+    word_classes(p.L, H, n - 1, ct);
+    word_classes(p.L, H, n, cy);
+    p.nt = ct.first[ct.n];
+    p.ny = cy.first[cy.n];
+    p.table = (int64_t)(kLT / 2) << p.L;
+    int64_t all = 0, most = 0;
+    for (int i = 0; i < cy.n; ++i) {
+        const int64_t z = (int64_t)host_binom(H, cy.ph[i]) * cy.ph[i] * (int64_t)host_binom(p.L, n - cy.ph[i]);
+        all += z;
+        if (z > most) most = z;
+    }
+    p.by_class = all > kScratchAll;
+    p.scratch_len = p.by_class ? most : all;
+}
+
+cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st)
+{
+    p.on = false;
+    const int H = p.omega - p.L;
+    WordClasses ct, cy;
+    word_classes(p.L, H, p.n - 1, ct);
+    word_classes(p.L, H, p.n, cy);
+    cudaError_t ez = cudaMemsetAsync(p.zeros, 0, sizeof(float) * fac_zeros(), st);
+    if (ez != cudaSuccess) return ez;
+    hop_table_kernel<<<(unsigned)((p.table + 255) / 256), 256, 0, st>>>(p.L, binom, p.low, p.up);
+    high_words_kernel<<<(unsigned)((p.nt + 255) / 256), 256, 0, st>>>(ct, H, binom, p.twords);
+    high_words_kernel<<<(unsigned)((p.ny + 255) / 256), 256, 0, st>>>(cy, H, binom, p.ywords);
+    count_launches(3);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int KP = padded(p.omega);
+    p.smem = layout_r(KP, H, p.n).total;
+    e = cudaFuncSetAttribute(remove_fn_of(KP), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e != cudaSuccess) return e;
+    p.grid_t = 2 * sm_count();                    // two CTAs per SM share its tensor memory
+    p.grid_y = kACtas * sm_count();
+    p.on = true;
+    return cudaSuccess;
+}
+
+int64_t fac_partials(const FacPlan &p) { return p.grid_y; }
+
+
+cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, const float *x, float *y,
+                       Tickets *tk, cudaStream_t st, const int *skip, const HxDot *dot)
+{
+    const int L = p.L, H = p.omega - L, N = p.n, KP = padded(p.omega);
+    WordClasses ct, cy;
+    word_classes(L, H, N - 1, ct);
+    word_classes(L, H, N, cy);
+    RemoveArgs R{};
+    AddArgs A{};
+    R.omega = A.omega = p.omega;
+    R.N = A.N = N;
+    R.L = A.L = L;
+    R.H = A.H = H;
+    for (int k = 0; k <= kLT; ++k) {
+        R.lo_off[k + 1] = R.lo_off[k] + (int)host_binom(L, k);
+        A.lo_off[k + 1] = R.lo_off[k + 1];
+    }
+    R.words = p.twords;
+    R.up = p.up;
+    R.low = A.low = p.low;
+    R.binom = A.binom = binom;
+    R.scratch = p.scratch;
+    R.zeros = p.zeros;
+    A.scratch = p.scratch;
+    A.words = p.ywords;
+    A.nclass = cy.n;
+    for (int i = 0; i < cy.n; ++i) A.ph[i] = cy.ph[i];
+    for (int i = 0; i <= cy.n; ++i) A.first[i] = cy.first[i];
+    int64_t z = 0;
+    for (int i = 0; i < cy.n && !p.by_class; ++i) {
+        const int k = N - cy.ph[i];
+        R.zbase[k] = A.zbase[k] = z;
+        z += (int64_t)host_binom(H, cy.ph[i]) * cy.ph[i] * (int64_t)host_binom(L, k);
+    }
+    auto remove = [&](int64_t first, int64_t end) -> cudaError_t {
+        R.first = first;
+        R.end = end;
+        const int64_t grid = p.grid_t < end - first ? p.grid_t : end - first;
+        const void *args[] = {&R, &G, &d, &x, &y, &tk, &skip};
+        return cudaLaunchKernel(remove_fn_of(KP), dim3((unsigned)grid), dim3((unsigned)remove_threads(KP)),
+                                const_cast<void **>(args), p.smem, st);
+    };
+    auto add = [&](int c0, int c1) -> cudaError_t {
+        A.c0 = c0;
+        A.c1 = c1;
+        const int64_t nb = cy.first[c1] - cy.first[c0];
+        const int64_t grid = p.grid_y < nb ? p.grid_y : nb;
+        add_kernel<<<(unsigned)grid, kAThreads, 0, st>>>(A, G, d, x, y, tk, skip, dot ? dot->blk_part : nullptr,
+                                                         dot ? dot->out : nullptr);
+        return cudaGetLastError();
+    };
+    if (!p.by_class) {
+        const cudaError_t e = remove(0, p.nt);
+        if (e != cudaSuccess) return e;
+        A.first_launch = A.last_launch = 1;
+        count_launches(2);
+        return add(0, cy.n);
+    }
+    // class by class, the low pairs k ascending: the words t with k low pairs give
+    // the scratch of the rows with k and the partial y of the rows with k + 1
+    int left = cy.n;
+    A.first_launch = 1;
+    for (int k = 0; k <= L; ++k) {
+        for (int i = 0; i < ct.n; ++i)
+            if (N - 1 - ct.ph[i] == k) {
+                const cudaError_t e = remove(ct.first[i], ct.first[i + 1]);
+                if (e != cudaSuccess) return e;
+                count_launches(1);
+            }
+        for (int i = 0; i < cy.n; ++i)
+            if (N - cy.ph[i] == k) {
+                A.last_launch = --left == 0;
+                const cudaError_t e = add(i, i + 1);
+                if (e != cudaSuccess) return e;
+                A.first_launch = 0;
+                count_launches(1);
+            }
+    }
+    return cudaSuccess;
+}
+
+}  // namespace pd

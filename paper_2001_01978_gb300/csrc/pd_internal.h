@@ -78,15 +78,13 @@ struct Blocks {
     int64_t nblocks;
     int max_block;                   // max_k C(L, k) over admissible k
     int max_hh;                      // max over blocks of the number of high->high hops
-    int max_stage;                   // max over blocks of the elements of all neighbour blocks
-                                     // (ph C(L, k+1) + (H - ph) C(L, k-1))
     const uint64_t *blk_h;           // [nblocks] high words, ascending
     const uint64_t *blk_base;        // [nblocks] index of the block's first state
     const uint16_t *lowword;         // [2^L] L-bit words grouped by popcount, ascending
     const uint16_t *rankL;           // [2^L] rank of a word within its popcount group
     const uint64_t *binom;           // [64*64]
     int lo_off[kMaxLow + 2];         // group offsets into lowword
-    int variant;                     // H*x kernel: 0 automatic, 1 staged per neighbour, 2 all staged
+    int variant;                     // H*x kernel (pairdiag_options.hx_variant); 2 concerns FP32 alone
     // truncated model space (Sec. 3.5): kept_map[full index] = position among the
     // kept states, -1 for a dropped state; nullptr = the full space.  Vectors of
     // a truncated handle hold the kept states only, in basis order.
@@ -94,6 +92,25 @@ struct Blocks {
     // the blocks holding at least one kept state (the truncated H*x walks only these)
     const uint64_t *kept_blk_h, *kept_blk_base;
     int64_t kept_nblocks;
+};
+
+// The FP32 product by pair removal on the tensor cores (variant 2, pd_hxf.cu).
+// It has tables of its own: high words of the states with one pair less (twords)
+// and of the states (ywords), by class of pairs in the low orbits.
+struct FacPlan {
+    bool on = false;
+    int omega = 0, n = 0, L = 0;
+    int64_t nt = 0, ny = 0;              // words
+    int64_t table = 0;                   // entries of up
+    bool by_class = false;               // the rows of one class (low pairs) at a time
+    int64_t scratch_len = 0;             // floats of scratch
+    int grid_t = 0, grid_y = 0;
+    size_t smem = 0;
+    uint32_t *twords = nullptr, *ywords = nullptr;   // device
+    uint16_t *low = nullptr;             // [2^L] low words
+    uint32_t *up = nullptr;              // hops of the low words
+    float *scratch = nullptr;
+    float *zeros = nullptr;              // [fac_zeros()]
 };
 
 // ---- many problems at once (batched solver) ---------------------------------
@@ -132,7 +149,7 @@ struct Tickets {
     unsigned long long hx_next;      // next block of a persistent H*x launch
     unsigned long long hx_done;      // CTAs of that launch that have finished
     unsigned long long vec_done;     // CTAs of a streaming kernel whose partial sums are written
-    unsigned long long pad;
+    unsigned long long pad;          // variant 2: an element could not be split (not finite)
     GridBar bar;                     // the fused Lanczos step's barriers
 };
 
@@ -305,7 +322,7 @@ cudaError_t hx_batch_launch(const BatchBlocks &BB, const HxProblem &P, int preci
                             unsigned long long *counter, int grid, cudaStream_t st, const int *skip, int skip_stride);
 int hx_batch_grid(const BatchBlocks &BB, int precision);
 size_t hx_smem_bytes(const Blocks &B, int precision);
-int hx_variant(const Blocks &B, int precision);   // kernel variant a launch will use (1 or 2)
+int hx_variant(const Blocks &B, int precision);   // kernel variant hx_launch will use
 // y = H x (Eq. 2 in the pair basis) over the persistent grid.
 // skip (nullable, device): when *skip != 0 the launched kernels return at once.
 // dot (nullable): also x^T y, the Lanczos alpha, with one partial sum per basis
@@ -319,6 +336,19 @@ cudaError_t hx_launch(const Blocks &B, const HxProblem &P, int precision, const 
                       Tickets *tk, int grid, cudaStream_t st, const int *skip = nullptr,
                       const HxDot *dot = nullptr);
 int hx_grid(const Blocks &B, int precision);
+// variant 2 (pd_hxf.cu).  fac_fits: whether it serves a problem; fac_sizes: the
+// lengths of the device arrays, which the caller allocates; fac_build fills them.
+// fac_partials: doubles that a fused dot needs in blk_part.  fac_launch: as
+// hx_launch for FP32.
+int fac_low(int omega);
+bool fac_fits(int omega, int n, int64_t dim);
+bool fac_pays(int omega, int n, int64_t dim);
+void fac_sizes(int omega, int n, FacPlan &p);
+size_t fac_zeros();
+cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st);
+int64_t fac_partials(const FacPlan &p);
+cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, const float *x, float *y,
+                       Tickets *tk, cudaStream_t st, const int *skip, const HxDot *dot);
 // Truncation (Sec. 3.5).  The bin of a state is floor((D - lo) / (hi - lo) * bins)
 // in FP64, clamped to bins - 1, with D its diagonal element summed in ascending
 // orbit order; lo/hi the extreme diagonal elements.
