@@ -856,14 +856,24 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
     }
     bool use_fac = o.hx_variant == 2;             // variant 2 where it serves the problem
     if (o.hx_variant == 0) {
-        // untuned: direct gathers; far from half filling (fewer than 3 in 10 orbits
-        // occupied, or empty) deep gather groups and 13 low orbits, the fastest
-        // schedules measured at Omega = 24..38
+        // untuned: direct gathers.  The block split follows the dimension: a CTA
+        // owns a block, so few large blocks leave SMs idle or end the launch on
+        // one of them (FP64, 12 low orbits / the split taken here: C(12,6) 22.6 /
+        // 12.1 us, C(16,8) 47 / 18.5 us, C(18,8) 48 / 27 us, C(20,10) 89 / 67 us,
+        // C(22,9) 203 / 151 us).  Far from half filling (fewer than 3 in 10 orbits
+        // occupied, or empty) most blocks hold a few rows: more low orbits, and in
+        // large spaces deep gather groups (C(28,22) FP32: variant 3, 12 low orbits
+        // 188 us, variant 4, 13 low orbits 141 us; C(24,18) 48 / 85 us; C(20,17)
+        // 10 / 12 / 13 low orbits 14.4 / 15.4 / 17.3 us).
         const int minority = std::min(n_pairs, omega - n_pairs);
         const bool low_filling = 10 * minority < 3 * omega;
-        use_fac = o.precision == PD_PREC_MIXED && fac_pays(omega, n_pairs, (int64_t)host_binom(omega, n_pairs));
-        o.hx_variant = low_filling ? 4 : 3;
-        if (o.low_bits == 0 && low_filling) o.low_bits = 13;
+        const int64_t dim = (int64_t)host_binom(omega, n_pairs);
+        use_fac = o.precision == PD_PREC_MIXED && fac_pays(omega, n_pairs, dim);
+        o.hx_variant = low_filling && dim >= 300000 ? 4 : 3;
+        if (o.low_bits == 0) {
+            if (low_filling) o.low_bits = dim < 30000 ? 10 : dim < 300000 ? 12 : 13;
+            else o.low_bits = dim < 300000 ? 10 : dim < 2000000 ? 11 : 12;
+        }
     }
     pairdiag *h = new pairdiag();
     h->omega = omega; h->n = n_pairs; h->opt = o;
