@@ -317,6 +317,11 @@ scale_kernel(const T *src, T *dst, int64_t n, const double *__restrict__ div, in
 // all of them hold bit-identical coefficients.
 constexpr int kStepThreads = 512;
 constexpr int kStepWarps = kStepThreads / 32;
+// The fewest packs of a CTA of the step kernel.  An FP64 step is bound by the
+// FP64 pipes (two multiply-adds per clock and SM) and small steps of either type
+// by the latency of their loads, so even short vectors are spread over many SMs:
+// with 2048 packs per CTA a 43758-element FP64 step ran on 11 SMs.
+constexpr int64_t kStepMinPacks = 128;
 constexpr unsigned kBarPolls = 1u << 24;      // x >= 64 ns: a barrier gives up after about a second
 
 // Dot-product accumulator of the step kernel, one pack at a time.  FP32: the
@@ -432,15 +437,15 @@ __device__ __forceinline__ void load_group(Pack<T, W> (&q)[KG], const T *__restr
         if (KG == 1 || j0 + u < m) q[u] = load_pack<T, W, true>(Q + (int64_t)(j0 + u) * ldq, c, n);
 }
 
-// Ownership: the packs form chunks of kStepThreads; CTA b owns the K
-// consecutive chunks b*K .. b*K + K - 1, thread t pack t of each.  Local pack
+// Ownership: CTA b owns `slice` consecutive packs from b * slice on, in chunks
+// of kStepThreads, thread t pack t of each (the last chunk may be short).  Local pack
 // slot (chunk l of the CTA, thread t) = l * kStepThreads + t.
 // KG: vectors per group pass (1, 2, 4 or 8, chosen per launch so that the
 // last group issues few predicated-off multiply-adds)
 template <typename T, int W, bool SMEM, int KG>
 __global__ void __launch_bounds__(kStepThreads, 1)
 step_kernel(const T *__restrict__ Q, int64_t ldq, int i, LanczosScalars *S, T *p, int64_t n,
-            typename StepRed<T>::P *part, GridBar *gb, T *qnext)
+            const int64_t slice, typename StepRed<T>::P *part, GridBar *gb, T *qnext)
 {
     using R = StepRed<T>;
     using P = typename R::P;
@@ -469,13 +474,13 @@ step_kernel(const T *__restrict__ Q, int64_t ldq, int i, LanczosScalars *S, T *p
     const T *qi = Q + (int64_t)i * ldq;
     const T *qm = Q + (int64_t)(i > 0 ? i - 1 : 0) * ldq;
     const int64_t nc = (n + W - 1) / W;
-    const int64_t nchunk = (nc + kStepThreads - 1) / kStepThreads;
     const int64_t G = gridDim.x;
-    const int64_t K = (nchunk + G - 1) / G;
-    const int64_t first = (int64_t)blockIdx.x * K;
-    const int64_t mine = first < nchunk ? (nchunk - first < K ? nchunk - first : K) : 0;   // chunks of this CTA
+    const int64_t first = (int64_t)blockIdx.x * slice;
+    const int64_t packs = first < nc ? (nc - first < slice ? nc - first : slice) : 0;   // packs of this CTA
+    const int64_t mine = (packs + kStepThreads - 1) / kStepThreads;                     // in chunks
     const int ng = (m + KG - 1) / KG;
-    auto pack_of = [&](int64_t l) { return (first + l) * kStepThreads + tid; };
+    auto pack_of = [&](int64_t l) { return first + l * kStepThreads + tid; };
+    auto has = [&](int64_t l) { return l * kStepThreads + tid < packs; };
 
     // phase 1: p <- p - alpha q_i - beta_{i-1} q_{i-1}; c_j = Q_j^T p (j <= i).
     // Two chunks per iteration, all their loads issued before the first use.
@@ -484,7 +489,7 @@ step_kernel(const T *__restrict__ Q, int64_t ldq, int i, LanczosScalars *S, T *p
         PackAcc<T> acc[KG];
         for (int64_t l = 0; l < mine; l += 2) {
             const int64_t c0 = pack_of(l), c1 = pack_of(l + 1);
-            const bool ok0 = c0 < nc, ok1 = l + 1 < mine && c1 < nc;
+            const bool ok0 = has(l), ok1 = has(l + 1);
             Pack<T, W> v[2], q[2][KG];
             if (g == 0) {
                 Pack<T, W> x[2], y[2];
@@ -567,7 +572,7 @@ step_kernel(const T *__restrict__ Q, int64_t ldq, int i, LanczosScalars *S, T *p
         for (int u = 0; u < KG; ++u) cg[u] = (j0 + u < m) ? scT[j0 + u] : T(0);
         for (int64_t l = 0; l < mine; l += 2) {
             const int64_t c0 = pack_of(l), c1 = pack_of(l + 1);
-            const bool ok0 = c0 < nc, ok1 = l + 1 < mine && c1 < nc;
+            const bool ok0 = has(l), ok1 = has(l + 1);
             Pack<T, W> v[2], q[2][KG];
             if (ok0) {
                 v[0] = SMEM ? sv[l * kStepThreads + tid] : load_pack<T, W, false>(p, c0, n);
@@ -634,7 +639,7 @@ step_kernel(const T *__restrict__ Q, int64_t ldq, int i, LanczosScalars *S, T *p
     const T f = s_ab[2];
     for (int64_t l = 0; l < mine; ++l) {
         const int64_t cc = pack_of(l);
-        if (cc >= nc) continue;
+        if (!has(l)) continue;
         Pack<T, W> v = SMEM ? sv[l * kStepThreads + tid] : load_pack<T, W, false>(p, cc, n);
 #pragma unroll
         for (int k = 0; k < W; ++k) v.v[k] = v.v[k] * f;
@@ -1695,10 +1700,10 @@ int step_plan_t(int64_t n, int64_t ldq, const void *Q, const void *p, StepPlan *
     }
     const bool pk = packable<T>({Q, p}, ldq);
     const int64_t units = pack_units<T>(n, pk);
-    const int64_t nchunk = (units + kStepThreads - 1) / kStepThreads;
-    // at least four chunks of kStepThreads packs per CTA, at most one CTA per SM
-    int64_t grid = std::min<int64_t>(std::max<int64_t>((nchunk + 3) / 4, 1), (int64_t)sm_count());
-    int64_t slice = (nchunk + grid - 1) / grid * kStepThreads;      // packs per CTA, whole chunks
+    // at most one CTA per SM, each with at least kStepMinPacks packs
+    int64_t grid = std::min<int64_t>(std::max<int64_t>((units + kStepMinPacks - 1) / kStepMinPacks, 1), (int64_t)sm_count());
+    auto slice_of = [&](int64_t g) { return ((units + g - 1) / g + 31) / 32 * 32; };   // packs per CTA, whole warps
+    int64_t slice = slice_of(grid);
     const size_t smem = (size_t)slice * step_pack_bytes<T>(pk);
     bool in_smem = smem <= kStepSmemMax;
     int per_sm = in_smem ? step_per_sm<T>(pk, true, smem) : 0;
@@ -1707,7 +1712,7 @@ int step_plan_t(int64_t n, int64_t ldq, const void *Q, const void *p, StepPlan *
         per_sm = step_per_sm<T>(pk, false, 0);
         if (per_sm < 1) return 0;
         grid = std::min<int64_t>(grid, (int64_t)per_sm * sm_count());
-        slice = (nchunk + grid - 1) / grid * kStepThreads;
+        slice = slice_of(grid);
     }
     plan->grid = (int)grid;
     plan->slice = slice;
@@ -1723,8 +1728,8 @@ cudaError_t step_t(const StepPlan &plan, const T *Q, int64_t ldq, int i, Lanczos
 {
     using P = typename StepRed<T>::P;
     P *pp = reinterpret_cast<P *>(part);
-    void *args[] = {(void *)&Q, (void *)&ldq, (void *)&i, (void *)&S, (void *)&p, (void *)&n, (void *)&pp,
-                    (void *)&gb, (void *)&qnext};
+    void *args[] = {(void *)&Q, (void *)&ldq, (void *)&i, (void *)&S, (void *)&p, (void *)&n, (void *)&plan.slice,
+                    (void *)&pp, (void *)&gb, (void *)&qnext};
     const void *fn = step_fn<T>(plan.packed, plan.in_smem, step_group<T>(i + 1));
     const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(plan.grid), dim3(kStepThreads), args, plan.smem, st);
     count_launches(1);
