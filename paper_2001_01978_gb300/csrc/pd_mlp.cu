@@ -92,30 +92,80 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase)
 }
 
 // stage rows [r0, r0 + 128) x k [k0, k0 + 64) of op(X) (row index r, column k)
-// into the canonical layout; zero outside [0, nrow) x [k0, kend)
+// into the canonical layout; zero outside [0, nrow) x [k0, kend).  Operands start
+// on 16-byte boundaries and ld is a multiple of 8, so whole packs of eight are
+// read with 16-byte loads: along k where k is contiguous (eight rows x four packs
+// per warp, so that both the reads and the 16-byte stores are whole lines), and
+// along r where it is not, an 8 x 8 tile per thread transposed in registers.
 template <bool TR>
 __device__ __forceinline__ void stage_slice(unsigned char *dst, const bf16 *__restrict__ X, int ld, int r0, int nrow,
                                             int k0, int kend)
 {
     const bf16 zero = __float2bfloat16(0.0f);
-    for (int it = threadIdx.x; it < kTileM * (kSliceK / 8); it += blockDim.x) {
-        const int r = it % kTileM, kc = it / kTileM;        // consecutive threads: consecutive rows
-        const int gr = r0 + r;
-        __align__(16) bf16 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int gk = k0 + kc * 8 + j;
-            v[j] = (gr < nrow && gk < kend) ? (TR ? X[(size_t)gk * ld + gr] : X[(size_t)gr * ld + gk]) : zero;
+    if constexpr (!TR) {
+#pragma unroll 4
+        for (int it = threadIdx.x; it < kTileM * (kSliceK / 8); it += 128) {
+            const int r = (it >> 6) * 8 + (it & 7), kc = (it >> 3) & 7;
+            const int gr = r0 + r, gk = k0 + kc * 8;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (gr < nrow && gk + 8 <= kend) {
+                v = __ldg(reinterpret_cast<const uint4 *>(X + (size_t)gr * ld + gk));
+            } else if (gr < nrow && gk < kend) {
+                __align__(16) bf16 e[8];
+                for (int j = 0; j < 8; ++j) e[j] = gk + j < kend ? X[(size_t)gr * ld + gk + j] : zero;
+                v = *reinterpret_cast<const uint4 *>(e);
+            }
+            *reinterpret_cast<uint4 *>(dst + (r >> 3) * 1024 + kc * 128 + (r & 7) * 16) = v;
         }
-        *reinterpret_cast<uint4 *>(dst + (r >> 3) * 1024 + kc * 128 + (r & 7) * 16) =
-            *reinterpret_cast<const uint4 *>(v);
+    } else {
+        const int rt = threadIdx.x & 15, kt = threadIdx.x >> 4;   // 16 x 8 tiles of 8 x 8
+        const int gr = r0 + rt * 8, gk = k0 + kt * 8;
+        uint4 in[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {                         // row gk + j of X: eight consecutive r
+            in[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (gk + j < kend && gr + 8 <= nrow) {
+                in[j] = __ldg(reinterpret_cast<const uint4 *>(X + (size_t)(gk + j) * ld + gr));
+            } else if (gk + j < kend && gr < nrow) {
+                __align__(16) bf16 e[8];
+                for (int i = 0; i < 8; ++i) e[i] = gr + i < nrow ? X[(size_t)(gk + j) * ld + gr + i] : zero;
+                in[j] = *reinterpret_cast<const uint4 *>(e);
+            }
+        }
+        auto word = [&](int j, int q) { return q == 0 ? in[j].x : q == 1 ? in[j].y : q == 2 ? in[j].z : in[j].w; };
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const unsigned sel = (r & 1) ? 0x7632u : 0x5410u;
+            const uint4 v = make_uint4(__byte_perm(word(0, r / 2), word(1, r / 2), sel),
+                                       __byte_perm(word(2, r / 2), word(3, r / 2), sel),
+                                       __byte_perm(word(4, r / 2), word(5, r / 2), sel),
+                                       __byte_perm(word(6, r / 2), word(7, r / 2), sel));
+            *reinterpret_cast<uint4 *>(dst + rt * 1024 + kt * 128 + r * 16) = v;
+        }
     }
 }
 
-template <bool TA, bool TB>
+__device__ __forceinline__ float silu(float z) { return z / (1.0f + __expf(-z)); }
+__device__ __forceinline__ float dsilu(float z)
+{
+    const float s = 1.0f / (1.0f + __expf(-z));
+    return s * (1.0f + z * (1.0f - s));
+}
+
+// What becomes of the accumulator: EP_STORE writes C (or adds it, split K);
+// EP_SILU (forward) Z = C + bias, act = silu(Z); EP_DSILU (backward) C is dA,
+// act = dA silu'(Z), its column sums are added to bias_grad.
+enum { EP_STORE = 0, EP_SILU = 1, EP_DSILU = 2 };
+struct Epilogue {
+    const float *bias = nullptr, *Z = nullptr;
+    bf16 *act = nullptr;
+    float *bias_grad = nullptr;
+};
+
+template <bool TA, bool TB, int EP>
 __global__ void __launch_bounds__(128)
 gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__restrict__ B, int ldb,
-               float *__restrict__ C, int ldc, int *err)
+               float *__restrict__ C, int ldc, const Epilogue ep, int *err)
 {
     __shared__ __align__(1024) unsigned char sA[kTileM * kSliceK * 2];
     __shared__ __align__(1024) unsigned char sB[kTileN * kSliceK * 2];
@@ -190,14 +240,65 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
                          : "r"(taddr)
                          : "memory");
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-            if (row < M) {
-                float *dst = C + (size_t)row * ldc + c0;
+            const bool in = row < M;
+            float *dst = C + (size_t)(in ? row : 0) * ldc + c0;
+            float f[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) f[j] = __uint_as_float(v[j]);
+            if constexpr (EP == EP_STORE) {
+                if (in && split) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) atomicAdd(dst + j, f[j]);
+                } else if (in) {
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        *reinterpret_cast<float4 *>(dst + j) = make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]);
+                }
+                continue;
+            }
+            float g[32];                              // what act receives
+            if constexpr (EP == EP_SILU) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    const float f = __uint_as_float(v[j]);
-                    if (split) atomicAdd(dst + j, f);
-                    else dst[j] = f;
+                    f[j] += __ldg(ep.bias + c0 + j);
+                    g[j] = silu(f[j]);
                 }
+            } else {
+                const float *z = ep.Z + (size_t)(in ? row : 0) * ldc + c0;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    const float4 z4 = __ldg(reinterpret_cast<const float4 *>(z + j));
+                    g[j] = in ? f[j] * dsilu(z4.x) : 0.0f;
+                    g[j + 1] = in ? f[j + 1] * dsilu(z4.y) : 0.0f;
+                    g[j + 2] = in ? f[j + 2] * dsilu(z4.z) : 0.0f;
+                    g[j + 3] = in ? f[j + 3] * dsilu(z4.w) : 0.0f;
+                }
+            }
+            if (in) {
+                bf16 *act = ep.act + (size_t)row * ldc + c0;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4)
+                    *reinterpret_cast<float4 *>(dst + j) = make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]);
+#pragma unroll
+                for (int j = 0; j < 32; j += 8) {
+                    __align__(16) __nv_bfloat162 h[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(g[j + 2 * q], g[j + 2 * q + 1]);
+                    *reinterpret_cast<uint4 *>(act + j) = *reinterpret_cast<const uint4 *>(h);
+                }
+            }
+            if constexpr (EP == EP_DSILU) {
+                // 32 columns x 32 rows of the warp: lane l ends with column l's sum
+                // (each step halves the columns a lane still carries)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int j = 0; j < o; ++j) {
+                        const bool up = (lane & o) != 0;
+                        const float keep = up ? g[j + o] : g[j], give = up ? g[j] : g[j + o];
+                        g[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                atomicAdd(ep.bias_grad + c0 + lane, g[0]);
             }
         }
     }
@@ -207,43 +308,23 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-// C[M, 128] = op(A) op(B) (split K over ksplit CTAs per row tile, C zeroed first)
-template <bool TA, bool TB>
-void gemm(int M, int N, int K, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int ksplit,
-          int *err, cudaStream_t st)
+// C[M, 128] = op(A) op(B); with ksplit > 1 it is added to C, which the caller has
+// zeroed (split K over ksplit CTAs per row tile)
+template <bool TA, bool TB, int EP = EP_STORE>
+void gemm(int M, int K, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int ksplit, int *err,
+          cudaStream_t st, const Epilogue &ep = Epilogue{})
 {
-    (void)N;                                   // always kTileN (the layer width)
     dim3 grid((M + kTileM - 1) / kTileM, ksplit);
-    if (ksplit > 1) cudaMemsetAsync(C, 0, sizeof(float) * (size_t)M * ldc, st);
     // 18 KB of unused dynamic shared memory keep at most four CTAs on an SM,
     // so their 4 x 128 TMEM columns fit the SM's 512 and no allocation waits
     static const cudaError_t attr =       // static + dynamic shared memory above 48 KB needs the opt-in
-        cudaFuncSetAttribute(gemm_tc_kernel<TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmPadSmem);
+        cudaFuncSetAttribute(gemm_tc_kernel<TA, TB, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmPadSmem);
     (void)attr;
-    gemm_tc_kernel<TA, TB><<<grid, 128, kGemmPadSmem, st>>>(M, K, A, lda, B, ldb, C, ldc, err);
+    gemm_tc_kernel<TA, TB, EP><<<grid, 128, kGemmPadSmem, st>>>(M, K, A, lda, B, ldb, C, ldc, ep, err);
     count_launches(1);
 }
 
 // ---- elementwise pieces ------------------------------------------------------
-__device__ __forceinline__ float silu(float z) { return z / (1.0f + __expf(-z)); }
-__device__ __forceinline__ float dsilu(float z)
-{
-    const float s = 1.0f / (1.0f + __expf(-z));
-    return s * (1.0f + z * (1.0f - s));
-}
-
-// Z += bias (in place, FP32), A = silu(Z) in bfloat16
-__global__ void bias_silu_kernel(float *__restrict__ Z, const float *__restrict__ bias, bf16 *__restrict__ Aout,
-                                 int rows)
-{
-    const int64_t n = (int64_t)rows * kH;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float z = Z[i] + bias[i % kH];
-        Z[i] = z;
-        Aout[i] = __float2bfloat16(silu(z));
-    }
-}
-
 // out[r] = A3[r,:] . w4 + b4 (one warp per row)
 __global__ void head_kernel(const bf16 *__restrict__ A3, const bf16 *__restrict__ w4, const float *__restrict__ b4,
                             float *__restrict__ out, int rows)
@@ -256,61 +337,38 @@ __global__ void head_kernel(const bf16 *__restrict__ A3, const bf16 *__restrict_
     if (lane == 0) out[r] = s + b4[0];
 }
 
-// dout = 2 (out - t) / rows; loss partial sums
-__global__ void loss_kernel(const float *__restrict__ out, const float *__restrict__ t, float *__restrict__ dout,
-                            int rows, double *__restrict__ loss)
-{
-    __shared__ double sh[256];
-    double acc = 0.0;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
-        const float d = out[r] - t[r];
-        dout[r] = 2.0f * d / (float)rows;
-        acc += (double)d * d;
-    }
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(loss, sh[0] / rows);
-}
-
-// head backward: g_w4[j] = sum_r A3[r,j] dout[r], g_b4 = sum dout; dZ3 = dout w4 silu'(Z3)
+// dout = 2 (out - t) / rows and the loss; head backward: g_w4[j] = sum_r A3[r,j]
+// dout[r], g_b4 = sum dout; dZ3 = dout w4 silu'(Z3) and its column sums
 __global__ void head_back_kernel(const bf16 *__restrict__ A3, const float *__restrict__ Z3, const bf16 *__restrict__ w4,
-                                 const float *__restrict__ dout, int rows, float *__restrict__ gw4,
+                                 const float *__restrict__ out, const float *__restrict__ t, int rows,
+                                 float *__restrict__ dout, double *__restrict__ loss, float *__restrict__ gw4,
                                  float *__restrict__ gb4, bf16 *__restrict__ dZ, float *__restrict__ gb3)
 {
     const int j = threadIdx.x;                 // column (blockDim.x == kH)
     float sw = 0.0f, sb = 0.0f, sz = 0.0f;
+    double sl = 0.0;
     const float wj = __bfloat162float(w4[j]);
+#pragma unroll 4
     for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const float d = dout[r];
+        const float e = out[r] - t[r];
+        const float d = 2.0f * e / (float)rows;
         const size_t i = (size_t)r * kH + j;
         sw += __bfloat162float(A3[i]) * d;
-        if (j == 0) sb += d;
+        if (j == 0) {
+            dout[r] = d;
+            sb += d;
+            sl += (double)e * e;
+        }
         const float dz = d * wj * dsilu(Z3[i]);
         dZ[i] = __float2bfloat16(dz);
         sz += dz;
     }
     atomicAdd(&gw4[j], sw);
     atomicAdd(&gb3[j], sz);
-    if (j == 0) atomicAdd(gb4, sb);
-}
-
-// dZ = dA silu'(Z) (dA FP32 from a product), bias gradient column sums
-__global__ void dsilu_kernel(const float *__restrict__ dA, const float *__restrict__ Z, int rows,
-                             bf16 *__restrict__ dZ, float *__restrict__ gb)
-{
-    const int j = threadIdx.x;
-    float sz = 0.0f;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const size_t i = (size_t)r * kH + j;
-        const float dz = dA[i] * dsilu(Z[i]);
-        dZ[i] = __float2bfloat16(dz);
-        sz += dz;
+    if (j == 0) {
+        atomicAdd(gb4, sb);
+        atomicAdd(loss, sl / rows);
     }
-    atomicAdd(&gb[j], sz);
 }
 
 __global__ void to_bf16_kernel(const float *__restrict__ src, bf16 *__restrict__ dst, int n)
@@ -344,6 +402,7 @@ struct pairdiag_mlp {
     bf16 *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;   // backward intermediates, one per layer
     float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *dA1 = nullptr, *dA2 = nullptr;
     float *out = nullptr, *t = nullptr, *dout = nullptr;
+    float *Xf = nullptr;         // the inputs as given (FP32)
     int *err = nullptr;          // set by a tensor-core product whose bounded wait expired
     double *loss = nullptr;
     int steps = 0;
@@ -355,11 +414,11 @@ namespace {
 void mlp_free_work(pairdiag_mlp *m)
 {
     void *p[] = {m->X, m->A1, m->A2, m->A3, m->dZ1, m->dZ2, m->dZ3, m->Z1, m->Z2, m->Z3, m->dA1, m->dA2,
-                 m->out, m->t, m->dout};
+                 m->out, m->t, m->dout, m->Xf};
     for (void *q : p)
         if (q) cudaFree(q);
     m->X = m->A1 = m->A2 = m->A3 = m->dZ1 = m->dZ2 = m->dZ3 = nullptr;
-    m->Z1 = m->Z2 = m->Z3 = m->dA1 = m->dA2 = m->out = m->t = m->dout = nullptr;
+    m->Z1 = m->Z2 = m->Z3 = m->dA1 = m->dA2 = m->out = m->t = m->dout = m->Xf = nullptr;
     m->cap = 0;
 }
 
@@ -369,6 +428,7 @@ int mlp_reserve(pairdiag_mlp *m, int rows)
     mlp_free_work(m);
     const size_t nh = (size_t)rows * kH;
     PD_CUDA(cudaMalloc(&m->X, sizeof(bf16) * (size_t)rows * kF));
+    PD_CUDA(cudaMalloc(&m->Xf, sizeof(float) * (size_t)rows * kF));
     PD_CUDA(cudaMalloc(&m->A1, sizeof(bf16) * nh));
     PD_CUDA(cudaMalloc(&m->A2, sizeof(bf16) * nh));
     PD_CUDA(cudaMalloc(&m->A3, sizeof(bf16) * nh));
@@ -407,14 +467,14 @@ int mlp_forward(pairdiag_mlp *m, int rows)
 {
     cudaStream_t st = m->st;
     to_bf16_kernel<<<grid1(kNParams), 256, 0, st>>>(m->theta, m->wb, kNParams);
-    gemm<false, false>(rows, kH, kF, m->X, kF, m->wb + oW1, kH, m->Z1, kH, 1, m->err, st);
-    bias_silu_kernel<<<grid1((int64_t)rows * kH), 256, 0, st>>>(m->Z1, m->theta + ob1, m->A1, rows);
-    gemm<false, false>(rows, kH, kH, m->A1, kH, m->wb + oW2, kH, m->Z2, kH, 1, m->err, st);
-    bias_silu_kernel<<<grid1((int64_t)rows * kH), 256, 0, st>>>(m->Z2, m->theta + ob2, m->A2, rows);
-    gemm<false, false>(rows, kH, kH, m->A2, kH, m->wb + oW3, kH, m->Z3, kH, 1, m->err, st);
-    bias_silu_kernel<<<grid1((int64_t)rows * kH), 256, 0, st>>>(m->Z3, m->theta + ob3, m->A3, rows);
+    gemm<false, false, EP_SILU>(rows, kF, m->X, kF, m->wb + oW1, kH, m->Z1, kH, 1, m->err, st,
+                                Epilogue{m->theta + ob1, nullptr, m->A1, nullptr});
+    gemm<false, false, EP_SILU>(rows, kH, m->A1, kH, m->wb + oW2, kH, m->Z2, kH, 1, m->err, st,
+                                Epilogue{m->theta + ob2, nullptr, m->A2, nullptr});
+    gemm<false, false, EP_SILU>(rows, kH, m->A2, kH, m->wb + oW3, kH, m->Z3, kH, 1, m->err, st,
+                                Epilogue{m->theta + ob3, nullptr, m->A3, nullptr});
     head_kernel<<<(rows * 32 + 255) / 256, 256, 0, st>>>(m->A3, m->wb + ow4, m->theta + ob4, m->out, rows);
-    count_launches(5);
+    count_launches(2);
     PD_CUDA(cudaGetLastError());
     return PD_OK;
 }
@@ -423,36 +483,38 @@ int mlp_forward(pairdiag_mlp *m, int rows)
 int mlp_backward(pairdiag_mlp *m, int rows)
 {
     cudaStream_t st = m->st;
-    const int ks = std::max(1, std::min(64, rows / 256));
+    // weight gradients: 128 rows per CTA (two slices), at most 64 CTAs
+    const int ks = std::max(1, std::min(64, (rows + 127) / 128));
     PD_CUDA(cudaMemsetAsync(m->grad, 0, sizeof(float) * kNParams, st));
     PD_CUDA(cudaMemsetAsync(m->loss, 0, sizeof(double), st));
-    loss_kernel<<<std::max(1, std::min(64, (rows + 255) / 256)), 256, 0, st>>>(m->out, m->t, m->dout, rows, m->loss);
-    const int gr = std::max(1, std::min(1024, rows));
-    head_back_kernel<<<gr, kH, 0, st>>>(m->A3, m->Z3, m->wb + ow4, m->dout, rows, m->grad + ow4, m->grad + ob4,
-                                        m->dZ3, m->grad + ob3);
-    // layer 3: gW3 = A2^T dZ3 (written straight into the gradient), dA2 = dZ3 W3^T
-    gemm<true, false>(kH, kH, rows, m->A2, kH, m->dZ3, kH, m->grad + oW3, kH, ks, m->err, st);
-    gemm<false, true>(rows, kH, kH, m->dZ3, kH, m->wb + oW3, kH, m->dA2, kH, 1, m->err, st);
-    dsilu_kernel<<<gr, kH, 0, st>>>(m->dA2, m->Z2, rows, m->dZ2, m->grad + ob2);
+    head_back_kernel<<<std::max(1, std::min(2 * sm_count(), rows)), kH, 0, st>>>(
+        m->A3, m->Z3, m->wb + ow4, m->out, m->t, rows, m->dout, m->loss, m->grad + ow4, m->grad + ob4, m->dZ3,
+        m->grad + ob3);
+    // layer 3: gW3 = A2^T dZ3 (added straight into the gradient), dA2 = dZ3 W3^T, dZ2 = dA2 silu'(Z2)
+    gemm<true, false>(kH, rows, m->A2, kH, m->dZ3, kH, m->grad + oW3, kH, ks, m->err, st);
+    gemm<false, true, EP_DSILU>(rows, kH, m->dZ3, kH, m->wb + oW3, kH, m->dA2, kH, 1, m->err, st,
+                                Epilogue{nullptr, m->Z2, m->dZ2, m->grad + ob2});
     // layer 2
-    gemm<true, false>(kH, kH, rows, m->A1, kH, m->dZ2, kH, m->grad + oW2, kH, ks, m->err, st);
-    gemm<false, true>(rows, kH, kH, m->dZ2, kH, m->wb + oW2, kH, m->dA1, kH, 1, m->err, st);
-    dsilu_kernel<<<gr, kH, 0, st>>>(m->dA1, m->Z1, rows, m->dZ1, m->grad + ob1);
+    gemm<true, false>(kH, rows, m->A1, kH, m->dZ2, kH, m->grad + oW2, kH, ks, m->err, st);
+    gemm<false, true, EP_DSILU>(rows, kH, m->dZ2, kH, m->wb + oW2, kH, m->dA1, kH, 1, m->err, st,
+                                Epilogue{nullptr, m->Z1, m->dZ1, m->grad + ob1});
     // layer 1: gW1 = X^T dZ1
-    gemm<true, false>(kF, kH, rows, m->X, kF, m->dZ1, kH, m->grad + oW1, kH, ks, m->err, st);
-    count_launches(4);
+    gemm<true, false>(kF, rows, m->X, kF, m->dZ1, kH, m->grad + oW1, kH, ks, m->err, st);
+    count_launches(1);
     PD_CUDA(cudaGetLastError());
     return PD_OK;
 }
 
+// X is rounded to bfloat16 on the device; every caller synchronises m->st
+// before it returns, so X and t outlive the copies
 int mlp_load_inputs(pairdiag_mlp *m, int rows, const float *X, const float *t)
 {
     PD_TRY(mlp_reserve(m, rows));
-    std::vector<bf16> xb((size_t)rows * kF);
-    for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16(X[i]);
-    PD_CUDA(cudaMemcpyAsync(m->X, xb.data(), sizeof(bf16) * xb.size(), cudaMemcpyHostToDevice, m->st));
+    PD_CUDA(cudaMemcpyAsync(m->Xf, X, sizeof(float) * (size_t)rows * kF, cudaMemcpyHostToDevice, m->st));
+    to_bf16_kernel<<<grid1((int64_t)rows * kF), 256, 0, m->st>>>(m->Xf, m->X, rows * kF);
+    count_launches(1);
+    PD_CUDA(cudaGetLastError());
     if (t) PD_CUDA(cudaMemcpyAsync(m->t, t, sizeof(float) * rows, cudaMemcpyHostToDevice, m->st));
-    PD_CUDA(cudaStreamSynchronize(m->st));          // host staging buffers go out of scope
     return PD_OK;
 }
 
