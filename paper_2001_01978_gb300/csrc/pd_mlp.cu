@@ -37,27 +37,26 @@ using bf16 = __nv_bfloat16;
 // accumulator in tensor memory (TMEM).
 // A(m,k) = TA ? A[k*lda + m] : A[m*lda + k];  B(k,n) = TB ? B[n*ldb + k] : B[k*ldb + n].
 // Every product of the network has N = 128 (the layer width).  One CTA of 128
-// threads computes a 128 x 128 tile of C over a range of K (split K over
+// threads computes a 128 x NT tile of C over a range of K (split K over
 // gridDim.y, added with atomics into a zeroed C):
-//   - the four warps stage a 128 x 64 slice of A and of B^T in shared memory in
+//   - the four warps stage 64-wide slices of A and of B^T in shared memory in
 //     the canonical K-major layout without swizzle: 8 x 16-byte core matrices,
 //     element (r, k) at (r / 8) * 1024 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2
 //     bytes, so the leading (K) byte offset of the descriptor is 128 and the
 //     stride (8-row) byte offset 1024;
-//   - one thread issues four tcgen05.mma (M = N = 128, K = 16 each) into the
-//     TMEM accumulator (128 lanes = rows of C, 128 columns) and commits them
+//   - one thread issues four tcgen05.mma (M = 128, N = NT, K = 16 each) into the
+//     TMEM accumulator (128 lanes = rows of C, NT columns) and commits them
 //     to an mbarrier, which every thread waits on before the slice is
 //     overwritten;
 //   - the epilogue reads the accumulator with tcgen05.ld (each warp its 32
-//     lanes) and writes C.
+//     lanes), applies the bias and activation or silu', and writes.
 // Waits are bounded: on expiry the kernel sets *err, still frees its TMEM and
 // returns (the caller reports PD_ETIMEOUT).  The network's products are tiny
 // (M = the orbit rows of the problems, K <= rows), so staging by threads
 // instead of TMA is no bottleneck.
 constexpr int kTileM = 128, kTileN = 128, kSliceK = 64;
-constexpr int kTmemCols = 128;                 // one FP32 column per output column
 constexpr long long kSpinLimit = 1ll << 26;    // mbarrier polls before giving up
-constexpr int kGemmPadSmem = 18 * 1024;
+constexpr int kGemmPadSmem = 10 * 1024;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -71,11 +70,6 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr)
     d |= (uint64_t)1 << 46;                               // descriptor version of this architecture
     return d;                                             // base offset 0, no swizzle
 }
-
-// instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
-// K-major, N = 128, M = 128
-constexpr uint32_t kIdescBf16 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTileN >> 3) << 17) |
-                                ((uint32_t)(kTileM >> 4) << 24);
 
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase)
 {
@@ -91,20 +85,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase)
     return false;
 }
 
-// stage rows [r0, r0 + 128) x k [k0, k0 + 64) of op(X) (row index r, column k)
+// stage rows [r0, r0 + ROWS) x k [k0, k0 + 64) of op(X) (row index r, column k)
 // into the canonical layout; zero outside [0, nrow) x [k0, kend).  Operands start
 // on 16-byte boundaries and ld is a multiple of 8, so whole packs of eight are
 // read with 16-byte loads: along k where k is contiguous (eight rows x four packs
 // per warp, so that both the reads and the 16-byte stores are whole lines), and
 // along r where it is not, an 8 x 8 tile per thread transposed in registers.
-template <bool TR>
+template <bool TR, int ROWS>
 __device__ __forceinline__ void stage_slice(unsigned char *dst, const bf16 *__restrict__ X, int ld, int r0, int nrow,
                                             int k0, int kend)
 {
     const bf16 zero = __float2bfloat16(0.0f);
     if constexpr (!TR) {
-#pragma unroll 4
-        for (int it = threadIdx.x; it < kTileM * (kSliceK / 8); it += 128) {
+#pragma unroll
+        for (int it = threadIdx.x; it < ROWS * (kSliceK / 8); it += 128) {
             const int r = (it >> 6) * 8 + (it & 7), kc = (it >> 3) & 7;
             const int gr = r0 + r, gk = k0 + kc * 8;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -118,7 +112,9 @@ __device__ __forceinline__ void stage_slice(unsigned char *dst, const bf16 *__re
             *reinterpret_cast<uint4 *>(dst + (r >> 3) * 1024 + kc * 128 + (r & 7) * 16) = v;
         }
     } else {
-        const int rt = threadIdx.x & 15, kt = threadIdx.x >> 4;   // 16 x 8 tiles of 8 x 8
+        constexpr int kRt = ROWS / 8;                            // kRt x 8 tiles of 8 x 8
+        const int rt = threadIdx.x % kRt, kt = threadIdx.x / kRt;
+        if (kt >= kSliceK / 8) return;
         const int gr = r0 + rt * 8, gk = k0 + kt * 8;
         uint4 in[8];
 #pragma unroll
@@ -162,17 +158,20 @@ struct Epilogue {
     float *bias_grad = nullptr;
 };
 
-template <bool TA, bool TB, int EP>
+template <bool TA, bool TB, int EP, int NT>
 __global__ void __launch_bounds__(128)
 gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__restrict__ B, int ldb,
                float *__restrict__ C, int ldc, const Epilogue ep, int *err)
 {
     __shared__ __align__(1024) unsigned char sA[kTileM * kSliceK * 2];
-    __shared__ __align__(1024) unsigned char sB[kTileN * kSliceK * 2];
+    __shared__ __align__(1024) unsigned char sB[NT * kSliceK * 2];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * kTileM;
+    const int m0 = blockIdx.x * kTileM, n0 = blockIdx.z * NT;
+    constexpr uint32_t kCols = NT;                     // tensor-memory columns
+    constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) |
+                                ((uint32_t)(kTileM >> 4) << 24);   // FP32 accumulator, BF16, both K-major
     const int kchunk = ((K + gridDim.y - 1) / gridDim.y + kSliceK - 1) / kSliceK * kSliceK;
     const int kbeg = blockIdx.y * kchunk, kend = min(K, kbeg + kchunk);
     if (kbeg >= kend) return;                          // CTA-uniform: nothing to add
@@ -180,7 +179,7 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
-                     "r"(kTmemCols)
+                     "r"(kCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -197,8 +196,8 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
     uint32_t phase = 0;
     bool timed_out = false;
     for (int k0 = kbeg; k0 < kend && !timed_out; k0 += kSliceK) {
-        stage_slice<TA>(sA, A, lda, m0, M, k0, kend);
-        stage_slice<!TB>(sB, B, ldb, 0, kTileN, k0, kend);   // row n of B^T: B(k, n)
+        stage_slice<TA, kTileM>(sA, A, lda, m0, M, k0, kend);
+        stage_slice<!TB, NT>(sB, B, ldb, n0, kTileN, k0, kend);   // row n of B^T: B(k, n)
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // generic-proxy stores -> async proxy
         __syncthreads();
         if (tid == 0) {
@@ -209,7 +208,7 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
                 const uint32_t accum = (k0 == kbeg && sk == 0) ? 0u : 1u;
                 asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-                             "l"(da), "l"(db), "r"(kIdescBf16), "r"(accum)
+                             "l"(da), "l"(db), "r"(kIdesc), "r"(accum)
                              : "memory");
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(barp)
@@ -226,9 +225,10 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
     } else {
         // epilogue: warp w owns TMEM lanes (rows) 32w .. 32w + 31
         const int row = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < kTileN; c0 += 32) {
+        for (int cc = 0; cc < NT; cc += 32) {
+            const int c0 = n0 + cc;
             uint32_t v[32];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cc;
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
                          "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
                          "%28, %29, %30, %31}, [%32];\n"
@@ -305,7 +305,7 @@ gemm_tc_kernel(int M, int K, const bf16 *__restrict__ A, int lda, const bf16 *__
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
 }
 
 // C[M, 128] = op(A) op(B); with ksplit > 1 it is added to C, which the caller has
@@ -314,13 +314,14 @@ template <bool TA, bool TB, int EP = EP_STORE>
 void gemm(int M, int K, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int ksplit, int *err,
           cudaStream_t st, const Epilogue &ep = Epilogue{})
 {
-    dim3 grid((M + kTileM - 1) / kTileM, ksplit);
-    // 18 KB of unused dynamic shared memory keep at most four CTAs on an SM,
-    // so their 4 x 128 TMEM columns fit the SM's 512 and no allocation waits
-    static const cudaError_t attr =       // static + dynamic shared memory above 48 KB needs the opt-in
-        cudaFuncSetAttribute(gemm_tc_kernel<TA, TB, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmPadSmem);
-    (void)attr;
-    gemm_tc_kernel<TA, TB, EP><<<grid, 128, kGemmPadSmem, st>>>(M, K, A, lda, B, ldb, C, ldc, ep, err);
+    // 32 columns per CTA: a 3333-row product has 27 row tiles, so whole rows would
+    // leave most SMs idle and each CTA with a long epilogue (loss and gradient of
+    // 3333 rows 250 us with 128 columns per CTA)
+    constexpr int NT = 32;
+    dim3 grid((M + kTileM - 1) / kTileM, ksplit, kTileN / NT);
+    // unused dynamic shared memory keeps at most seven CTAs on an SM, so their
+    // 7 x 32 TMEM columns leave room for other kernels and no allocation waits
+    gemm_tc_kernel<TA, TB, EP, NT><<<grid, 128, kGemmPadSmem, st>>>(M, K, A, lda, B, ldb, C, ldc, ep, err);
     count_launches(1);
 }
 
