@@ -144,6 +144,11 @@ struct pairdiag {
     int64_t full_dim = 0, full_nnz = 0;   // C(Omega, N) and its off-diagonal nonzeros
     int32_t *d_kmap = nullptr;       // truncated space (Sec. 3.5): full index -> kept index, -1 dropped
     uint64_t *d_kblk_h = nullptr, *d_kblk_base = nullptr;   // the blocks holding kept states
+    int64_t *d_kblk_first = nullptr;
+    int *d_kblk_rows = nullptr;
+    uint64_t *d_kfull = nullptr;     // full index and low word of every kept state
+    uint16_t *d_klow = nullptr;
+    void *d_xf[2] = {nullptr, nullptr};   // x in the full space, zeros at the dropped states (per storage type)
     // the block list in the order the persistent H*x kernels take it when
     // there are few blocks per CTA: largest blocks first (ascending high word
     // within a size), so the launch does not end on one CTA's large block
@@ -214,7 +219,8 @@ void free_all(pairdiag *h)
     void *ptrs[] = {h->d_blk_h, h->d_blk_base, h->d_binom, h->d_lowword, h->d_rankL, h->d_G64,
                     h->d_d64, h->d_G32, h->d_d32, h->d_tk, h->d_blkdot, h->d_part, h->d_S, h->d_small,
                     h->d_Q[0], h->d_Q[1], h->d_p[0], h->d_p[1], h->d_v64, h->d_w64,
-                    h->d_L64, h->d_L32, h->d_lockc, h->d_kmap, h->d_kblk_h, h->d_kblk_base,
+                    h->d_L64, h->d_L32, h->d_lockc, h->d_kmap, h->d_kblk_h, h->d_kblk_base, h->d_kblk_first,
+                    h->d_kblk_rows, h->d_kfull, h->d_klow, h->d_xf[0], h->d_xf[1],
                     h->d_lpt_h, h->d_lpt_base, h->d_Gff, h->d_dff};
     // the blocks go back to the library's cache: no queued kernel may still use
     // them.  Every kernel and copy of the handle runs on its stream, so that
@@ -415,9 +421,14 @@ int hx(pairdiag *h, int precision, const void *x, void *y, const int *skip = nul
     if (precision == 1 && h->fac.on && !B.kept_map)
         PD_CUDA(fac_launch(h->fac, h->d_binom, h->d_G32, h->d_d32, static_cast<const float *>(x),
                            static_cast<float *>(y), h->d_tk, h->st, skip, dot_out ? &dot : nullptr));
-    else
+    else {
+        if (hx_kept_direct(B, precision)) {
+            PD_CUDA(kept_scatter_launch(precision, h->d_kfull, h->dim, x, h->d_xf[precision], h->st, skip));
+            x = h->d_xf[precision];
+        }
         PD_CUDA(hx_launch(B, P, precision, x, y, h->d_tk, h->hxgrid[precision], h->st, skip,
                           dot_out ? &dot : nullptr));
+    }
     if (ev) PD_CUDA(cudaEventRecord(ev->second, h->st));
     return PD_OK;
 }
@@ -1191,7 +1202,8 @@ void drop_space(pairdiag *h)
     cudaStreamSynchronize(h->st);
     void **vecs[] = {&h->d_Q[0], &h->d_Q[1], &h->d_p[0], &h->d_p[1], (void **)&h->d_v64, (void **)&h->d_w64,
                      (void **)&h->d_L64, (void **)&h->d_L32, (void **)&h->d_kmap, (void **)&h->d_kblk_h,
-                     (void **)&h->d_kblk_base};
+                     (void **)&h->d_kblk_base, (void **)&h->d_kblk_first, (void **)&h->d_kblk_rows,
+                     (void **)&h->d_kfull, (void **)&h->d_klow, &h->d_xf[0], &h->d_xf[1]};
     for (void **v : vecs) {
         pool_free(*v);
         *v = nullptr;
@@ -1203,6 +1215,9 @@ void drop_space(pairdiag *h)
     h->B.kept_map = nullptr;
     h->B.kept_blk_h = h->B.kept_blk_base = nullptr;
     h->B.kept_nblocks = 0;
+    h->B.kept_blk_first = nullptr;
+    h->B.kept_blk_rows = nullptr;
+    h->B.kept_low = nullptr;
     h->dim = h->full_dim;
     h->nnz = h->full_nnz;
     h->ldq = (h->dim + 3) / 4 * 4;
@@ -1295,14 +1310,41 @@ int build_truncation(pairdiag *h, int64_t limit, int64_t bins, int64_t *kept)
         PD_CUDA(cudaMemcpyAsync(bh.data(), B.blk_h, sizeof(uint64_t) * bh.size(), cudaMemcpyDeviceToHost, st));
         PD_CUDA(cudaMemcpyAsync(bb.data(), B.blk_base, sizeof(uint64_t) * bb.size(), cudaMemcpyDeviceToHost, st));
         PD_CUDA(cudaStreamSynchronize(st));
-        std::vector<uint64_t> kh, kb;
+        // (the most kept states first, so that a launch does not end on a large block)
+        std::vector<uint32_t> order;
         for (size_t b = 0; b < cnt.size(); ++b)
-            if (cnt[b] > 0) {
-                kh.push_back(bh[b]);
-                kb.push_back(bb[b]);
-            }
+            if (cnt[b] > 0) order.push_back((uint32_t)b);
+        if ((int64_t)order.size() <= kLptMaxBlocks)
+            std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) { return cnt[a] > cnt[b]; });
+        std::vector<uint64_t> kh, kb;
+        std::vector<int64_t> kf;
+        std::vector<int> kr;
+        for (uint32_t b : order) {
+            kh.push_back(bh[b]);
+            kb.push_back(bb[b]);
+            kf.push_back(first[b]);
+            kr.push_back(cnt[b]);
+        }
         PD_TRY(upload(&h->d_kblk_h, kh));
         PD_TRY(upload(&h->d_kblk_base, kb));
+        PD_TRY(upload(&h->d_kblk_first, kf));
+        PD_TRY(upload(&h->d_kblk_rows, kr));
+        // lists of the kept states, and x in the full space: without room for
+        // them the product looks every state up in the map
+        const bool room = dalloc(&h->d_kfull, (size_t)total) == PD_OK && dalloc(&h->d_klow, (size_t)total) == PD_OK &&
+                          dalloc((double **)&h->d_xf[0], (size_t)full) == PD_OK &&
+                          dalloc((float **)&h->d_xf[1], (size_t)full) == PD_OK;
+        if (room) {
+            PD_CUDA(kept_list_launch(B, h->d_kmap, h->d_kfull, h->d_klow, grid, st));
+            PD_CUDA(cudaMemsetAsync(h->d_xf[0], 0, sizeof(double) * (size_t)full, st));
+            PD_CUDA(cudaMemsetAsync(h->d_xf[1], 0, sizeof(float) * (size_t)full, st));
+        } else {
+            void **part[] = {(void **)&h->d_kfull, (void **)&h->d_klow, &h->d_xf[0], &h->d_xf[1]};
+            for (void **q : part) {
+                pool_free(*q);
+                *q = nullptr;
+            }
+        }
         h->B.kept_nblocks = (int64_t)kh.size();
         return PD_OK;
     }();
@@ -1330,6 +1372,9 @@ int pairdiag_truncate(pairdiag_t *h, int64_t dimension_limit, int64_t bins, int6
         h->B.kept_map = h->d_kmap;
         h->B.kept_blk_h = h->d_kblk_h;
         h->B.kept_blk_base = h->d_kblk_base;
+        h->B.kept_blk_first = h->d_kblk_first;
+        h->B.kept_blk_rows = h->d_kblk_rows;
+        h->B.kept_low = h->d_xf[0] && h->d_xf[1] ? h->d_klow : nullptr;
         h->hxgrid[0] = hx_grid(h->B, 0);
         h->hxgrid[1] = hx_grid(h->B, 1);
         h->hxgrid[2] = hx_grid(h->B, 2);
@@ -1346,7 +1391,12 @@ int pairdiag_truncate(pairdiag_t *h, int64_t dimension_limit, int64_t bins, int6
             if (r == PD_OK && cudaStreamSynchronize(h->st) != cudaSuccess) r = fail(PD_ECUDA, "product start");
             if (r == PD_OK) {
                 const HxProblem P1{g1, d0, nullptr, nullptr};
-                cudaError_t ce = hx_launch(h->B, P1, 0, h->d_v64, h->d_w64, h->d_tk, h->hxgrid[0], h->st);
+                const bool direct = hx_kept_direct(h->B, 0);
+                cudaError_t ce = direct ? kept_scatter_launch(0, h->d_kfull, kept, h->d_v64, h->d_xf[0], h->st, nullptr)
+                                        : cudaSuccess;
+                if (ce == cudaSuccess)
+                    ce = hx_launch(h->B, P1, 0, direct ? (const void *)h->d_xf[0] : (const void *)h->d_v64, h->d_w64,
+                                   h->d_tk, h->hxgrid[0], h->st);
                 if (ce == cudaSuccess)
                     ce = multidot_launch(0, h->d_w64, kept, 1, h->d_v64, kept, h->d_part, &h->d_S->dots[0], h->st,
                                          nullptr, &h->d_tk->vec_done);

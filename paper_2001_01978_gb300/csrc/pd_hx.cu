@@ -128,8 +128,9 @@ __device__ __forceinline__ FF operator+(FF a, FF b)
 // x^T y over this warp's rows of one basis block (y as stored) into sw[warp]
 // (lane 0).  No barrier: thread 0 adds the warp sums in warp order after the
 // barrier that opens the next block (block_sum_deferred).
+// (ro: the rows' places in sx; null = the rows themselves)
 template <typename T, typename A, int R>
-__device__ __forceinline__ void warp_dot(const A *acc, const T *sx, int nk, double *sw)
+__device__ __forceinline__ void warp_dot(const A *acc, const T *sx, int nk, double *sw, const int *ro = nullptr)
 {
     // float-float rows: the dot in FP64 of the rows as written (FP64)
     using D = typename std::conditional<std::is_same<A, FF>::value, double, T>::type;
@@ -137,7 +138,7 @@ __device__ __forceinline__ void warp_dot(const A *acc, const T *sx, int nk, doub
 #pragma unroll
     for (int i = 0; i < R; ++i) {
         const int r = threadIdx.x + i * kThreads;
-        if (r < nk) d.add((D)sx[r], D(acc[i]));
+        if (r < nk) d.add((D)sx[ro ? ro[i] : r], D(acc[i]));
     }
     const double s = warp_reduce(d);
     if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = s;
@@ -517,7 +518,7 @@ struct Smem3 {
 // the eight partial sums in warp order (a fixed order).  acc[0] of warp 0
 // holds the row's diagonal and low->low terms on entry and the row's y on
 // exit; y (of type TY) is written here.
-template <typename T, typename A, int R, typename TY>
+template <typename T, typename A, int R, bool KEPT, typename TY>
 __device__ __forceinline__ void hx3_small(const Smem3<T, A> &s, const int L, const int k, const int ph,
                                           const int nemp, const int nhh, const uint64_t base,
                                           const uint16_t *__restrict__ lw, TY *__restrict__ y, const int nk,
@@ -529,8 +530,9 @@ __device__ __forceinline__ void hx3_small(const Smem3<T, A> &s, const int L, con
     A a = (w == 0) ? acc[0] : A(0);
     if (r < nk) {
         const uint32_t l = __ldg(lw + r);
+        const int ro = KEPT ? (int)s.rank[l] : r;
 #pragma unroll 2
-        for (int j = w; j < nhh; j += kW) a += s.hg[j] * A(__ldg(s.hp[j] + r));
+        for (int j = w; j < nhh; j += kW) a += s.hg[j] * A(__ldg(s.hp[j] + ro));
         if (k < L)
             for (int ai = w; ai < ph; ai += kW) {
                 const T *xb = s.xo[ai];
@@ -569,7 +571,10 @@ __device__ __forceinline__ void hx3_small(const Smem3<T, A> &s, const int L, con
 
 // The rows of one block in variant 3 (RR rows per thread): diagonal, low->low
 // from the staged block, then the gathers; writes y and the fused dot.
-template <typename T, typename A, int RR, bool DEEP, typename TY>
+// KEPT (a truncated space): the rows are the block's kept states, lw holds their
+// low words, base is the first kept index, and row r lies at offset rank(lw[r])
+// of the block; x is the full-space vector with zeros at the dropped states.
+template <typename T, typename A, int RR, bool DEEP, bool KEPT, typename TY>
 __device__ __forceinline__ void hx3_rows(const Smem3<T, A> &s, const int omega, const int L, const uint64_t h,
                                          const uint64_t base, const uint16_t *__restrict__ lw,
                                          TY *__restrict__ y, double *swdot, const int k, const int ph,
@@ -580,18 +585,21 @@ __device__ __forceinline__ void hx3_rows(const Smem3<T, A> &s, const int omega, 
     A Dh = A(0);
     for (uint64_t w = h; w; w &= w - 1) Dh += s.d[L + __ffsll((long long)w) - 1];
     uint32_t lr[RR];
+    int ro[RR];                                   // the row's offset in the block
     A acc[RR];
 #pragma unroll
     for (int i = 0; i < RR; ++i) {
         const int r = tid + i * kThreads;
         lr[i] = 0;
+        ro[i] = r;
         acc[i] = A(0);
         if (r < nk) {
             const uint32_t l = __ldg(lw + r);
             lr[i] = l;
+            if (KEPT) ro[i] = s.rank[l];
             A D = A(0);
             for (uint32_t w = l; w; w &= w - 1) D += s.d[__ffs(w) - 1];
-            acc[i] = (D + Dh) * A(s.x[r]);
+            acc[i] = (D + Dh) * A(s.x[ro[i]]);
             // low -> low (own block, shared memory)
             A a = acc[i];
             uint32_t oc = l;
@@ -611,8 +619,8 @@ __device__ __forceinline__ void hx3_rows(const Smem3<T, A> &s, const int omega, 
         }
     }
     if (nk <= 32) {                               // block-uniform
-        hx3_small<T, A, RR>(s, L, k, ph, nemp, nhh, base, lw, y, nk, acc);
-        if (swdot) warp_dot<T, A, RR>(acc, s.x, nk, swdot);
+        hx3_small<T, A, RR, KEPT>(s, L, k, ph, nemp, nhh, base, lw, y, nk, acc);
+        if (swdot) warp_dot<T, A, RR>(acc, s.x, nk, swdot, ro);
         return;
     }
     // warps without a row of this block skip the gathers (warp-uniform)
@@ -634,7 +642,7 @@ __device__ __forceinline__ void hx3_rows(const Smem3<T, A> &s, const int omega, 
                 const A g = s.hg[j];
 #pragma unroll
                 for (int i = 0; i < RR; ++i)
-                    if (rv[i]) acc[i] += g * A(__ldg(xb + tid + i * kThreads));
+                    if (rv[i]) acc[i] += g * A(__ldg(xb + ro[i]));
             }
         }
         for (int j0 = 0; DEEP && j0 < nhh; j0 += kHH) {
@@ -644,7 +652,7 @@ __device__ __forceinline__ void hx3_rows(const Smem3<T, A> &s, const int omega, 
                 const bool ok = j0 + u < nhh;
                 const T *xb = s.hp[ok ? j0 + u : 0];
 #pragma unroll
-                for (int i = 0; i < RR; ++i) v[u][i] = (ok && rv[i]) ? __ldg(xb + tid + i * kThreads) : T(0);
+                for (int i = 0; i < RR; ++i) v[u][i] = (ok && rv[i]) ? __ldg(xb + ro[i]) : T(0);
             }
 #pragma unroll
             for (int u = 0; u < kHH; ++u) {
@@ -714,16 +722,18 @@ __device__ __forceinline__ void hx3_rows(const Smem3<T, A> &s, const int omega, 
         const int r = tid + i * kThreads;
         if (r < nk) y[base + r] = TY(acc[i]);
     }
-    if (swdot) warp_dot<T, A, RR>(acc, s.x, nk, swdot);
+    if (swdot) warp_dot<T, A, RR>(acc, s.x, nk, swdot, ro);
 }
 
 // One basis block of y = H x in variant 3.  Called by every thread after a
 // barrier that frees the previous block's shared memory.
-template <typename T, typename A, int R, bool DEEP, typename TY>
+// KEPT: kept_first and kept_rows are the block's kept states, kept_low their low words
+template <typename T, typename A, int R, bool DEEP, typename TY, bool KEPT = false>
 __device__ __forceinline__ void hx3_block(const Smem3<T, A> &s, const int omega, const int L, const int H,
                                           const int N, const uint64_t h, const uint64_t base,
                                           const uint16_t *__restrict__ lowword, const T *__restrict__ x,
-                                          TY *__restrict__ y, double *swdot)
+                                          TY *__restrict__ y, double *swdot, const int64_t kept_first = 0,
+                                          const int kept_rows = 0, const uint16_t *__restrict__ kept_low = nullptr)
 {
     const int tid = threadIdx.x;
     const int ph = __popcll(h);
@@ -734,7 +744,9 @@ __device__ __forceinline__ void hx3_block(const Smem3<T, A> &s, const int omega,
     const int nk = (int)s.bin[k];
     int lo_off = 0;
     for (int j = 0; j < k; ++j) lo_off += (int)s.bin[j];
-    const uint16_t *lw = lowword + lo_off;
+    const uint16_t *lw = KEPT ? kept_low + kept_first : lowword + lo_off;
+    const int nr = KEPT ? kept_rows : nk;         // rows to compute, and the index of the first
+    const uint64_t first = KEPT ? (uint64_t)kept_first : base;
 
     for (int r = tid; r < nk; r += kThreads) s.x[r] = x[base + r];
     if (tid < 32) {                               // warp 0: positions and prefix sums of the high pairs
@@ -810,19 +822,20 @@ __device__ __forceinline__ void hx3_block(const Smem3<T, A> &s, const int omega,
     }
     __syncthreads();                              // hop tables visible
     // the row work, unrolled for the rows per thread this block needs
-    const int rpt = (nk + kThreads - 1) / kThreads;
-    if (rpt <= 1) hx3_rows<T, A, 1, DEEP>(s, omega, L, h, base, lw, y, swdot, k, ph, nemp, nhh, nk);
+    const int rpt = (nr + kThreads - 1) / kThreads;
+    if (rpt <= 1) hx3_rows<T, A, 1, DEEP, KEPT>(s, omega, L, h, first, lw, y, swdot, k, ph, nemp, nhh, nr);
     else if (rpt <= 2)
-        hx3_rows<T, A, (R < 2 ? R : 2), DEEP>(s, omega, L, h, base, lw, y, swdot, k, ph, nemp, nhh, nk);
+        hx3_rows<T, A, (R < 2 ? R : 2), DEEP, KEPT>(s, omega, L, h, first, lw, y, swdot, k, ph, nemp, nhh, nr);
     else if (rpt <= 4)
-        hx3_rows<T, A, (R < 4 ? R : 4), DEEP>(s, omega, L, h, base, lw, y, swdot, k, ph, nemp, nhh, nk);
-    else hx3_rows<T, A, R, DEEP>(s, omega, L, h, base, lw, y, swdot, k, ph, nemp, nhh, nk);
+        hx3_rows<T, A, (R < 4 ? R : 4), DEEP, KEPT>(s, omega, L, h, first, lw, y, swdot, k, ph, nemp, nhh, nr);
+    else hx3_rows<T, A, R, DEEP, KEPT>(s, omega, L, h, first, lw, y, swdot, k, ph, nemp, nhh, nr);
 }
 
 // OCC: resident CTAs per SM the register budget is cut for (4: 64 registers;
 // 5: 48 registers, variant 5, more warps to hide the gathers' latency).
 // TY: the type of y (double for float-float rows of an FP32 x)
-template <typename T, typename A, int R, bool DEEP, int OCC = 4, typename TY = T>
+// KEPT: a truncated space (x zero-extended to the full space, see kept_scatter_kernel)
+template <typename T, typename A, int R, bool DEEP, int OCC = 4, typename TY = T, bool KEPT = false>
 __global__ void __launch_bounds__(kThreads, OCC)
 hx3_kernel(const Blocks B, const A *__restrict__ Gg, const A *__restrict__ dg, const T *__restrict__ x,
            TY *__restrict__ y, Tickets *tk, const int *__restrict__ skip, double *blk_part, double *dot_out)
@@ -843,6 +856,9 @@ hx3_kernel(const Blocks B, const A *__restrict__ Gg, const A *__restrict__ dg, c
         s.bin[i] = __ldg(B.binom + (L + p) * kBinomStride + m);
     }
 
+    const int64_t nb = KEPT ? B.kept_nblocks : B.nblocks;
+    const uint64_t *__restrict__ bh = KEPT ? B.kept_blk_h : B.blk_h;
+    const uint64_t *__restrict__ bbase = KEPT ? B.kept_blk_base : B.blk_base;
     if (tid == 0) s_next[0] = (long long)atomicAdd(&tk->hx_next, 1ull);
     long long prev = -1;
     for (int it = 0;; it ^= 1) {
@@ -850,14 +866,31 @@ hx3_kernel(const Blocks B, const A *__restrict__ Gg, const A *__restrict__ dg, c
         const long long b = s_next[it];
         if (tid == 0) {
             block_sum_deferred(blk_part, prev, swdot);
-            if (b < B.nblocks) s_next[it ^ 1] = (long long)atomicAdd(&tk->hx_next, 1ull);
+            if (b < nb) s_next[it ^ 1] = (long long)atomicAdd(&tk->hx_next, 1ull);
         }
-        if (b >= B.nblocks) break;
-        hx3_block<T, A, R, DEEP>(s, omega, L, H, N, __ldg(B.blk_h + b), __ldg(B.blk_base + b), B.lowword, x, y,
-                           blk_part ? swdot : nullptr);
+        if (b >= nb) break;
+        if constexpr (KEPT)
+            hx3_block<T, A, R, DEEP, TY, true>(s, omega, L, H, N, __ldg(bh + b), __ldg(bbase + b), B.lowword, x, y,
+                                               blk_part ? swdot : nullptr, __ldg(B.kept_blk_first + b),
+                                               __ldg(B.kept_blk_rows + b), B.kept_low);
+        else
+            hx3_block<T, A, R, DEEP>(s, omega, L, H, N, __ldg(bh + b), __ldg(bbase + b), B.lowword, x, y,
+                                     blk_part ? swdot : nullptr);
         prev = b;
     }
-    hx_finish(tk, B.nblocks, blk_part, dot_out, sred);
+    hx_finish(tk, nb, blk_part, dot_out, sred);
+}
+
+// x of a truncated space into the full-space vector xf, which holds zeros at the
+// dropped states (they are never written)
+template <typename T>
+__global__ void __launch_bounds__(kThreads)
+kept_scatter_kernel(const uint64_t *__restrict__ full, int64_t n, const T *__restrict__ x, T *__restrict__ xf,
+                    const int *__restrict__ skip)
+{
+    if (skip && *skip) return;
+    for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads)
+        xf[__ldg(full + i)] = __ldg(x + i);
 }
 
 // Batched form of variant 3: the blocks of many problems in one launch (the
@@ -916,14 +949,16 @@ constexpr size_t kSmemLimit = 200 * 1024;
 template <typename T, typename A>
 bool use_v3(const Blocks &B)
 {
-    if ((B.variant < 2 || B.variant > 5) || B.kept_map) return false;
+    if ((B.variant < 2 || B.variant > 5) || (B.kept_map && !B.kept_low)) return false;
     return layout3<T, A>(B.omega, B.L, B.H, B.n, B.max_block, B.max_hh).total <= kSmemLimit;
 }
 
 template <typename T, typename A, int R>
 const void *kernel_fn(const Blocks &B)
 {
-    if (B.kept_map) return (const void *)hx_kernel<T, A, R, true>;
+    if (B.kept_map)
+        return use_v3<T, A>(B) ? (const void *)hx3_kernel<T, A, R, false, 4, T, true>
+                               : (const void *)hx_kernel<T, A, R, true>;
     if (use_v3<T, A>(B))
         return B.variant == 4   ? (const void *)hx3_kernel<T, A, R, true>
                : B.variant == 5 ? (const void *)hx3_kernel<T, A, R, false, 5>
@@ -948,7 +983,10 @@ cudaError_t launch_t(const Blocks &B, const A *G, const A *d, const void *x, voi
     if (err != cudaSuccess) return err;
     double *bp = dot ? dot->blk_part : nullptr;
     double *out = dot ? dot->out : nullptr;
-    if (B.kept_map)
+    if (B.kept_map && use_v3<T, A>(B))
+        hx3_kernel<T, A, R, false, 4, T, true><<<grid, kThreads, smem, st>>>(B, G, d, static_cast<const T *>(x),
+                                                                             static_cast<T *>(y), tk, skip, bp, out);
+    else if (B.kept_map)
         hx_kernel<T, A, R, true><<<grid, kThreads, smem, st>>>(B, G, d, static_cast<const T *>(x),
                                                                static_cast<T *>(y), tk, skip, bp, out);
     else if (use_v3<T, A>(B) && B.variant == 4)
@@ -1146,6 +1184,25 @@ trunc_map_kernel(const Blocks B, const double *__restrict__ d, double lo, double
     }
 }
 
+// full index and low word of every kept state
+__global__ void __launch_bounds__(kThreads)
+kept_list_kernel(const Blocks B, const int32_t *__restrict__ map, uint64_t *__restrict__ full,
+                 uint16_t *__restrict__ low)
+{
+    for (long long b = blockIdx.x; b < B.nblocks; b += gridDim.x) {
+        const uint64_t h = B.blk_h[b], base = B.blk_base[b];
+        const int k = B.n - __popcll(h);
+        const int nk = (int)B.binom[B.L * kBinomStride + k];
+        const uint16_t *lw = B.lowword + B.lo_off[k];
+        for (int r = threadIdx.x; r < nk; r += blockDim.x) {
+            const int32_t m = map[base + r];
+            if (m < 0) continue;
+            full[m] = base + r;
+            low[m] = lw[r];
+        }
+    }
+}
+
 // ---- occupation numbers 2 <v| S+_p S-_p |v> ------------------------------------
 __global__ void __launch_bounds__(kThreads)
 occ_kernel(const Blocks B, const double *__restrict__ v, double *__restrict__ part)
@@ -1267,6 +1324,26 @@ int hx_grid(const Blocks &B, int precision)
 {
     if (precision == 2) return ff_fits(B) ? grid_ff(B) : 0;
     return precision == 0 ? grid_prec<double, double>(B) : grid_prec<float, float>(B);
+}
+
+bool hx_kept_direct(const Blocks &B, int precision)
+{
+    return B.kept_map && (precision == 0 ? use_v3<double, double>(B) : use_v3<float, float>(B));
+}
+
+cudaError_t kept_scatter_launch(int dtype, const uint64_t *full, int64_t n, const void *x, void *xf, cudaStream_t st,
+                                const int *skip)
+{
+    const int64_t g = (n + kThreads - 1) / kThreads;
+    const int grid = (int)(g < 8 * sm_count() ? (g > 0 ? g : 1) : 8 * sm_count());
+    if (dtype == 0)
+        kept_scatter_kernel<double><<<grid, kThreads, 0, st>>>(full, n, static_cast<const double *>(x),
+                                                               static_cast<double *>(xf), skip);
+    else
+        kept_scatter_kernel<float><<<grid, kThreads, 0, st>>>(full, n, static_cast<const float *>(x),
+                                                              static_cast<float *>(xf), skip);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 cudaError_t hx_launch(const Blocks &B, const HxProblem &P, int precision, const void *x, void *y,
@@ -1459,6 +1536,14 @@ cudaError_t trunc_map_launch(const Blocks &B, const double *d64, double lo, doub
                              int64_t cut, const int64_t *blk_first, int32_t *map, int grid, cudaStream_t st)
 {
     trunc_map_kernel<<<grid, kThreads, 0, st>>>(B, d64, lo, hi, bins, cut, blk_first, map);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t kept_list_launch(const Blocks &B, const int32_t *map, uint64_t *full, uint16_t *low, int grid,
+                             cudaStream_t st)
+{
+    kept_list_kernel<<<grid, kThreads, 0, st>>>(B, map, full, low);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -92,6 +92,11 @@ struct Blocks {
     // the blocks holding at least one kept state (the truncated H*x walks only these)
     const uint64_t *kept_blk_h, *kept_blk_base;
     int64_t kept_nblocks;
+    // their first kept index and number of kept states, and the low words of all
+    // kept states; nullptr where the product looks every state up in kept_map
+    const int64_t *kept_blk_first;
+    const int *kept_blk_rows;
+    const uint16_t *kept_low;
 };
 
 // The FP32 product by pair removal on the tensor cores (variant 2, pd_hxf.cu).
@@ -336,6 +341,13 @@ cudaError_t hx_launch(const Blocks &B, const HxProblem &P, int precision, const 
                       Tickets *tk, int grid, cudaStream_t st, const int *skip = nullptr,
                       const HxDot *dot = nullptr);
 int hx_grid(const Blocks &B, int precision);
+// whether a truncated product takes a full-space x (zeros at the dropped
+// states), which kept_scatter_launch fills from the kept states' x
+bool hx_kept_direct(const Blocks &B, int precision);
+cudaError_t kept_scatter_launch(int dtype, const uint64_t *full, int64_t n, const void *x, void *xf, cudaStream_t st,
+                                const int *skip);
+cudaError_t kept_list_launch(const Blocks &B, const int32_t *map, uint64_t *full, uint16_t *low, int grid,
+                             cudaStream_t st);
 // variant 2 (pd_hxf.cu).  fac_fits: whether it serves a problem; fac_sizes: the
 // lengths of the device arrays, which the caller allocates; fac_build fills them.
 // fac_partials: doubles that a fused dot needs in blk_part.  fac_launch: as
