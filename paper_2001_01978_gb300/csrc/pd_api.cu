@@ -155,6 +155,7 @@ struct pairdiag {
     uint64_t *d_lpt_h = nullptr, *d_lpt_base = nullptr;
     Blocks B{};
     FacPlan fac;                     // the FP32 product by pair removal
+    unsigned char *d_fac = nullptr;  // its tables and scratch
     int device = 0;
     cudaStream_t st = nullptr;
     // tables
@@ -202,13 +203,6 @@ struct pairdiag {
 
 namespace {
 
-void free_fac(FacPlan &f)
-{
-    for (void *p : {(void *)f.twords, (void *)f.ywords, (void *)f.low, (void *)f.up, (void *)f.scratch, (void *)f.zeros})
-        pool_free(p);
-    f = FacPlan{};
-}
-
 void free_all(pairdiag *h)
 {
     for (auto &ev : h->hx_events) {
@@ -221,13 +215,12 @@ void free_all(pairdiag *h)
                     h->d_Q[0], h->d_Q[1], h->d_p[0], h->d_p[1], h->d_v64, h->d_w64,
                     h->d_L64, h->d_L32, h->d_lockc, h->d_kmap, h->d_kblk_h, h->d_kblk_base, h->d_kblk_first,
                     h->d_kblk_rows, h->d_kfull, h->d_klow, h->d_xf[0], h->d_xf[1],
-                    h->d_lpt_h, h->d_lpt_base, h->d_Gff, h->d_dff};
+                    h->d_lpt_h, h->d_lpt_base, h->d_Gff, h->d_dff, h->d_fac};
     // the blocks go back to the library's cache: no queued kernel may still use
     // them.  Every kernel and copy of the handle runs on its stream, so that
     // stream's completion is enough (other streams of the caller go on).
     cudaStreamSynchronize(h->st);
     for (void *p : ptrs) pool_free(p);
-    free_fac(h->fac);
 }
 
 template <typename T>
@@ -341,16 +334,30 @@ int build_fac(pairdiag *h)
     f = FacPlan{};
     if (!fac_fits(h->omega, h->n, h->full_dim)) return PD_OK;
     fac_sizes(h->omega, h->n, f);
-    const bool ok = dalloc(&f.twords, (size_t)f.nt) == PD_OK && dalloc(&f.ywords, (size_t)f.ny) == PD_OK &&
-                    dalloc(&f.low, (size_t)1 << f.L) == PD_OK && dalloc(&f.up, (size_t)f.table) == PD_OK &&
-                    dalloc(&f.zeros, fac_zeros()) == PD_OK &&
-                    dalloc(&f.scratch, (size_t)std::max<int64_t>(f.scratch_len, 1)) == PD_OK;
-    if (!ok) {                                    // no room: the kernels without scratch serve the handle
-        free_fac(f);
+    // one allocation for all of it
+    size_t off = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = off;
+        off = (off + bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t at_t = place(sizeof(uint32_t) * (size_t)f.nt), at_y = place(sizeof(uint32_t) * (size_t)f.ny),
+                 at_low = place(sizeof(uint16_t) << f.L), at_up = place(sizeof(uint32_t) * (size_t)f.table),
+                 at_z = place(sizeof(float) * fac_zeros()), at_s = place(sizeof(float) * (size_t)f.scratch_len);
+    if (dalloc(&h->d_fac, off) != PD_OK) {        // no room: the kernels without scratch serve the handle
+        h->d_fac = nullptr;
+        f = FacPlan{};
         return PD_OK;
     }
+    f.twords = reinterpret_cast<uint32_t *>(h->d_fac + at_t);
+    f.ywords = reinterpret_cast<uint32_t *>(h->d_fac + at_y);
+    f.low = reinterpret_cast<uint16_t *>(h->d_fac + at_low);
+    f.up = reinterpret_cast<uint32_t *>(h->d_fac + at_up);
+    f.zeros = reinterpret_cast<float *>(h->d_fac + at_z);
+    f.scratch = reinterpret_cast<float *>(h->d_fac + at_s);
+    // (on the legacy stream: the blocking uploads that follow in pairdiag_create
+    // are ordered after it)
     PD_CUDA(fac_build(f, h->d_binom, h->st));
-    PD_CUDA(cudaStreamSynchronize(h->st));        // the handle may move to another stream
     return PD_OK;
 }
 
