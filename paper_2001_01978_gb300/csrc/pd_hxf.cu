@@ -576,7 +576,7 @@ add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const
 {
     if (skip && *skip) return;                    // CTA-uniform
     __shared__ double sred[kAThreads / 32];
-    __shared__ uint32_t bin[kMaxHigh * (kMaxHigh + kLT)];   // C(L + p, m), m < N + 2
+    __shared__ uint32_t bin[kMaxHigh * (kMaxHigh + kLT + 1)];   // C(L + p, m), m < N + 2, N < omega
     const int lane = threadIdx.x & 31;
     const int NB = A.N + 2;
     for (int i = threadIdx.x; i < A.H * NB; i += kAThreads)
