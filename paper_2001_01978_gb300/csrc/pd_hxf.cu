@@ -189,16 +189,22 @@ __device__ __forceinline__ void copy_async4(float *dst, const float *src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
-// The last warp: block of t with high word h into buffer bs.  Lane j: high orbit
-// j.  k = N - popcount(h) low pairs in block h of x, k - 1 in the words t.  With
-// A, B(j) the binomials of the pair on j at its own ordinal and one lower, EA, EB
-// their sums over the occupied high orbits below j, block h + q of x starts at
+// Block of t with high word h, by one warp; lane j: high orbit j.  k = N -
+// popcount(h) low pairs in block h of x, k - 1 in the words t.  With A, B(j) the
+// binomials of the pair on j at its own ordinal and one lower, EA, EB their sums
+// over the occupied high orbits below j, block h + q of x starts at
 //     EB(q) + C(L + q, k + #below) + base(h) - EA(q)     (modulo 2^32)
 // and its place among the words of its class is, with R(j) = C(j, ordinal from 1)
 // and S(j) = C(j, ordinal + 1),   ER(q) + C(q, #below + 1) + sum S - ES(q).
-__device__ __forceinline__ void prepare_block(BlockSmem &bs, const RemoveArgs &A, const uint32_t h,
-                                              const uint32_t *bin, const uint32_t *crk, const float *dh,
-                                              const float *__restrict__ x)
+struct HighWord {
+    uint32_t base;                       // start of block h of x
+    float dh;                            // diagonal sum of its high orbits
+    bool hop;                            // this lane's orbit exists and is empty; if so:
+    uint32_t x;                          // start of block h + q of x
+    int64_t z;                           // where the results for orbit q go in the scratch
+};
+__device__ __forceinline__ HighWord high_word(const RemoveArgs &A, const uint32_t h, const uint32_t *bin,
+                                              const uint32_t *crk, const float *dh)
 {
     const int lane = threadIdx.x & 31;
     const int N = A.N, H = A.H;
@@ -223,27 +229,39 @@ __device__ __forceinline__ void prepare_block(BlockSmem &bs, const RemoveArgs &A
         const uint32_t ts = __shfl_up_sync(0xffffffffu, is, o);
         if (lane >= o) { ia += ta; ib += tb; ir += tr; is += ts; }
     }
-    const uint32_t base = __shfl_sync(0xffffffffu, ia, 31), stot = __shfl_sync(0xffffffffu, is, 31);
+    const uint32_t stot = __shfl_sync(0xffffffffu, is, 31);
+    HighWord w;
+    w.base = __shfl_sync(0xffffffffu, ia, 31);
+    w.hop = lane < H && !occ;
+    // (lanes of empty orbits: the inclusive sums are the exclusive ones)
+    w.x = ib + bq + w.base - ia;
+    const uint64_t place = (uint32_t)(ir + c1 + stot - is);
+    const int nt = A.lo_off[k] - A.lo_off[k - 1];
+    w.z = A.zbase[k - 1] + (int64_t)(place * (uint64_t)(ph + 1) + (uint64_t)io) * nt;
+    w.dh = occ ? dh[lane] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w.dh += __shfl_xor_sync(0xffffffffu, w.dh, o);
+    return w;
+}
+
+// the last warp: block of t with high word h into buffer bs
+__device__ __forceinline__ void prepare_block(BlockSmem &bs, const RemoveArgs &A, const uint32_t h,
+                                              const uint32_t *bin, const uint32_t *crk, const float *dh,
+                                              const float *__restrict__ x)
+{
+    const int lane = threadIdx.x & 31;
+    const int k = A.N - __popc(h);
+    const HighWord w = high_word(A, h, bin, crk, dh);
     if (k <= A.L) {                               // block h exists (t is not the full low word)
         const int nk = A.lo_off[k + 1] - A.lo_off[k];
-        for (int r = lane; r < nk; r += 32) copy_async4(bs.x + r, x + base + r);
+        for (int r = lane; r < nk; r += 32) copy_async4(bs.x + r, x + w.base + r);
     }
-    if (occ || lane >= H) {
-        bs.xe[lane] = A.zeros;
-    } else {
-        // (lanes of empty orbits: the inclusive sums are the exclusive ones)
-        bs.xe[lane] = x + (uint32_t)(ib + bq + base - ia);
-        const uint64_t place = (uint32_t)(ir + c1 + stot - is);
-        const int nt = A.lo_off[k] - A.lo_off[k - 1];
-        bs.ze[lane] = A.scratch + A.zbase[k - 1] + (int64_t)(place * (uint64_t)(ph + 1) + (uint64_t)io) * nt;
-    }
-    float Dh = occ ? dh[lane] : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) Dh += __shfl_xor_sync(0xffffffffu, Dh, o);
+    bs.xe[lane] = w.hop ? x + w.x : A.zeros;
+    if (w.hop) bs.ze[lane] = A.scratch + w.z;
     if (lane == 0) {
         bs.h = h;
-        bs.base = base;
-        bs.dh = Dh;
+        bs.base = w.base;
+        bs.dh = w.dh;
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
@@ -299,6 +317,63 @@ __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&v)[8])
                  : "memory");
 }
 
+// G and the tables of a CTA into shared memory
+template <int KP>
+__device__ __forceinline__ void stage_tables(const RemoveArgs &A, const float *__restrict__ G, const float *__restrict__ d,
+                                             unsigned char *g_smem, uint32_t *bin, uint32_t *crk, float *dh, float *dlow,
+                                             const int threads)
+{
+    using C = Cfg<KP>;
+    const int omega = A.omega, L = A.L, H = A.H, N = A.N, tid = threadIdx.x;
+    // G in the operand layout, high and low parts (row n: the orbit that
+    // receives the pair, column k: the orbit it leaves)
+    for (int i = tid; i < C::kN * KP; i += threads) {
+        const int n = i / KP, k = i % KP;
+        auto orbit = [&](int c) { return c < kLT ? (c < L ? c : -1) : (c - kLT < H ? L + c - kLT : -1); };
+        const int on = orbit(n), ok = orbit(k);
+        const float g = (on >= 0 && ok >= 0 && on != ok) ? G[on * omega + ok] : 0.0f;
+        const float hi = to_tf32(g);
+        unsigned char *p = g_smem + (n >> 3) * (KP * 32) + (k >> 2) * 128 + (n & 7) * 16 + (k & 3) * 4;
+        *reinterpret_cast<float *>(p) = hi;
+        *reinterpret_cast<float *>(p + 4 * C::kN * KP) = to_tf32(g - hi);
+    }
+    for (int i = tid; i < H * (N + 2); i += threads)
+        bin[i] = (uint32_t)__ldg(A.binom + (L + i / (N + 2)) * kBinomStride + i % (N + 2));
+    for (int i = tid; i < H * (H + 2); i += threads)
+        crk[i] = (uint32_t)__ldg(A.binom + (i / (H + 2)) * kBinomStride + i % (H + 2));
+    for (int i = tid; i < H; i += threads) dh[i] = d[L + i];
+    for (int i = tid; i < 128; i += threads) {   // diagonal sums of the two halves of a low word
+        const int w = i & 63, p0 = i < 64 ? 0 : 6;
+        float v = 0.0f;
+        for (int p = 0; p < 6; ++p)
+            if ((w >> p & 1) && p0 + p < L) v += d[p0 + p];
+        dlow[i] = v;
+    }
+}
+
+// Z = V G of one tile (one thread): TF32 operands, FP32 accumulator, both K-major, M = 128
+template <int KP>
+__device__ __forceinline__ void issue_product(const uint32_t tmem, const uint32_t g_smem, const uint32_t bar)
+{
+    using C = Cfg<KP>;
+    constexpr uint32_t idesc =
+        (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(C::kN >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+    const uint64_t b0 = g_desc<KP>(g_smem);
+#pragma unroll
+    for (int s = 0; s < 3; ++s)
+#pragma unroll
+        for (int kk = 0; kk < KP / 8; ++kk) {
+            const uint32_t a = tmem + (s == 1 ? KP : 0) + 8 * kk;
+            const uint64_t db = b0 + (uint64_t)(((s == 2 ? 4 * C::kN * KP : 0) + kk * 256) >> 4);
+            const uint32_t accum = (s || kk) ? 1u : 0u;
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                         "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem + 2 * KP),
+                         "r"(a), "l"(db), "r"(idesc), "r"(accum)
+                         : "memory");
+        }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+
 // What bounds it: instruction issue and the latency of a tile's chain (gather,
 // split, tensor-memory store, product, load, scatter).  Two CTAs of three groups
 // share an SM's tensor memory, so that one group's gathers overlap another's
@@ -320,7 +395,7 @@ remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G,
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t s_bar[C::kGroups];
     __shared__ uint32_t s_tmem;
-    const int omega = A.omega, L = A.L, H = A.H, N = A.N;
+    const int L = A.L, H = A.H, N = A.N;
     const LayoutR lay = layout_r(KP, H, N);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, group = warp >> 2;
     uint32_t *bin = reinterpret_cast<uint32_t *>(smem + lay.bin), *crk = reinterpret_cast<uint32_t *>(smem + lay.crk);
@@ -338,30 +413,7 @@ remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G,
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&s_bar[g])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    // G in the operand layout, high and low parts (row n: the orbit that
-    // receives the pair, column k: the orbit it leaves)
-    for (int i = tid; i < C::kN * KP; i += C::kThreads) {
-        const int n = i / KP, k = i % KP;
-        auto orbit = [&](int c) { return c < kLT ? (c < L ? c : -1) : (c - kLT < H ? L + c - kLT : -1); };
-        const int on = orbit(n), ok = orbit(k);
-        const float g = (on >= 0 && ok >= 0 && on != ok) ? G[on * omega + ok] : 0.0f;
-        const float hi = to_tf32(g);
-        unsigned char *p = smem + lay.b + (n >> 3) * (KP * 32) + (k >> 2) * 128 + (n & 7) * 16 + (k & 3) * 4;
-        *reinterpret_cast<float *>(p) = hi;
-        *reinterpret_cast<float *>(p + 4 * C::kN * KP) = to_tf32(g - hi);
-    }
-    for (int i = tid; i < H * (N + 2); i += C::kThreads)
-        bin[i] = (uint32_t)__ldg(A.binom + (L + i / (N + 2)) * kBinomStride + i % (N + 2));
-    for (int i = tid; i < H * (H + 2); i += C::kThreads)
-        crk[i] = (uint32_t)__ldg(A.binom + (i / (H + 2)) * kBinomStride + i % (H + 2));
-    for (int i = tid; i < H; i += C::kThreads) dh[i] = d[L + i];
-    for (int i = tid; i < 128; i += C::kThreads) {   // diagonal sums of the two halves of a low word
-        const int w = i & 63, p0 = i < 64 ? 0 : 6;
-        float v = 0.0f;
-        for (int p = 0; p < 6; ++p)
-            if ((w >> p & 1) && p0 + p < L) v += d[p0 + p];
-        dlow[i] = v;
-    }
+    stage_tables<KP>(A, G, d, smem + lay.b, bin, crk, dh, dlow, C::kThreads);
     if (tid < 3) bufs[tid].x[kSpare] = 0.0f;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // G: generic stores -> tensor core reads
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -462,30 +514,11 @@ remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G,
                     asm volatile("bar.sync %0, 128;\n" ::"r"(group + 1) : "memory");
                     if ((tid & (kTile - 1)) == 0) {
                         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        // TF32 operands, FP32 accumulator, both K-major, M = 128
-                        constexpr uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) |
-                                                   ((uint32_t)(C::kN >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
-                        const uint64_t b0 = g_desc<KP>(smem_u32(smem + lay.b));
-#pragma unroll
-                        for (int s = 0; s < 3; ++s)
-#pragma unroll
-                            for (int kk = 0; kk < KP / 8; ++kk) {
-                                const uint32_t a = tmem + (s == 1 ? KP : 0) + 8 * kk;
-                                const uint64_t db = b0 + (uint64_t)(((s == 2 ? 4 * C::kN * KP : 0) + kk * 256) >> 4);
-                                const uint32_t accum = (s || kk) ? 1u : 0u;
-                                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                             "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(
-                                                 tmem + 2 * KP),
-                                             "r"(a), "l"(db), "r"(idesc), "r"(accum)
-                                             : "memory");
-                            }
-                        asm volatile(
-                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
-                            : "memory");
+                        issue_product<KP>(tmem, smem_u32(smem + lay.b), bar);
                     }
                     __syncwarp();
                     if ((c + C::kGroups) * kTile < nt) load(c + C::kGroups);   // overlaps the product
-                    if (!mbar_wait(bar, phase)) gave_up = true;
+                    if (gave_up || !mbar_wait(bar, phase)) gave_up = true;
                     phase ^= 1u;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     for_each<KP / 8>([&](auto gc) {
@@ -520,6 +553,245 @@ remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G,
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s_tmem), "r"(kTmemCols) : "memory");
     if (arrive_last(&tk->hx_done) && tid == 0) tk->hx_next = 0ull;
+}
+
+// ---- pair removal, small blocks -------------------------------------------------
+// Classes whose blocks have few words t (1, 12 or 66 of the 128 of a tile): a
+// group of four warps takes several high words of one class together.  Far from
+// half filling these are nearly all blocks: 565,000 of the 600,000 of Omega=34,
+// N=9, whose lone tiles held 12 words and less and left one of the two groups of
+// remove_kernel's CTA without work.
+constexpr int kSmallWords = 66;          // most words t per block of such a class
+constexpr int kSmallRows = 660;          // most rows, and words t, of the blocks taken together
+constexpr int kSmallStride = 664;        // floats per orbit of their partial results
+constexpr int kSmallBlocks = 32;         // most blocks taken together
+constexpr int kSmallClasses = 6;
+constexpr int kSmallGroups = 2;          // groups per CTA; two CTAs per SM
+// Fewest such blocks that get a launch of their own (in remove_kernel / on their
+// own): 990 blocks, C(30,4), 31.0 / 38.7 us, 1456, C(26,5), 33.8 / 40.4 us, 3682,
+// C(40,4), 71.8 / 43.1 us.
+constexpr int kSmallMin = 2000;
+
+struct SmallArgs {
+    RemoveArgs r;
+    int n;                               // classes
+    int k[kSmallClasses], m[kSmallClasses];   // low pairs of the rows; blocks per item
+    int64_t first[kSmallClasses], end[kSmallClasses];   // words of the class
+    int64_t item[kSmallClasses + 1];     // number of the class's first item
+};
+struct LayoutS {
+    size_t b, dlow, bin, crk, dh, group, part, x, h, base, bdh, xe, ze, per_group, total;
+};
+__host__ __device__ inline LayoutS layout_s(int KP, int H, int N)
+{
+    LayoutS s;
+    const int np = (KP + 15) / 16 * 16;
+    size_t off = 0;
+    s.b = off;    off = align16(off + sizeof(float) * 2 * np * KP);
+    s.dlow = off; off = align16(off + sizeof(float) * 128);
+    s.bin = off;  off = align16(off + sizeof(uint32_t) * H * (N + 2));
+    s.crk = off;  off = align16(off + sizeof(uint32_t) * H * (H + 2));
+    s.dh = off;   off = align16(off + sizeof(float) * H);
+    s.group = off;
+    off = 0;      // per group
+    s.part = off; off += sizeof(float) * kLT * kSmallStride;
+    s.x = off;    off += sizeof(float) * kSmallStride;
+    s.h = off;    off += sizeof(uint32_t) * kSmallBlocks;
+    s.base = off; off += sizeof(uint32_t) * kSmallBlocks;
+    s.bdh = off;  off += sizeof(float) * kSmallBlocks;
+    s.xe = off;   off += sizeof(uint32_t) * kSmallBlocks * H;
+    s.ze = off;   off += sizeof(uint32_t) * kSmallBlocks * H;
+    s.per_group = align16(off);
+    s.total = s.group + kSmallGroups * s.per_group;
+    return s;
+}
+
+// What bounds it: the latency of an item's chain (starts of the blocks, gather,
+// product, scatter, rows: about 8 us), of which only four overlap per SM, because
+// the operands of four tiles fill its tensor memory.  Omega=34, N=9: 0.73 ms for
+// these blocks and 0.57 ms for the others, against 5.1 ms for both in
+// remove_kernel.  Measured and not kept: the rows' sums over the set bits of a
+// low word instead of twelve predicated loads, 0.76 ms.
+template <int KP>
+__global__ void __launch_bounds__(128 * kSmallGroups, 2)
+remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict__ G, const float *__restrict__ d,
+                    const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip)
+{
+    using C = Cfg<KP>;
+    static_assert(kSmallGroups * C::kCols <= kTmemCols, "tensor memory of a CTA");
+    if (skip && *skip) return;                    // CTA-uniform
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t s_bar[kSmallGroups];
+    __shared__ uint32_t s_tmem;
+    const RemoveArgs &A = S.r;
+    const int L = A.L, H = A.H, N = A.N;
+    const LayoutS lay = layout_s(KP, H, N);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, group = warp >> 2, gt = tid & 127;
+    uint32_t *bin = reinterpret_cast<uint32_t *>(smem + lay.bin), *crk = reinterpret_cast<uint32_t *>(smem + lay.crk);
+    float *dlow = reinterpret_cast<float *>(smem + lay.dlow), *dh = reinterpret_cast<float *>(smem + lay.dh);
+    unsigned char *mine = smem + lay.group + group * lay.per_group;
+    float *part = reinterpret_cast<float *>(mine + lay.part), *bx = reinterpret_cast<float *>(mine + lay.x);
+    uint32_t *bh = reinterpret_cast<uint32_t *>(mine + lay.h), *bbase = reinterpret_cast<uint32_t *>(mine + lay.base);
+    float *bdh = reinterpret_cast<float *>(mine + lay.bdh);
+    uint32_t *xe = reinterpret_cast<uint32_t *>(mine + lay.xe), *ze = reinterpret_cast<uint32_t *>(mine + lay.ze);
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int g = 0; g < kSmallGroups; ++g)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&s_bar[g])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    stage_tables<KP>(A, G, d, smem + lay.b, bin, crk, dh, dlow, 128 * kSmallGroups);
+    if (gt == 0) bx[kSmallRows] = 0.0f;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // G: generic stores -> tensor core reads
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = s_tmem + (uint32_t)group * C::kCols;
+    const uint32_t trow = tmem + ((uint32_t)(warp & 3) << 21);       // this warp's 32 lanes
+    const uint32_t bar = smem_u32(&s_bar[group]);
+    uint32_t phase = 0;
+    bool gave_up = false, odd = false;
+    auto sync = [&] { asm volatile("bar.sync %0, 128;\n" ::"r"(group + 1) : "memory"); };
+
+    // Items in turn (sorted by class, so every group gets its share of each).
+    // Block i of an item belongs to warp i % 4; lane j holds the word of the
+    // warp's j-th block, loaded one item ahead.
+    struct Item {
+        int k, m;                        // low pairs of the rows, blocks
+        uint32_t word;
+    };
+    int c = 0;
+    auto fetch = [&](int64_t it) {
+        Item t{0, 0, 0u};
+        if (it >= S.item[S.n]) return t;
+        while (it >= S.item[c + 1]) ++c;
+        const int64_t b = S.first[c] + (it - S.item[c]) * S.m[c];
+        t.k = S.k[c];
+        t.m = (int)min((int64_t)S.m[c], S.end[c] - b);
+        const int i = (warp & 3) + 4 * lane;
+        if (i < t.m) t.word = __ldg(A.words + b + i);
+        return t;
+    };
+    const int64_t step = (int64_t)gridDim.x * kSmallGroups;
+    int64_t it = (int64_t)blockIdx.x * kSmallGroups + group;
+    Item cur = fetch(it);
+    while (cur.m > 0) {
+        it += step;
+        const Item nxt = fetch(it);
+        const int k = cur.k, m = cur.m;
+        const int lo_t = A.lo_off[k - 1], nt = A.lo_off[k] - lo_t;
+        const int lo_k = A.lo_off[k], nk = k <= L ? A.lo_off[k + 1] - lo_k : 0;
+        for (int j = 0, i = warp & 3; i < m; ++j, i += 4) {
+            const uint32_t h = __shfl_sync(0xffffffffu, cur.word, j);
+            const HighWord w = high_word(A, h, bin, crk, dh);
+            for (int r = lane; r < nk; r += 32) copy_async4(bx + i * nk + r, x + w.base + r);
+            if (w.hop) {
+                xe[i * H + lane] = w.x;
+                ze[i * H + lane] = (uint32_t)w.z;
+            }
+            if (lane == 0) {
+                bh[i] = h;
+                bbase[i] = w.base;
+                bdh[i] = w.dh;
+            }
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        sync();
+        const int words = m * nt;
+        for (int r0 = 0; r0 < words; r0 += kTile) {
+            const bool in = r0 + gt < words;
+            const int r = in ? r0 + gt : words - 1;
+            const int i = r / nt, t = r - i * nt;
+            const uint32_t h = bh[i];
+            uint32_t hop[kLT / 2];
+            // offsets into the item's rows; beyond its last row: the spare element
+            const uint32_t shift = (uint32_t)(4 * i * nk) * 0x10001u;
+#pragma unroll
+            for (int p = 0; p < kLT / 2; ++p)
+                hop[p] = __vminu2(__ldg(A.up + (p << L) + lo_t + t) + shift, 4 * kSmallRows * 0x10001u);
+            float vh[KP - kLT];
+#pragma unroll
+            for (int q = 0; q < KP - kLT; ++q)
+                vh[q] = q < H && !(h >> q & 1u) ? __ldg(x + (uint32_t)(xe[i * H + q] + t)) : 0.0f;
+            for_each<KP / 8>([&](auto gc) {
+                constexpr int g = decltype(gc)::value;
+                float v[8], hi[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int p = 8 * g + u;
+                    if (p < kLT) {
+                        const uint32_t off = (p & 1) ? hop[p / 2] >> 16 : hop[p / 2] & 0xffffu;
+                        v[u] = *reinterpret_cast<const float *>(reinterpret_cast<const char *>(bx) + off);
+                    } else {
+                        v[u] = vh[p - kLT];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    hi[u] = to_tf32(v[u]);
+                    v[u] -= hi[u];
+                }
+                tmem_st8(trow + 8 * g, hi);
+                tmem_st8(trow + KP + 8 * g, v);
+            });
+            asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+            sync();
+            if (gt == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                issue_product<KP>(tmem, smem_u32(smem + lay.b), bar);
+            }
+            __syncwarp();
+            if (gave_up || !mbar_wait(bar, phase)) gave_up = true;
+            phase ^= 1u;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            for_each<KP / 8>([&](auto gc) {
+                constexpr int g = decltype(gc)::value;
+                uint32_t z[8];
+                tmem_ld8(trow + 2 * KP + 8 * g, z);
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if (g == 0) odd |= __uint_as_float(z[0]) != __uint_as_float(z[0]);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int p = 8 * g + u;
+                    if (p < kLT) {
+                        const uint32_t off = (p & 1) ? hop[p / 2] >> 16 : hop[p / 2] & 0xffffu;
+                        *reinterpret_cast<float *>(reinterpret_cast<char *>(part) + p * kSmallStride * 4 + off) =
+                            __uint_as_float(z[u]);
+                    } else if (in && p - kLT < H && !(h >> (p - kLT) & 1u)) {
+                        A.scratch[(uint32_t)(ze[i * H + p - kLT] + t)] = __uint_as_float(z[u]);
+                    }
+                }
+            });
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        }
+        sync();
+#pragma unroll 2
+        for (int r = gt; r < m * nk; r += 128) {
+            const int i = r / nk, t = r - i * nk;
+            const uint32_t l = __ldg(A.low + lo_k + t);
+            const float D = (dlow[l & 63u] + dlow[64 + (l >> 6)]) + bdh[i];
+            float s = 0.0f;
+#pragma unroll
+            for (int o = 0; o < kLT; ++o)
+                if (l >> o & 1u) s += part[o * kSmallStride + r];
+            y[bbase[i] + t] = fmaf(D, bx[r], s);
+        }
+        sync();
+        cur = nxt;
+    }
+    if (odd) atomicOr(&tk->pad, 1ull);
+    if (gave_up) atomicExch(&tk->bar.err, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s_tmem), "r"(kTmemCols) : "memory");
 }
 
 // ---- pair addition --------------------------------------------------------------
@@ -562,6 +834,23 @@ __device__ __noinline__ float row_slow(const AddArgs &A, const float *__restrict
         }
     }
     return acc;
+}
+
+// the last CTA sums the partial dot products
+__device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float> &dot, Tickets *tk, double *part,
+                                           double *dot_out, double *sred)
+{
+    if (part) {
+        const double v = block_reduce(dot, sred);
+        if (threadIdx.x == 0) part[blockIdx.x] = v;
+    }
+    if (!arrive_last(&tk->hx_done)) return;
+    if (A.last_launch && threadIdx.x == 0) tk->pad = 0ull;
+    if (!part) return;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kAThreads) s += __ldcg(part + i);
+    s = block_sum(s, sred);
+    if (threadIdx.x == 0) *dot_out = A.first_launch ? s : *dot_out + s;
 }
 
 // y(h, l) += sum over the pairs a of h of scratch(h, a, l); fused x^T y.  Bound
@@ -642,18 +931,57 @@ add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const
             }
         }
     }
-    double v = 0.0;
-    if (part) {
-        v = block_reduce(dot, sred);
-        if (threadIdx.x == 0) part[blockIdx.x] = v;
+    finish_add(A, dot, tk, part, dot_out, sred);
+}
+
+// The rows of classes with small blocks (at most kAddSmall rows): one thread per
+// row, numbered through the class, where add_kernel has one block per CTA and
+// pass.  Omega=34, N=9 (990,000 blocks of 1, 12 and 66 rows): 0.18 ms for these
+// rows and 0.26 ms for the others, against 1.68 ms for both in add_kernel; 445 us
+// for 1.6 GB is 0.55 of the measured copy rate, the scattered y rows included.
+constexpr int kAddSmall = 66;
+__global__ void __launch_bounds__(kAThreads, kACtas)
+add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const float *__restrict__ d,
+                 const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip,
+                 double *part, double *dot_out)
+{
+    if (skip && *skip) return;                    // CTA-uniform
+    __shared__ double sred[kAThreads / 32];
+    __shared__ uint32_t bin[kMaxHigh * (kMaxHigh + kLT + 1)];
+    __shared__ float dh[kMaxHigh];
+    const int NB = A.N + 2;
+    for (int i = threadIdx.x; i < A.H * NB; i += kAThreads)
+        bin[i] = (uint32_t)__ldg(A.binom + (A.L + i / NB) * kBinomStride + i % NB);
+    for (int i = threadIdx.x; i < A.H; i += kAThreads) dh[i] = d[A.L + i];
+    const bool slow = *reinterpret_cast<volatile unsigned long long *>(&tk->pad) != 0ull;
+    __syncthreads();
+    DotAcc<float> dot;
+    for (int c = A.c0; c < A.c1; ++c) {
+        const int ph = A.ph[c], k = A.N - ph;
+        const uint32_t lo_k = A.lo_off[k], nk = A.lo_off[k + 1] - lo_k;
+        const int64_t rows = (A.first[c + 1] - A.first[c]) * nk;    // < 2^32
+        for (int64_t i = (int64_t)blockIdx.x * kAThreads + threadIdx.x; i < rows; i += (int64_t)gridDim.x * kAThreads) {
+            const uint32_t b = (uint32_t)i / nk, r = (uint32_t)i - b * nk;
+            const uint32_t h = __ldg(A.words + A.first[c] + b);
+            uint32_t base = r;
+            float Dh = 0.0f;
+            int o = k;
+            for (uint32_t w = h; w; w &= w - 1) {
+                const int j = __ffs(w) - 1;
+                base += bin[j * NB + ++o];
+                Dh += dh[j];
+            }
+            const float xr = part || k == 0 || slow ? __ldg(x + base) : 0.0f;
+            float acc = k == 0 ? Dh * xr : y[base];
+            const float *z = A.scratch + A.zbase[k] + (int64_t)b * ph * nk + r;
+#pragma unroll 4
+            for (int a = 0; a < ph; ++a, z += nk) acc += __ldg(z);
+            if (slow) acc = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr);
+            y[base] = acc;
+            if (part) dot.add(xr, acc);
+        }
     }
-    if (!arrive_last(&tk->hx_done)) return;
-    if (A.last_launch && threadIdx.x == 0) tk->pad = 0ull;
-    if (!part) return;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += kAThreads) s += __ldcg(part + i);
-    s = block_sum(s, sred);
-    if (threadIdx.x == 0) *dot_out = A.first_launch ? s : *dot_out + s;
+    finish_add(A, dot, tk, part, dot_out, sred);
 }
 
 template <int KP>
@@ -666,6 +994,11 @@ int padded(int omega)
 const void *remove_fn_of(int KP)
 {
     return KP == 16 ? remove_fn<16>() : KP == 24 ? remove_fn<24>() : KP == 32 ? remove_fn<32>() : remove_fn<40>();
+}
+// (up to 12 high orbits there are too few small blocks for a launch of their own)
+const void *remove_small_fn_of(int KP)
+{
+    return KP == 32 ? (const void *)remove_small_kernel<32> : KP == 40 ? (const void *)remove_small_kernel<40> : nullptr;
 }
 int remove_threads(int KP)
 {
@@ -685,8 +1018,8 @@ bool fac_fits(int omega, int n, int64_t dim)
 
 // Where variant 2 is the faster one and no less exact (variant 3 / variant 2,
 // FP32, back to back): C(17,6) 15.7 / 18.5 us, C(18,9) = 48620 18.7 / 20.6 us,
-// C(20,10) = 184756 31 / 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 7.4 ms,
-// C(34,9) 12.8 / 6.8 ms.  Far above half filling there are more words t than
+// C(20,10) = 184756 31 / 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 7.1 ms,
+// C(34,9) 12.8 / 1.8 ms.  Far above half filling there are more words t than
 // states and their rows are longer: C(24,16) 94 / 64 us, C(24,18) 48 / 41 us,
 // C(28,22) 141 / 211 us, and C(20,17) loses accuracy (2.2e-7 / 2.6e-7).
 bool fac_pays(int omega, int n, int64_t dim)
@@ -757,6 +1090,8 @@ cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st)
     const int KP = padded(p.omega);
     p.smem = layout_r(KP, H, p.n).total;
     e = cudaFuncSetAttribute(remove_fn_of(KP), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e == cudaSuccess && remove_small_fn_of(KP))
+        e = cudaFuncSetAttribute(remove_small_fn_of(KP), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
     if (e != cudaSuccess) return e;
     p.grid_t = 2 * sm_count();                    // two CTAs per SM share its tensor memory
     p.grid_y = kACtas * sm_count();
@@ -801,48 +1136,87 @@ cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, 
         R.zbase[k] = A.zbase[k] = z;
         z += (int64_t)host_binom(H, cy.ph[i]) * cy.ph[i] * (int64_t)host_binom(L, k);
     }
-    auto remove = [&](int64_t first, int64_t end) -> cudaError_t {
-        R.first = first;
-        R.end = end;
-        const int64_t grid = p.grid_t < end - first ? p.grid_t : end - first;
-        const void *args[] = {&R, &G, &d, &x, &y, &tk, &skip};
-        return cudaLaunchKernel(remove_fn_of(KP), dim3((unsigned)grid), dim3((unsigned)remove_threads(KP)),
-                                const_cast<void **>(args), p.smem, st);
+    const void *small_fn = remove_small_fn_of(KP);
+    // classes [c0, c1) of t: those of small blocks, at the end, on their own if
+    // they are many
+    auto remove = [&](int c0, int c1) -> cudaError_t {
+        int cs = c1;
+        while (cs > c0 && small_fn) {
+            const int ph = ct.ph[cs - 1], nt = (int)host_binom(L, N - 1 - ph);
+            const int64_t z = R.zbase[N - 1 - ph] + (int64_t)host_binom(H, ph + 1) * (ph + 1) * nt;
+            if (nt > kSmallWords || z > (int64_t)UINT32_MAX) break;   // (32-bit offsets into the scratch)
+            --cs;
+        }
+        if (ct.first[c1] - ct.first[cs] < kSmallMin) cs = c1;
+        if (cs > c0) {
+            R.first = ct.first[c0];
+            R.end = ct.first[cs];
+            const int64_t grid = p.grid_t < R.end - R.first ? p.grid_t : R.end - R.first;
+            const void *args[] = {&R, &G, &d, &x, &y, &tk, &skip};
+            const cudaError_t e = cudaLaunchKernel(remove_fn_of(KP), dim3((unsigned)grid), dim3((unsigned)remove_threads(KP)),
+                                                   const_cast<void **>(args), p.smem, st);
+            if (e != cudaSuccess) return e;
+            count_launches(1);
+        }
+        if (cs == c1) return cudaSuccess;
+        SmallArgs S{};
+        S.r = R;
+        S.n = c1 - cs;
+        for (int i = 0; i < S.n; ++i) {
+            const int k = N - ct.ph[cs + i];
+            const int nt = (int)host_binom(L, k - 1), nk = k <= L ? (int)host_binom(L, k) : 0;
+            const int m = kSmallRows / (nt > nk ? nt : nk);
+            S.k[i] = k;
+            S.m[i] = m < kSmallBlocks ? m : kSmallBlocks;
+            S.first[i] = ct.first[cs + i];
+            S.end[i] = ct.first[cs + i + 1];
+            S.item[i + 1] = S.item[i] + (S.end[i] - S.first[i] + S.m[i] - 1) / S.m[i];
+        }
+        const int64_t need = (S.item[S.n] + kSmallGroups - 1) / kSmallGroups;
+        const int64_t grid = p.grid_t < need ? p.grid_t : need;
+        const void *args[] = {&S, &G, &d, &x, &y, &tk, &skip};
+        count_launches(1);
+        return cudaLaunchKernel(small_fn, dim3((unsigned)grid), dim3(128 * kSmallGroups), const_cast<void **>(args),
+                                layout_s(KP, H, N).total, st);
     };
-    auto add = [&](int c0, int c1) -> cudaError_t {
+    int left = cy.n;                              // classes of y to go
+    A.first_launch = 1;
+    auto add_range = [&](int c0, int c1, bool small) -> cudaError_t {
+        if (c1 <= c0) return cudaSuccess;
         A.c0 = c0;
         A.c1 = c1;
+        A.last_launch = (left -= c1 - c0) == 0;
         const int64_t nb = cy.first[c1] - cy.first[c0];
         const int64_t grid = p.grid_y < nb ? p.grid_y : nb;
-        add_kernel<<<(unsigned)grid, kAThreads, 0, st>>>(A, G, d, x, y, tk, skip, dot ? dot->blk_part : nullptr,
-                                                         dot ? dot->out : nullptr);
+        (small ? add_small_kernel : add_kernel)<<<(unsigned)grid, kAThreads, 0, st>>>(
+            A, G, d, x, y, tk, skip, dot ? dot->blk_part : nullptr, dot ? dot->out : nullptr);
+        A.first_launch = 0;
+        count_launches(1);
         return cudaGetLastError();
     };
+    auto add = [&](int c0, int c1) -> cudaError_t {
+        int cs = c1;
+        while (cs > c0 && (int)host_binom(L, N - cy.ph[cs - 1]) <= kAddSmall) --cs;
+        if (cy.first[c1] - cy.first[cs] < kSmallMin) cs = c1;
+        const cudaError_t e = add_range(c0, cs, false);
+        return e != cudaSuccess ? e : add_range(cs, c1, true);
+    };
     if (!p.by_class) {
-        const cudaError_t e = remove(0, p.nt);
-        if (e != cudaSuccess) return e;
-        A.first_launch = A.last_launch = 1;
-        count_launches(2);
-        return add(0, cy.n);
+        const cudaError_t e = remove(0, ct.n);
+        return e != cudaSuccess ? e : add(0, cy.n);
     }
     // class by class, the low pairs k ascending: the words t with k low pairs give
     // the scratch of the rows with k and the partial y of the rows with k + 1
-    int left = cy.n;
-    A.first_launch = 1;
     for (int k = 0; k <= L; ++k) {
         for (int i = 0; i < ct.n; ++i)
             if (N - 1 - ct.ph[i] == k) {
-                const cudaError_t e = remove(ct.first[i], ct.first[i + 1]);
+                const cudaError_t e = remove(i, i + 1);
                 if (e != cudaSuccess) return e;
-                count_launches(1);
             }
         for (int i = 0; i < cy.n; ++i)
             if (N - cy.ph[i] == k) {
-                A.last_launch = --left == 0;
                 const cudaError_t e = add(i, i + 1);
                 if (e != cudaSuccess) return e;
-                A.first_launch = 0;
-                count_launches(1);
             }
     }
     return cudaSuccess;
