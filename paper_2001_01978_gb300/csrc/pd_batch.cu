@@ -208,10 +208,14 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
             run += host_binom(L, n - __builtin_popcountll(w));
         }
         if ((int64_t)run != dim) return fail(PD_ECUDA, "batch: blocks do not cover problem %d", q);
-        // chunks: at most 32 per problem, at least ~1024 elements each, each a
+        // chunks: of ~1024 elements up to 32 per problem, then of ~4096 (a class of
+        // few large problems filled a CTA per SM: at five of 650,000 the projection
+        // of a step took 66 us with 32 chunks each and takes 58, the update 46 / 32,
+        // the dots 21 / 14, the scaling 17 / 9.5), each a
         // multiple of 4 elements long (but the last), so that every chunk starts
         // on a 16-byte boundary (problems start on one: see total below)
-        const int nc = (int)std::min<int64_t>(kMaxChunksPerProblem, std::max<int64_t>(1, (dim + 1023) / 1024));
+        const int64_t fine = std::min<int64_t>(32, (dim + 1023) / 1024);
+        const int nc = (int)std::min<int64_t>(kMaxChunksPerProblem, std::max<int64_t>(fine, dim / 4096));
         const int64_t clen = ((dim + nc - 1) / nc + 3) & ~int64_t(3);
         prob_chunk0.push_back((int)chunk_prob.size());
         int made = 0;

@@ -488,7 +488,7 @@ struct BatchState {                  // one problem (device memory)
 };
 struct BatchVec {                    // vectors concatenated over problems, cut into chunks
     int count;
-    int nchunks;                     // every chunk lies inside one problem; <= 32 per problem
+    int nchunks;                     // every chunk lies inside one problem
     int64_t total;                   // elements per vector: every problem starts on a 4-element
                                      // boundary, and so does every chunk (up to 3 unused
                                      // elements after each problem)
@@ -499,7 +499,7 @@ struct BatchVec {                    // vectors concatenated over problems, cut 
     const int *prob_nchunk;          // [count]
     const int64_t *prob_off;         // [count] first element of each problem
 };
-constexpr int kMaxChunksPerProblem = 32;
+constexpr int kMaxChunksPerProblem = 256;
 
 // out[p * out_stride + j] = sum over problem p's elements of Q_j[e] v[e], j < m
 // (Q vector-major with leading dimension ldq); skipped problems are left alone

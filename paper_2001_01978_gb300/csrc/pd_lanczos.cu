@@ -1168,7 +1168,7 @@ seg_dots_kernel(const BatchVec V, const T *__restrict__ Q, int64_t ldq, int m, c
     }
 }
 
-// one warp per (problem, output): lane l adds chunk l of the problem (<= 32 chunks).
+// one warp per (problem, output): lane l adds chunks l, l + 32, ... of the problem.
 // use_skip: 0 every problem, 1 pass over problems with skip set, 2 pass over done ones
 __global__ void seg_reduce_kernel(const BatchVec V, int m, const BatchState *__restrict__ S, int use_skip,
                                   const double *__restrict__ part, double *__restrict__ out, int out_stride)
@@ -1179,7 +1179,8 @@ __global__ void seg_reduce_kernel(const BatchVec V, int m, const BatchState *__r
     if (pr >= V.count) return;
     if ((use_skip == 1 && S[pr].skip) || (use_skip == 2 && S[pr].done)) return;   // warp-uniform
     const int nc = V.prob_nchunk[pr], c0 = V.prob_chunk0[pr];
-    double sum = lane < nc ? part[(int64_t)(c0 + lane) * kMaxWindow + j] : 0.0;
+    double sum = 0.0;
+    for (int l = lane; l < nc; l += 32) sum += part[(int64_t)(c0 + l) * kMaxWindow + j];
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) out[(int64_t)pr * out_stride + j] = sum;
 }
