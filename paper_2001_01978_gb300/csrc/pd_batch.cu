@@ -103,6 +103,19 @@ struct ClassStream {
     }
 };
 
+// The FP32 products of a class's larger problems by pair removal (variant 2)
+struct FacProblem {
+    int p;                               // number in the class
+    int64_t off;                         // of its vectors
+    FacPlan plan;
+};
+constexpr int64_t kFacScratch = (int64_t)2048 << 18;   // floats: 2 GiB per class
+// Blocks per CTA of the two kernels: a CTA's start (G, tables, tensor memory)
+// costs about one block, and few CTAs leave SMs idle once problems finish.  4 / 8
+// / 16 / 32 blocks of t: 96 problems of 10 to 22 orbits 98.5 / 94.6 / 92.7 / 92.1
+// ms, twelve of them 29.5 / 29.1 / 30.6 / 32.9 ms.
+constexpr int kFacBlocks = 8, kFacRowBlocks = 4;
+
 // One size class: its problems, tables, buffers, stream and graphs.  Members
 // are destroyed in reverse order: the buffers first (after a synchronisation
 // of the class's stream), the stream last.
@@ -120,6 +133,10 @@ struct ClassRun {
     BatchState *S = nullptr;
     double *part = nullptr;
     int *ctl = nullptr;                  // [0] running problems, [1] cycle number, [2] reopened
+    std::vector<FacProblem> fac;
+    std::vector<FacBatch> fac_batch;     // one launch per tile width
+    Tickets *fac_tk = nullptr;           // [fac.size()]
+    int64_t rest_blocks = 0;             // blocks of the other problems, first in the list
     unsigned long long *counter = nullptr;   // [0] next block, [1] finished CTAs of the batched H*x
     char *Q32 = nullptr, *p32 = nullptr, *Q64 = nullptr, *p64 = nullptr;
     double *v64 = nullptr, *w64 = nullptr;
@@ -127,6 +144,106 @@ struct ClassRun {
     int reopened = 0;
     DevBuf buf;                          // destroyed first (declared last): syncs st
 };
+
+// whether the product of problem p goes by pair removal
+bool fac_take(ClassRun &c, int p, int om, int n, int64_t dim, int64_t off, int64_t &scratch)
+{
+    if (!fac_pays_batch(om, n, dim)) return false;
+    FacProblem f{p, off, {}};
+    fac_sizes(om, n, f.plan);
+    if (f.plan.by_class || scratch + f.plan.scratch_len > kFacScratch) return false;
+    scratch += f.plan.scratch_len;
+    c.fac.push_back(f);
+    return true;
+}
+
+// Tables and scratch of the class's products by pair removal.  Without room for
+// them every problem goes through the batched row-by-row kernel.
+int setup_removal(ClassRun &c, const uint64_t *binom, const std::vector<BatchDesc> &desc)
+{
+    if (c.fac.empty()) return PD_OK;
+    // by tile width, the largest problems first
+    std::stable_sort(c.fac.begin(), c.fac.end(), [](const FacProblem &a, const FacProblem &b) {
+        const int ka = fac_columns(a.plan.omega), kb = fac_columns(b.plan.omega);
+        return ka != kb ? ka > kb : a.plan.scratch_len > b.plan.scratch_len;
+    });
+    const int count = (int)c.fac.size();
+    // CTAs: several blocks each, and enough of them when the problems are few
+    const int sms = sm_count();
+    auto share = [&](int64_t blocks, int per_cta, int64_t fill) {
+        return (int)std::min<int64_t>(blocks, std::max<int64_t>((blocks + per_cta - 1) / per_cta, (fill + count - 1) / count));
+    };
+    std::vector<int2> ctas_t, ctas_y;
+    std::vector<int> nt(count), ny(count);
+    std::vector<size_t> first_t, first_y;
+    c.fac_batch.clear();
+    for (int i = 0, in_batch = 0; i < count; ++i, ++in_batch) {
+        const FacPlan &f = c.fac[i].plan;
+        if (c.fac_batch.empty() || c.fac_batch.back().columns != fac_columns(f.omega)) {
+            c.fac_batch.push_back(FacBatch{fac_columns(f.omega), 0, 0, 0, nullptr, nullptr, nullptr});
+            first_t.push_back(ctas_t.size());
+            first_y.push_back(ctas_y.size());
+            in_batch = 0;
+        }
+        nt[i] = share(f.nt, kFacBlocks, 2 * sms);
+        ny[i] = share(f.ny, kFacRowBlocks, 10 * sms);
+        for (int j = 0; j < nt[i]; ++j) ctas_t.push_back(make_int2(in_batch, j));
+        for (int j = 0; j < ny[i]; ++j) ctas_y.push_back(make_int2(in_batch, j));
+        c.fac_batch.back().grid_t += nt[i];
+        c.fac_batch.back().grid_y += ny[i];
+    }
+    size_t bytes = 0;
+    auto place = [&](size_t n) {
+        const size_t at = bytes;
+        bytes = (bytes + n + 255) & ~(size_t)255;
+        return at;
+    };
+    const FacPlan &f0 = c.fac[0].plan;            // 12 low orbits in all of them: one table
+    const size_t item = fac_item_size();
+    const size_t at_tk = place(sizeof(Tickets) * count), at_low = place(sizeof(uint16_t) << f0.L),
+                 at_up = place(sizeof(uint32_t) * (size_t)f0.table), at_z = place(sizeof(float) * fac_zeros()),
+                 at_i = place(item * count), at_ct = place(sizeof(int2) * ctas_t.size()),
+                 at_cy = place(sizeof(int2) * ctas_y.size());
+    std::vector<size_t> at_s(count), at_w(count);
+    for (int i = 0; i < count; ++i) {
+        at_s[i] = place(sizeof(float) * (size_t)c.fac[i].plan.scratch_len);
+        at_w[i] = place(sizeof(uint32_t) * (size_t)(c.fac[i].plan.nt + c.fac[i].plan.ny));
+    }
+    char *mem = nullptr;
+    if (c.buf.alloc(&mem, bytes) != PD_OK) {
+        c.fac.clear();
+        c.fac_batch.clear();
+        return PD_OK;
+    }
+    c.fac_tk = reinterpret_cast<Tickets *>(mem + at_tk);
+    std::vector<char> items(item * count);
+    for (int i = 0; i < count; ++i) {
+        FacPlan &f = c.fac[i].plan;
+        f.low = reinterpret_cast<uint16_t *>(mem + at_low);
+        f.up = reinterpret_cast<uint32_t *>(mem + at_up);
+        f.zeros = reinterpret_cast<float *>(mem + at_z);
+        f.scratch = reinterpret_cast<float *>(mem + at_s[i]);
+        f.twords = reinterpret_cast<uint32_t *>(mem + at_w[i]);
+        f.ywords = f.twords + f.nt;
+        PD_CUDA(fac_build(f, binom, c.st));
+        const BatchDesc &D = desc[c.fac[i].p];
+        fac_item(f, binom, c.P.G32 + D.g_off, c.P.d32 + D.d_off, c.fac[i].off, c.fac[i].p, c.fac_tk + i, nt[i], ny[i],
+                 items.data() + item * i);
+    }
+    PD_CUDA(cudaMemsetAsync(c.fac_tk, 0, sizeof(Tickets) * count, c.st));
+    PD_CUDA(cudaMemcpy(mem + at_i, items.data(), items.size(), cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemcpy(mem + at_ct, ctas_t.data(), sizeof(int2) * ctas_t.size(), cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemcpy(mem + at_cy, ctas_y.data(), sizeof(int2) * ctas_y.size(), cudaMemcpyHostToDevice));
+    for (size_t b = 0, i = 0; b < c.fac_batch.size(); ++b) {
+        FacBatch &B = c.fac_batch[b];
+        B.items = mem + at_i + item * i;
+        B.ctas_t = reinterpret_cast<const int2 *>(mem + at_ct) + first_t[b];
+        B.ctas_y = reinterpret_cast<const int2 *>(mem + at_cy) + first_y[b];
+        for (; i < c.fac.size() && fac_columns(c.fac[i].plan.omega) == B.columns; ++i)
+            B.smem = std::max(B.smem, c.fac[i].plan.smem);
+    }
+    return PD_OK;
+}
 
 // Host tables and device buffers of one class.
 int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, const int *n_pairs,
@@ -137,13 +254,15 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
     std::vector<BatchDesc> desc(count);
     std::vector<uint32_t> blk_prob;
     std::vector<uint64_t> blk_h, blk_base;
+    std::vector<uint32_t> fblk_prob;     // of the problems in c.fac
+    std::vector<uint64_t> fblk_h, fblk_base;
     std::vector<double> G64, d64;
     std::vector<float> G32, d32;
     std::map<int, int> tab_of_L;
     std::vector<uint16_t> lowword_all, rankL_all;
     std::vector<int> chunk_prob, chunk_len, prob_chunk0, prob_nchunk;
     std::vector<int64_t> chunk_start, prob_off;
-    int64_t total = 0;
+    int64_t total = 0, fac_scratch = 0;
     int max_omega = 1, max_L = 1, max_H = 0, max_block = 1, max_hh = 0, max_n = 0;
     for (int p = 0; p < count; ++p) {
         const int q = c.prob[p];
@@ -189,6 +308,8 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
             d64.push_back(dv);
             d32.push_back((float)dv);
         }
+        const bool by_removal = opt.precision == PD_PREC_MIXED && opt.hx_variant == 0 && L == fac_low(om) &&
+                                fac_take(c, p, om, n, dim, total, fac_scratch);
         // blocks of this problem
         const int kmin = std::max(0, n - H), kmax = std::min(n, L);
         std::vector<uint64_t> hw;
@@ -202,9 +323,9 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
         for (uint64_t w : hw) {
             const uint64_t bb = host_block_base(w, L, n);
             if (bb != run) return fail(PD_ECUDA, "batch: internal block index mismatch (problem %d)", q);
-            blk_prob.push_back((uint32_t)p);
-            blk_h.push_back(w);
-            blk_base.push_back(bb);
+            (by_removal ? fblk_prob : blk_prob).push_back((uint32_t)p);
+            (by_removal ? fblk_h : blk_h).push_back(w);
+            (by_removal ? fblk_base : blk_base).push_back(bb);
             run += host_binom(L, n - __builtin_popcountll(w));
         }
         if ((int64_t)run != dim) return fail(PD_ECUDA, "batch: blocks do not cover problem %d", q);
@@ -231,6 +352,11 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
         max_L = std::max(max_L, L);
         max_H = std::max(max_H, H);
     }
+
+    c.rest_blocks = (int64_t)blk_prob.size();
+    blk_prob.insert(blk_prob.end(), fblk_prob.begin(), fblk_prob.end());
+    blk_h.insert(blk_h.end(), fblk_h.begin(), fblk_h.end());
+    blk_base.insert(blk_base.end(), fblk_base.begin(), fblk_base.end());
 
     DevBuf &buf = c.buf;
     buf.st = c.st;
@@ -285,6 +411,7 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
     V.prob_chunk0 = d_pc0; V.prob_nchunk = d_pnc; V.prob_off = d_po;
     c.P = HxProblem{d_G64, d_d64, d_G32, d_d32, d_Gff, d_dff};
     c.total = total;
+    PD_TRY(setup_removal(c, d_binom, desc));
 
     PD_TRY(buf.alloc(&c.part, (size_t)V.nchunks * kMaxWindow));
     PD_TRY(buf.alloc(&c.S, (size_t)count));
@@ -315,10 +442,22 @@ int build_phase_graph(ClassRun &c, int dt, int window, char *Q, char *pvc, doubl
     const int skip_stride = (int)(sizeof(BatchState) / sizeof(int));
     const int sd = (int)(sizeof(BatchState) / sizeof(double));
     auto q = [&](int j) { return (void *)(Q + es * (size_t)j * (size_t)total); };
-    const int hx_grid_ = hx_batch_grid(BB, dt);
     cudaStream_t cs = nullptr;                    // the capturing stream
+    // FP32: the larger problems' products by pair removal, the others' row by row
+    const bool removal = dt == 1 && !c.fac_batch.empty();
+    BatchBlocks rest = BB;
+    if (removal) rest.nblocks = c.rest_blocks;
+    const int rest_grid = rest.nblocks > 0 ? hx_batch_grid(rest, dt) : 0;
+    auto product = [&](int i) -> int {
+        if (removal)
+            for (const FacBatch &b : c.fac_batch)
+                PD_CUDA(fac_batch_launch(b, (const float *)q(i), (float *)pv, cs, skip, skip_stride));
+        if (rest.nblocks > 0)
+            PD_CUDA(hx_batch_launch(rest, c.P, dt, q(i), pv, c.counter, rest_grid, cs, skip, skip_stride));
+        return PD_OK;
+    };
     auto step = [&](int i) -> int {
-        PD_CUDA(hx_batch_launch(BB, c.P, dt, q(i), pv, c.counter, hx_grid_, cs, skip, skip_stride));
+        PD_TRY(product(i));
         PD_CUDA(seg_dots_launch(dt, V, q(i), total, 1, pv, S, part, &S[0].c1, sd, cs));
         PD_CUDA(seg_recur_project_launch(dt, V, Q, total, i, pv, S, part, cs));
         PD_CUDA(seg_update_launch(dt, V, Q, total, i + 1, pv, S, part, cs));
@@ -595,11 +734,17 @@ extern "C" int pairdiag_batch_ground_state(int count, const int *omega, const in
         int ctl[3] = {0, 0, 0};
         cudaError_t e1 = cudaMemcpyAsync(hs.data(), c.S, sizeof(BatchState) * c.count, cudaMemcpyDeviceToHost, c.st);
         if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(ctl, c.ctl, sizeof ctl, cudaMemcpyDeviceToHost, c.st);
+        std::vector<Tickets> tk(c.fac_batch.empty() ? 0 : c.fac.size());
+        if (e1 == cudaSuccess && !tk.empty())
+            e1 = cudaMemcpyAsync(tk.data(), c.fac_tk, sizeof(Tickets) * tk.size(), cudaMemcpyDeviceToHost, c.st);
         if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(c.st);
         if (e1 != cudaSuccess) {
             rc = fail(PD_ECUDA, "batch: result copy failed: %s", cudaGetErrorString(e1));
             break;
         }
+        for (const Tickets &t : tk)
+            if (t.bar.err) rc = fail(PD_ECUDA, "batch: a wait inside a product ran out");
+        if (rc != PD_OK) break;
         // kernels that ran: both graphs' prologues and every executed loop body
         // (ctl[1] counts the cycle heads: one in each prologue, one per body)
         long long ran = 0;

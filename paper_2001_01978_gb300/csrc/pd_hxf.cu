@@ -33,6 +33,7 @@
 #include "pd_internal.h"
 
 #include <climits>
+#include <cstring>
 #include <type_traits>
 #include <utility>
 
@@ -386,12 +387,11 @@ __device__ __forceinline__ void issue_product(const uint32_t tmem, const uint32_
 // shared memory or the constant bank, 8, 10 or 12 low orbits, hops between high
 // orbits in registers): 0.127 to 0.18 ms.
 template <int KP>
-__global__ void __launch_bounds__(Cfg<KP>::kThreads, 2)
-remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G, const float *__restrict__ d,
-              const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip)
+__device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *__restrict__ G, const float *__restrict__ d,
+                                              const float *__restrict__ x, float *__restrict__ y, Tickets *tk,
+                                              const unsigned ctas)
 {
     using C = Cfg<KP>;
-    if (skip && *skip) return;                    // CTA-uniform
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t s_bar[C::kGroups];
     __shared__ uint32_t s_tmem;
@@ -552,7 +552,16 @@ remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G,
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s_tmem), "r"(kTmemCols) : "memory");
-    if (arrive_last(&tk->hx_done) && tid == 0) tk->hx_next = 0ull;
+    if (arrive_last(&tk->hx_done, ctas) && tid == 0) tk->hx_next = 0ull;
+}
+
+template <int KP>
+__global__ void __launch_bounds__(Cfg<KP>::kThreads, 2)
+remove_kernel(const __grid_constant__ RemoveArgs A, const float *__restrict__ G, const float *__restrict__ d,
+              const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip)
+{
+    if (skip && *skip) return;                    // CTA-uniform
+    remove_blocks<KP>(A, G, d, x, y, tk, gridDim.x);
 }
 
 // ---- pair removal, small blocks -------------------------------------------------
@@ -838,13 +847,13 @@ __device__ __noinline__ float row_slow(const AddArgs &A, const float *__restrict
 
 // the last CTA sums the partial dot products
 __device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float> &dot, Tickets *tk, double *part,
-                                           double *dot_out, double *sred)
+                                           double *dot_out, double *sred, const unsigned ctas)
 {
     if (part) {
         const double v = block_reduce(dot, sred);
         if (threadIdx.x == 0) part[blockIdx.x] = v;
     }
-    if (!arrive_last(&tk->hx_done)) return;
+    if (!arrive_last(&tk->hx_done, ctas)) return;
     if (A.last_launch && threadIdx.x == 0) tk->pad = 0ull;
     if (!part) return;
     double s = 0.0;
@@ -858,12 +867,10 @@ __device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float>
 // so that blocks of very different sizes balance.  Omega=24 (65 MB of scratch,
 // mostly in L2): 26 us alone with a cold cache, against 32 us with 256 threads
 // and 40 us with two rows per thread.
-__global__ void __launch_bounds__(kAThreads, kACtas)
-add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const float *__restrict__ d,
-           const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip, double *part,
-           double *dot_out)
+__device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
+                                           const float *__restrict__ x, float *__restrict__ y, Tickets *tk, double *part,
+                                           double *dot_out, const int cta, const int ctas)
 {
-    if (skip && *skip) return;                    // CTA-uniform
     __shared__ double sred[kAThreads / 32];
     __shared__ uint32_t bin[kMaxHigh * (kMaxHigh + kLT + 1)];   // C(L + p, m), m < N + 2, N < omega
     const int lane = threadIdx.x & 31;
@@ -874,15 +881,15 @@ add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const
     __syncthreads();
     DotAcc<float> dot;
     int c = A.c0;
-    int64_t b = A.first[A.c0] + blockIdx.x;
+    int64_t b = A.first[A.c0] + cta;
     const int64_t end = A.first[A.c1];
     uint32_t hn = b < end ? __ldg(A.words + b) : 0u;
-    for (; b < end; b += gridDim.x) {
+    for (; b < end; b += ctas) {
         while (b >= A.first[c + 1]) ++c;
         const int ph = A.ph[c], k = A.N - ph;
         const int lo_k = A.lo_off[k], nk = A.lo_off[k + 1] - lo_k;
         const uint32_t h = hn;
-        if (b + gridDim.x < end) hn = __ldg(A.words + b + gridDim.x);
+        if (b + ctas < end) hn = __ldg(A.words + b + ctas);
         const bool occ = h >> lane & 1u;
         uint32_t base = occ ? bin[lane * NB + k + 1 + __popc(h & ((1u << lane) - 1u))] : 0u;
 #pragma unroll
@@ -931,7 +938,16 @@ add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const
             }
         }
     }
-    finish_add(A, dot, tk, part, dot_out, sred);
+    finish_add(A, dot, tk, part, dot_out, sred, ctas);
+}
+
+__global__ void __launch_bounds__(kAThreads, kACtas)
+add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const float *__restrict__ d,
+           const float *__restrict__ x, float *__restrict__ y, Tickets *tk, const int *__restrict__ skip, double *part,
+           double *dot_out)
+{
+    if (skip && *skip) return;                    // CTA-uniform
+    add_blocks(A, G, d, x, y, tk, part, dot_out, blockIdx.x, gridDim.x);
 }
 
 // The rows of classes with small blocks (at most kAddSmall rows): one thread per
@@ -981,7 +997,63 @@ add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G,
             if (part) dot.add(xr, acc);
         }
     }
-    finish_add(A, dot, tk, part, dot_out, sred);
+    finish_add(A, dot, tk, part, dot_out, sred, gridDim.x);
+}
+
+// ---- many problems in one launch ------------------------------------------------
+// Each CTA belongs to one problem; it takes blocks from that problem's ticket.
+// Bound as the kernels of one problem are, and at the same rate: five problems of
+// 650,000 states 107 us for the removal and 29 us for the addition.  (One pair of
+// launches per problem, in one to eight parallel branches of the solver's graph,
+// was no faster than the row-by-row kernel over all of them: a launch of 250
+// blocks is mostly the start of its CTAs.)
+struct FacItem {
+    RemoveArgs r;
+    AddArgs a;
+    const float *G, *d;
+    Tickets *tk;
+    int64_t off;                         // of its vectors
+    int p;                               // number of its skip flag
+    int ctas_t, ctas_y;
+};
+static_assert(sizeof(FacItem) % 4 == 0, "copied in words");
+
+__device__ __forceinline__ void copy_item(FacItem &to, const FacItem *from)
+{
+    for (int i = threadIdx.x; i < (int)(sizeof(FacItem) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(&to)[i] = __ldg(reinterpret_cast<const uint32_t *>(from) + i);
+    __syncthreads();
+}
+
+template <int KP>
+__global__ void __launch_bounds__(Cfg<KP>::kThreads, 2)
+remove_batch_kernel(const FacItem *__restrict__ items, const int2 *__restrict__ ctas, const float *x, float *y,
+                    const int *__restrict__ skip, int skip_stride)
+{
+    __shared__ FacItem it;
+    const int2 c = ctas[blockIdx.x];
+    if (skip[items[c.x].p * skip_stride]) return;   // CTA-uniform
+    copy_item(it, items + c.x);
+    remove_blocks<KP>(it.r, it.G, it.d, x + it.off, y + it.off, it.tk, it.ctas_t);
+}
+
+__global__ void __launch_bounds__(kAThreads, kACtas)
+add_batch_kernel(const FacItem *__restrict__ items, const int2 *__restrict__ ctas, const float *x, float *y,
+                 const int *__restrict__ skip, int skip_stride)
+{
+    __shared__ FacItem it;
+    const int2 c = ctas[blockIdx.x];
+    if (skip[items[c.x].p * skip_stride]) return;   // CTA-uniform
+    copy_item(it, items + c.x);
+    add_blocks(it.a, it.G, it.d, x + it.off, y + it.off, it.tk, nullptr, nullptr, c.y, it.ctas_y);
+}
+
+const void *remove_batch_fn_of(int KP)
+{
+    return KP == 16   ? (const void *)remove_batch_kernel<16>
+           : KP == 24 ? (const void *)remove_batch_kernel<24>
+           : KP == 32 ? (const void *)remove_batch_kernel<32>
+                      : (const void *)remove_batch_kernel<40>;
 }
 
 template <int KP>
@@ -1025,6 +1097,17 @@ bool fac_fits(int omega, int n, int64_t dim)
 bool fac_pays(int omega, int n, int64_t dim)
 {
     return dim >= 60000 && 3 * n <= 2 * omega + 2 && fac_fits(omega, n, dim);
+}
+
+// The same line for many problems in one launch, which has its launches and the
+// start of its CTAs once for all.  Five problems of 650,000 states, row by row /
+// by removal: 224 / 136 us; fourteen of 200,000 to 490,000: 286 / 199 us.  A solve
+// of 96 problems of 10 to 22 orbits with the line at 60000 / 15000 / 3000 states:
+// 95.5 / 94.5 / 94.7 ms; of twelve of 18 to 22 orbits 86.7 / 84.9 / 84.9 ms; of 96
+// of 10 to 14 orbits 11.3 / 11.3 / 12.1 ms.
+bool fac_pays_batch(int omega, int n, int64_t dim)
+{
+    return dim >= 15000 && omega > kLT && 3 * n <= 2 * omega + 2 && fac_fits(omega, n, dim);
 }
 
 // classes of words with `pairs` pairs in all, the largest blocks first
@@ -1102,15 +1185,13 @@ cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st)
 int64_t fac_partials(const FacPlan &p) { return p.grid_y; }
 
 
-cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, const float *x, float *y,
-                       Tickets *tk, cudaStream_t st, const int *skip, const HxDot *dot)
+static void fill_args(const FacPlan &p, const uint64_t *binom, WordClasses &ct, WordClasses &cy, RemoveArgs &R, AddArgs &A)
 {
-    const int L = p.L, H = p.omega - L, N = p.n, KP = padded(p.omega);
-    WordClasses ct, cy;
+    const int L = p.L, H = p.omega - L, N = p.n;
     word_classes(L, H, N - 1, ct);
     word_classes(L, H, N, cy);
-    RemoveArgs R{};
-    AddArgs A{};
+    R = RemoveArgs{};
+    A = AddArgs{};
     R.omega = A.omega = p.omega;
     R.N = A.N = N;
     R.L = A.L = L;
@@ -1136,6 +1217,16 @@ cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, 
         R.zbase[k] = A.zbase[k] = z;
         z += (int64_t)host_binom(H, cy.ph[i]) * cy.ph[i] * (int64_t)host_binom(L, k);
     }
+}
+
+cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, const float *x, float *y,
+                       Tickets *tk, cudaStream_t st, const int *skip, const HxDot *dot)
+{
+    const int L = p.L, H = p.omega - L, N = p.n, KP = padded(p.omega);
+    WordClasses ct, cy;
+    RemoveArgs R;
+    AddArgs A;
+    fill_args(p, binom, ct, cy, R, A);
     const void *small_fn = remove_small_fn_of(KP);
     // classes [c0, c1) of t: those of small blocks, at the end, on their own if
     // they are many
@@ -1220,6 +1311,45 @@ cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, 
             }
     }
     return cudaSuccess;
+}
+
+size_t fac_item_size() { return sizeof(FacItem); }
+int fac_columns(int omega) { return padded(omega); }
+
+void fac_item(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, int64_t off, int number, Tickets *tk,
+              int ctas_t, int ctas_y, void *out)
+{
+    FacItem it{};
+    WordClasses ct, cy;
+    fill_args(p, binom, ct, cy, it.r, it.a);
+    it.r.first = 0;
+    it.r.end = p.nt;
+    it.a.c0 = 0;
+    it.a.c1 = cy.n;
+    it.a.first_launch = it.a.last_launch = 1;
+    it.G = G;
+    it.d = d;
+    it.tk = tk;
+    it.off = off;
+    it.p = number;
+    it.ctas_t = ctas_t;
+    it.ctas_y = ctas_y;
+    std::memcpy(out, &it, sizeof it);
+}
+
+cudaError_t fac_batch_launch(const FacBatch &b, const float *x, float *y, cudaStream_t st, const int *skip, int skip_stride)
+{
+    const FacItem *items = static_cast<const FacItem *>(b.items);
+    const void *fn = remove_batch_fn_of(b.columns);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e != cudaSuccess) return e;
+    const void *args[] = {&items, &b.ctas_t, &x, &y, &skip, &skip_stride};
+    e = cudaLaunchKernel(fn, dim3((unsigned)b.grid_t), dim3((unsigned)remove_threads(b.columns)), const_cast<void **>(args),
+                         b.smem, st);
+    if (e != cudaSuccess) return e;
+    add_batch_kernel<<<(unsigned)b.grid_y, kAThreads, 0, st>>>(items, b.ctas_y, x, y, skip, skip_stride);
+    count_launches(2);
+    return cudaGetLastError();
 }
 
 }  // namespace pd

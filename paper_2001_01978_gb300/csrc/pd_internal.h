@@ -270,14 +270,14 @@ __device__ __forceinline__ double warp_reduce(const DotAcc<float> &a)
 // partial sums.  Returns true in the one CTA that arrives last; by then the
 // partial sums of all CTAs are visible to it (read them with __ldcg).  That CTA
 // returns the ticket to zero.  No CTA waits for another.
-__device__ __forceinline__ bool arrive_last(unsigned long long *ticket)
+__device__ __forceinline__ bool arrive_last(unsigned long long *ticket, unsigned ctas)
 {
     __shared__ int s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();                                       // release this CTA's partial sums
         const unsigned long long t = atomicAdd(ticket, 1ull);
-        const int last = (t == (unsigned long long)gridDim.x - 1ull);
+        const int last = (t == (unsigned long long)ctas - 1ull);
         if (last) {
             *ticket = 0ull;
             __threadfence();                                   // acquire the others'
@@ -287,6 +287,7 @@ __device__ __forceinline__ bool arrive_last(unsigned long long *ticket)
     __syncthreads();
     return s_last != 0;
 }
+__device__ __forceinline__ bool arrive_last(unsigned long long *ticket) { return arrive_last(ticket, gridDim.x); }
 
 // out[j] = sum_b part[b * kMaxWindow + j] for j < m: warp w takes outputs w,
 // w + warps, ...; each lane a fixed strided subset of b, then a fixed xor tree,
@@ -361,6 +362,24 @@ cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st);
 int64_t fac_partials(const FacPlan &p);
 cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, const float *x, float *y,
                        Tickets *tk, cudaStream_t st, const int *skip, const HxDot *dot);
+// Many problems in one launch each of the two kernels: fac_item writes the
+// description of one problem (fac_item_size() bytes, for the device), whose
+// vectors start at x + off, y + off and whose skip flag is skip[number *
+// skip_stride]; ctas maps a CTA to (problem, CTA within the problem).  All
+// problems of a launch have the same fac_columns, and none goes class by class.
+struct FacBatch {
+    int columns;
+    int grid_t, grid_y;
+    size_t smem;
+    const void *items;
+    const int2 *ctas_t, *ctas_y;
+};
+bool fac_pays_batch(int omega, int n, int64_t dim);
+int fac_columns(int omega);
+size_t fac_item_size();
+void fac_item(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, int64_t off, int number, Tickets *tk,
+              int ctas_t, int ctas_y, void *out);
+cudaError_t fac_batch_launch(const FacBatch &b, const float *x, float *y, cudaStream_t st, const int *skip, int skip_stride);
 // Truncation (Sec. 3.5).  The bin of a state is floor((D - lo) / (hi - lo) * bins)
 // in FP64, clamped to bins - 1, with D its diagonal element summed in ascending
 // orbit order; lo/hi the extreme diagonal elements.
