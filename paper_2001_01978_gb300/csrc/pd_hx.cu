@@ -882,7 +882,11 @@ hx3_kernel(const Blocks B, const A *__restrict__ Gg, const A *__restrict__ dg, c
 }
 
 // x of a truncated space into the full-space vector xf, which holds zeros at the
-// dropped states (they are never written)
+// dropped states (they are never written).  The kept rows then gather from xf as
+// the full product does, without a look-up of every target in the index map, and
+// threads go to kept rows only: 250,000 of the 2.7e6 states of Omega=24, FP32,
+// 163 us with the map (hx_kernel<..., true>) and 63 us, this copy included; bound
+// by instruction issue, as the full product.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 kept_scatter_kernel(const uint64_t *__restrict__ full, int64_t n, const T *__restrict__ x, T *__restrict__ xf,
@@ -945,7 +949,8 @@ constexpr size_t kSmemLimit = 200 * 1024;
 
 // Variant 3 (lean loops; also where variant 2, the FP32 product of pd_hxf.cu,
 // does not serve the call), 4 (deep gather groups) or 5 (lean loops, 5 CTAs per
-// SM) on request, when the shared memory fits (full space only)
+// SM) on request, when the shared memory fits; on a truncated space all of them
+// are the lean loops over the kept rows
 template <typename T, typename A>
 bool use_v3(const Blocks &B)
 {

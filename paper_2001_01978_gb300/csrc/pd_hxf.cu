@@ -28,7 +28,10 @@
 // [orbit][row], one writer each); the block's partial y is written once.
 // Results for a high orbit q belong to block h + q at the same low word: they go
 // to a scratch vector, ordered by (block of y, ordinal of q, row), where
-// add_kernel streams them: y(h, l) += sum_a scratch(h, a, l).  No two threads
+// add_kernel streams them: y(h, l) += sum_a scratch(h, a, l).  The scratch is
+// written and read as data used once, so that L2 keeps x and the caller's
+// vectors (plain stores / streaming stores: C(24,12) 96.2 / 94.7 us and 10.09 /
+// 9.96 ms for a solve around it, C(28,14) 1.71 / 1.61 ms, C(30,15) 6.89 / 6.53 ms).  No two threads
 // add to the same element, so the sums have a fixed order.
 #include "pd_internal.h"
 
@@ -538,7 +541,7 @@ __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *
                                 const uint32_t off = (p & 1) ? slot[p / 2] >> 16 : slot[p / 2] & 0xffffu;
                                 *reinterpret_cast<float *>(smem + p * kStride * 4 + off) = __uint_as_float(z[t]);
                             } else if (to >> (p - kLT) & 1u) {
-                                bs.ze[p - kLT][r] = __uint_as_float(z[t]);
+                                __stcs(bs.ze[p - kLT] + r, __uint_as_float(z[t]));
                             }
                         }
                     });
@@ -778,7 +781,7 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
                         *reinterpret_cast<float *>(reinterpret_cast<char *>(part) + p * kSmallStride * 4 + off) =
                             __uint_as_float(z[u]);
                     } else if (to >> (p - kLT) & 1u) {
-                        A.scratch[(uint32_t)(ze[i * H + p - kLT] + t)] = __uint_as_float(z[u]);
+                        __stcs(A.scratch + (uint32_t)(ze[i * H + p - kLT] + t), __uint_as_float(z[u]));
                     }
                 }
             });
@@ -1094,8 +1097,8 @@ bool fac_fits(int omega, int n, int64_t dim)
 
 // Where variant 2 is the faster one and no less exact (variant 3 / variant 2,
 // FP32, back to back): C(17,6) 15.7 / 18.5 us, C(18,9) = 48620 18.7 / 20.6 us,
-// C(20,10) = 184756 31 / 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 7.1 ms,
-// C(34,9) 12.8 / 1.8 ms.  Far above half filling there are more words t than
+// C(20,10) = 184756 31 / 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 6.5 ms,
+// C(34,9) 12.8 / 1.7 ms.  Far above half filling there are more words t than
 // states and their rows are longer: C(24,16) 94 / 64 us, C(24,18) 48 / 41 us,
 // C(28,22) 141 / 211 us, and C(20,17) loses accuracy (2.2e-7 / 2.6e-7).
 bool fac_pays(int omega, int n, int64_t dim)
