@@ -157,7 +157,7 @@ class ClockSampler:
 
 def hx_source_hash() -> str:
     h = hashlib.sha256()
-    for f in ("pd_hx.cu", "pd_internal.h"):
+    for f in ("pd_hx.cu", "pd_hxf.cu", "pd_internal.h"):
         h.update((ROOT / "paper_2001_01978_gb300" / "csrc" / f).read_bytes())
     return h.hexdigest()[:16]
 

@@ -93,9 +93,11 @@ typedef struct {
                                CTAs per SM (fewer registers, more warps).  Variant 2 falls
                                back to 3 where it does not apply (more than 40 orbits, 2^32
                                states or more, no or only full orbits, no room for its
-                               scratch), 2-5 fall back to 1
-                               when their shared memory does not fit.  A truncated handle (pairdiag_truncate) runs
-                               variant 1 */
+                               scratch), 2-5 fall back to 1 when their shared memory does not
+                               fit.  A truncated handle (pairdiag_truncate) computes its kept
+                               rows by variant 3 on x spread over the full space (2-5; 12 bytes
+                               per state of the full space), by variant 1 through the index
+                               map where 1 is asked for or that memory is missing */
 } pairdiag_options;
 
 typedef struct {

@@ -49,8 +49,8 @@ constexpr int kSpare = kRows;            // slot of hops that do not exist (read
 constexpr int kStride = 928;             // floats per orbit of the partial results
 // Scratch (floats): all rows at once up to 2 GiB, else class by class (the rows
 // with k low pairs, k ascending), which bounds it at the largest class: 1.2 GB
-// instead of 5.2 GB at Omega=30, 5 GB instead of 22 GB at Omega=32.  Measured
-// at once / by class: Omega=24 0.096 / 0.28 ms (26 short launches), Omega=28
+// instead of 5.2 GB at Omega=30, 5 GB instead of 22 GB at Omega=32.  Measured,
+// when the line was drawn, at once / by class: Omega=24 0.096 / 0.28 ms (26 short launches), Omega=28
 // 1.79 / 1.97 ms, Omega=30 7.45 / 7.36 ms.
 constexpr int64_t kScratchAll = (int64_t)2048 << 18;
 constexpr int kTile = 128;               // words t per tile: the lanes of tensor memory
@@ -383,9 +383,9 @@ __device__ __forceinline__ void issue_product(const uint32_t tmem, const uint32_
 // share an SM's tensor memory, so that one group's gathers overlap another's
 // product; the high orbits of the next tile are loaded while the product runs;
 // the ninth (thirteenth) warp prepares the next block's pointers.  Omega=24:
-// 78 us alone with a cold cache for 3.9e8 hops (48e6 warp instructions, 0.55 of
+// 75 us alone with a cold cache for 3.9e8 hops (46e6 warp instructions, 0.55 of
 // the issue slots), where the row-by-row kernel (pd_hx.cu, variant 3) took
-// 215 us; both kernels together 0.096 ms.  Measured and not kept: FP32
+// 215 us; both kernels together 0.0945 ms.  Measured and not kept: FP32
 // multiply-adds instead of the tensor cores (packed pairs, coefficients from
 // shared memory or the constant bank, 8, 10 or 12 low orbits, hops between high
 // orbits in registers): 0.127 to 0.18 ms.
@@ -872,7 +872,7 @@ __device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float>
 // y(h, l) += sum over the pairs a of h of scratch(h, a, l); fused x^T y.  Bound
 // by the latency of streaming reads: 16 loads per thread in flight, small CTAs
 // so that blocks of very different sizes balance.  Omega=24 (65 MB of scratch,
-// mostly in L2): 26 us alone with a cold cache, against 32 us with 256 threads
+// mostly in L2): 25 us alone with a cold cache, against 32 us with 256 threads
 // and 40 us with two rows per thread.
 __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
                                            const float *__restrict__ x, float *__restrict__ y, Tickets *tk, double *part,
