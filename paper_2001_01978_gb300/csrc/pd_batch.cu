@@ -217,6 +217,9 @@ int setup_removal(ClassRun &c, const uint64_t *binom, const std::vector<BatchDes
     }
     c.fac_tk = reinterpret_cast<Tickets *>(mem + at_tk);
     std::vector<char> items(item * count);
+    // the uploads of binom, G and d ran on the default stream, whose order c.st
+    // does not follow
+    PD_CUDA(cudaStreamSynchronize(nullptr));
     for (int i = 0; i < count; ++i) {
         FacPlan &f = c.fac[i].plan;
         f.low = reinterpret_cast<uint16_t *>(mem + at_low);
@@ -231,9 +234,9 @@ int setup_removal(ClassRun &c, const uint64_t *binom, const std::vector<BatchDes
                  items.data() + item * i);
     }
     PD_CUDA(cudaMemsetAsync(c.fac_tk, 0, sizeof(Tickets) * count, c.st));
-    PD_CUDA(cudaMemcpy(mem + at_i, items.data(), items.size(), cudaMemcpyHostToDevice));
-    PD_CUDA(cudaMemcpy(mem + at_ct, ctas_t.data(), sizeof(int2) * ctas_t.size(), cudaMemcpyHostToDevice));
-    PD_CUDA(cudaMemcpy(mem + at_cy, ctas_y.data(), sizeof(int2) * ctas_y.size(), cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemcpyAsync(mem + at_i, items.data(), items.size(), cudaMemcpyHostToDevice, c.st));
+    PD_CUDA(cudaMemcpyAsync(mem + at_ct, ctas_t.data(), sizeof(int2) * ctas_t.size(), cudaMemcpyHostToDevice, c.st));
+    PD_CUDA(cudaMemcpyAsync(mem + at_cy, ctas_y.data(), sizeof(int2) * ctas_y.size(), cudaMemcpyHostToDevice, c.st));
     for (size_t b = 0, i = 0; b < c.fac_batch.size(); ++b) {
         FacBatch &B = c.fac_batch[b];
         B.items = mem + at_i + item * i;
@@ -743,7 +746,7 @@ extern "C" int pairdiag_batch_ground_state(int count, const int *omega, const in
             break;
         }
         for (const Tickets &t : tk)
-            if (t.bar.err) rc = fail(PD_ECUDA, "batch: a wait inside a product ran out");
+            if (t.bar.err) rc = fail(PD_ETIMEOUT, "batch: a wait inside a product ran out");
         if (rc != PD_OK) break;
         // kernels that ran: both graphs' prologues and every executed loop body
         // (ctl[1] counts the cycle heads: one in each prologue, one per body)
