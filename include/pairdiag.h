@@ -381,7 +381,12 @@ typedef struct {
  *                    whose refined residual misses tol continue in FP64 cycles from
  *                    the refined vector
  *   opt            : nullable; window, max_restarts, precision, seed, low_bits and
- *                    mixed_floor are used; start PD_START_RANDOM or PD_START_MLP, mode 0
+ *                    mixed_floor are used; start PD_START_RANDOM or PD_START_MLP, mode 0.
+ *                    hx_variant 1: the staged kernel; 2: FP32 products by pair removal
+ *                    on every problem of more than 12 orbits that they serve (block
+ *                    split 12, scratch up to 2 GiB per class), the others and FP64 by
+ *                    variant 3; 0: likewise from 15000 states, below two thirds filling;
+ *                    3-5: variant 3
  *   mlp            : the warm-start network for PD_START_MLP (else nullable); one
  *                    network pass serves the orbits of all problems
  *   e0, status     : host [count] outputs (PD_OK or PD_ENOCONV per problem)

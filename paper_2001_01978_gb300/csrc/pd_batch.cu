@@ -145,10 +145,11 @@ struct ClassRun {
     DevBuf buf;                          // destroyed first (declared last): syncs st
 };
 
-// whether the product of problem p goes by pair removal
-bool fac_take(ClassRun &c, int p, int om, int n, int64_t dim, int64_t off, int64_t &scratch)
+// whether the product of problem p goes by pair removal: where it is the faster
+// one, or (variant 2 asked for) wherever it serves the problem
+bool fac_take(ClassRun &c, int p, int om, int n, int64_t dim, int64_t off, bool asked, int64_t &scratch)
 {
-    if (!fac_pays_batch(om, n, dim)) return false;
+    if (asked ? om <= fac_low(om) || !fac_fits(om, n, dim) : !fac_pays_batch(om, n, dim)) return false;
     FacProblem f{p, off, {}};
     fac_sizes(om, n, f.plan);
     if (f.plan.by_class || scratch + f.plan.scratch_len > kFacScratch) return false;
@@ -311,8 +312,8 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
             d64.push_back(dv);
             d32.push_back((float)dv);
         }
-        const bool by_removal = opt.precision == PD_PREC_MIXED && opt.hx_variant == 0 && L == fac_low(om) &&
-                                fac_take(c, p, om, n, dim, total, fac_scratch);
+        const bool by_removal = opt.precision == PD_PREC_MIXED && (opt.hx_variant == 0 || opt.hx_variant == 2) &&
+                                L == fac_low(om) && fac_take(c, p, om, n, dim, total, opt.hx_variant == 2, fac_scratch);
         // blocks of this problem
         const int kmin = std::max(0, n - H), kmax = std::min(n, L);
         std::vector<uint64_t> hw;
@@ -406,8 +407,9 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
     BB.lowword_all = d_lw; BB.rankL_all = d_rk; BB.binom = d_binom;
     BB.max_omega = max_omega; BB.max_L = max_L; BB.max_H = max_H; BB.max_block = max_block; BB.max_hh = max_hh;
     BB.max_n = max_n;
-    // the batched H*x: direct gathers (variant 3) unless the caller asks for the staged form
-    BB.variant = (opt.hx_variant == 1 || opt.hx_variant == 2) ? 1 : 3;
+    // the batched H*x of the other problems and of FP64: direct gathers (variant 3)
+    // unless the caller asks for the staged form
+    BB.variant = opt.hx_variant == 1 ? 1 : 3;
     BatchVec &V = c.V;
     V.count = count; V.nchunks = (int)chunk_prob.size(); V.total = total;
     V.chunk_prob = d_cp; V.chunk_start = d_cs; V.chunk_len = d_cl;
