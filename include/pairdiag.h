@@ -185,7 +185,9 @@ int pairdiag_rank_dev(const pairdiag_t *h, const uint64_t *states_dev, int64_t c
  *     runs on the FP32 pipes.  The mixed form's FP64 Rayleigh refinement takes
  *     this product.  PD_ENOTSUP on a truncated handle or where its shared
  *     memory does not fit.
- * x_dev and y_dev must not overlap.  Asynchronous.
+ * x_dev and y_dev must not overlap.  Asynchronous.  A mixed handle's FP32
+ * product by pair removal waits for the tensor cores; should such a wait run
+ * out (pairdiag_set_wait_limit), every row of y written from then on is NaN.
  */
 int pairdiag_hx_dev(pairdiag_t *h, int precision, const void *x_dev, void *y_dev);
 
@@ -521,6 +523,14 @@ int pairdiag_get_profile(pairdiag_t *h, int precision, int64_t *hx_launches, dou
  * The results agree to rounding.  Applies from the next solve.
  */
 int pairdiag_set_step_fusion(pairdiag_t *h, int on);
+
+/*
+ * Bound of each wait inside the handle's FP32 product by pair removal, in polls
+ * of up to a millisecond (default 2^12; at most 2^20).  When one runs out, a
+ * solve returns PD_ETIMEOUT and a single product leaves NaN in y; a solve after
+ * that starts afresh.  0: the first wait gives up at once (a test of that path).
+ */
+int pairdiag_set_wait_limit(pairdiag_t *h, int polls);
 
 /*
  * Fused multiply-add throughput of the current device in the arithmetic of

@@ -14,6 +14,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -467,12 +468,15 @@ int lock_project(pairdiag *h, int dtype, void *v, const int *skip)
     return PD_OK;
 }
 
-// err: the barrier error flag, copied back with the cycle's scalars.
-// PD_ETIMEOUT (and the barrier state reset) when a grid-wide wait of a fused
-// step gave up.
-int check_barrier(pairdiag *h, int err)
+// err: the flags of the waits, copied back with the cycle's scalars.  PD_ETIMEOUT
+// when a product's wait gave up, or (and the barrier state reset) a grid-wide
+// wait of a fused step.
+static_assert(offsetof(Tickets, expired) == offsetof(Tickets, bar) + offsetof(GridBar, err) + sizeof(int),
+              "both flags in one copy");
+int check_waits(pairdiag *h, const int (&err)[2])
 {
-    if (!err) return PD_OK;
+    if (err[1]) return fail(PD_ETIMEOUT, "a wait inside an FP32 product (pair removal) ran out");
+    if (!err[0]) return PD_OK;
     PD_CUDA(cudaMemsetAsync(&h->d_tk->bar, 0, sizeof(GridBar), h->st));
     PD_CUDA(cudaStreamSynchronize(h->st));
     return fail(PD_ETIMEOUT, "a grid-wide barrier of the fused Lanczos step timed out");
@@ -564,7 +568,7 @@ int run_cycles(pairdiag *h, int dtype, double tol, int max_cycles, CycleStats &c
     // One synchronisation per cycle: the end of a cycle (its Ritz values) and
     // step 0 of the next (the restart test) are read back together.
     double ab[2] = {0.0, 0.0}, th[2] = {0.0, 0.0};
-    int used = 0, berr = 0;
+    int used = 0, werr[2] = {0, 0};
     auto begin_cycle = [&]() -> int {
         if (h->n_locked) {                        // restart vector orthogonal to the locked states
             PD_TRY(lock_project(h, dtype, Q, nullptr));
@@ -575,7 +579,7 @@ int run_cycles(pairdiag *h, int dtype, double tol, int max_cycles, CycleStats &c
         PD_TRY(lanczos_step(h, dtype, 0, m));
         PD_CUDA(cudaMemcpyAsync(&ab[0], &S->alpha[0], sizeof(double), cudaMemcpyDeviceToHost, st));
         PD_CUDA(cudaMemcpyAsync(&ab[1], &S->beta[0], sizeof(double), cudaMemcpyDeviceToHost, st));
-        PD_CUDA(cudaMemcpyAsync(&berr, &h->d_tk->bar.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PD_CUDA(cudaMemcpyAsync(werr, &h->d_tk->bar.err, sizeof werr, cudaMemcpyDeviceToHost, st));
         return PD_OK;
     };
     auto end_cycle = [&](int cycle) -> int {     // after the synchronisation
@@ -590,7 +594,7 @@ int run_cycles(pairdiag *h, int dtype, double tol, int max_cycles, CycleStats &c
     bool pending = false;                         // the previous cycle's end is still to be read
     for (int cycle = 0; cycle <= max_cycles; ++cycle) {
         PD_CUDA(cudaStreamSynchronize(st));
-        PD_TRY(check_barrier(h, berr));
+        PD_TRY(check_waits(h, werr));
         if (pending) {
             PD_TRY(end_cycle(cycle - 1));
             ++cs.restarts;
@@ -630,10 +634,10 @@ int run_cycles(pairdiag *h, int dtype, double tol, int max_cycles, CycleStats &c
         PD_CUDA(scale_launch(dtype, Q, Q, dim, &S->norm2, 1, st));
         PD_CUDA(cudaMemcpyAsync(th, S->theta, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
         PD_CUDA(cudaMemcpyAsync(&used, &S->used, sizeof(int), cudaMemcpyDeviceToHost, st));
-        PD_CUDA(cudaMemcpyAsync(&berr, &h->d_tk->bar.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PD_CUDA(cudaMemcpyAsync(werr, &h->d_tk->bar.err, sizeof werr, cudaMemcpyDeviceToHost, st));
         if (h->opt.mode == 1 || cycle == max_cycles) {   // no next cycle
             PD_CUDA(cudaStreamSynchronize(st));
-            PD_TRY(check_barrier(h, berr));
+            PD_TRY(check_waits(h, werr));
             PD_TRY(end_cycle(cycle));
             if (h->opt.mode == 1) cs.converged = true;
             return PD_OK;
@@ -731,6 +735,9 @@ int ground_state_impl(pairdiag *h, double tol, double *e0, double *vec_dev, bool
     PD_CUDA(cudaSetDevice(h->device));
     const int64_t dim = h->dim;
     const int win = std::min<int64_t>(std::max(1, h->opt.window), std::min<int64_t>(dim, kMaxWindow));
+    // (an earlier product whose wait gave up has left its rows NaN; it says
+    // nothing about this solve)
+    if (h->fac.on) PD_CUDA(cudaMemsetAsync(&h->d_tk->expired, 0, sizeof(int), h->st));
     CycleStats cs;
     int status = PD_OK;
     int fp32_iters = 0;
@@ -967,6 +974,14 @@ int pairdiag_set_step_fusion(pairdiag_t *h, int on)
 {
     if (!h) return fail(PD_EINVAL, "null handle");
     h->step_fusion = on != 0;
+    return PD_OK;
+}
+
+int pairdiag_set_wait_limit(pairdiag_t *h, int polls)
+{
+    if (!h) return fail(PD_EINVAL, "null handle");
+    if (polls < 0 || polls > 1 << 20) return fail(PD_EINVAL, "polls outside 0..2^20");
+    h->fac.polls = polls;
     return PD_OK;
 }
 

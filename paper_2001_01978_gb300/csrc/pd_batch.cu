@@ -748,7 +748,7 @@ extern "C" int pairdiag_batch_ground_state(int count, const int *omega, const in
             break;
         }
         for (const Tickets &t : tk)
-            if (t.bar.err) rc = fail(PD_ETIMEOUT, "batch: a wait inside a product ran out");
+            if (t.expired) rc = fail(PD_ETIMEOUT, "batch: a wait inside a product ran out");
         if (rc != PD_OK) break;
         // kernels that ran: both graphs' prologues and every executed loop body
         // (ctl[1] counts the cycle heads: one in each prologue, one per body)

@@ -35,6 +35,8 @@
 // add to the same element, so the sums have a fixed order.
 #include "pd_internal.h"
 
+#include <math_constants.h>
+
 #include <climits>
 #include <cstring>
 #include <type_traits>
@@ -57,7 +59,7 @@ constexpr int kTile = 128;               // words t per tile: the lanes of tenso
 constexpr int kMaxHigh = 28;             // high orbits (12 + 28 = 40 columns)
 constexpr size_t kSmemMax = 112 * 1024;   // two CTAs per SM
 constexpr int kTmemCols = 256;           // tensor-memory columns of a CTA: two CTAs fill an SM
-constexpr int kWaitLimit = 1 << 14;      // mbarrier polls (each suspended up to a millisecond) before a wait gives up
+constexpr int kDrainPolls = 1 << 12;     // polls of the wait for a product in flight after its wait gave up
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~size_t(15); }
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -178,6 +180,7 @@ __host__ __device__ inline LayoutR layout_r(int KP, int H, int N)
 struct RemoveArgs {
     int omega, N, L, H;
     int lo_off[kLT + 2];
+    int polls;                           // of a wait before it gives up
     int64_t first, end;                  // blocks of t of this launch, in words
     int64_t zbase[kLT + 1];              // scratch of the rows with k low pairs
     const uint32_t *words;
@@ -283,9 +286,9 @@ __device__ __forceinline__ uint64_t g_desc(uint32_t saddr)
     return d;
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase)
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t phase, int polls)
 {
-    for (int it = 0; it < kWaitLimit; ++it) {
+    for (int it = 0; it < polls; ++it) {
         uint32_t done;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}\n"
@@ -295,6 +298,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase)
         if (done) return true;
     }
     return false;
+}
+
+// A bounded wait for a product.  When it expires, what the launch writes is void
+// (the add kernels write NaN) and the CTA takes no more blocks, at most one that
+// is prepared already; the product's operands and tensor memory are still in use,
+// so it is waited for once more.
+__device__ __noinline__ void expired(uint32_t bar, uint32_t phase, int *s_void)
+{
+    *reinterpret_cast<volatile int *>(s_void) = 1;
+    mbar_poll(bar, phase, kDrainPolls);
+}
+__device__ __forceinline__ void wait_product(uint32_t bar, uint32_t phase, int polls, int *s_void)
+{
+    if (!mbar_poll(bar, phase, polls)) expired(bar, phase, s_void);
 }
 
 __device__ __forceinline__ float to_tf32(float v)
@@ -389,6 +406,12 @@ __device__ __forceinline__ void issue_product(const uint32_t tmem, const uint32_
 // multiply-adds instead of the tensor cores (packed pairs, coefficients from
 // shared memory or the constant bank, 8, 10 or 12 low orbits, hops between high
 // orbits in registers): 0.127 to 0.18 ms.
+__device__ __forceinline__ void report_void(Tickets *tk)
+{
+    atomicOr(&tk->mark, kMarkVoid);
+    atomicExch(&tk->expired, 1);
+}
+
 template <int KP>
 __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *__restrict__ G, const float *__restrict__ d,
                                               const float *__restrict__ x, float *__restrict__ y, Tickets *tk,
@@ -398,6 +421,7 @@ __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t s_bar[C::kGroups];
     __shared__ uint32_t s_tmem;
+    __shared__ int s_void;                        // a wait gave up
     const int L = A.L, H = A.H, N = A.N;
     const LayoutR lay = layout_r(KP, H, N);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, group = warp >> 2;
@@ -418,6 +442,7 @@ __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *
     }
     stage_tables<KP>(A, G, d, smem + lay.b, bin, crk, dh, dlow, C::kThreads);
     if (tid < 3) bufs[tid].x[kSpare] = 0.0f;
+    if (tid == 0) s_void = 0;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // G: generic stores -> tensor core reads
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -426,11 +451,11 @@ __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *
     const uint32_t trow = tmem + ((uint32_t)(warp & 3) << 21);       // this warp's 32 lanes
     const uint32_t bar = smem_u32(&s_bar[group < C::kGroups ? group : 0]);
     uint32_t phase = 0;
-    bool gave_up = false, odd = false;            // odd: a row of Z is NaN
+    bool odd = false;                             // a row of Z is NaN
 
     auto take = [&](BlockSmem &bs) {              // the last warp
-        long long b = 0;
-        if (lane == 0) b = A.first + (long long)atomicAdd(&tk->hx_next, 1ull);
+        long long b = A.end;                      // (none after a wait gave up)
+        if (lane == 0 && !*reinterpret_cast<volatile int *>(&s_void)) b = A.first + (long long)atomicAdd(&tk->hx_next, 1ull);
         b = __shfl_sync(0xffffffffu, b, 0);
         if (b < A.end) prepare_block(bs, A, __ldg(A.words + b), bin, crk, dh, x);
         if (lane == 0) bs.b = b;
@@ -525,7 +550,7 @@ __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *
                     }
                     __syncwarp();
                     if ((c + C::kGroups) * kTile < nt) load(c + C::kGroups);   // overlaps the product
-                    if (gave_up || !mbar_wait(bar, phase)) gave_up = true;
+                    wait_product(bar, phase, A.polls, &s_void);
                     phase ^= 1u;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     for_each<KP / 8>([&](auto gc) {
@@ -553,12 +578,12 @@ __device__ __forceinline__ void remove_blocks(const RemoveArgs &A, const float *
         __syncthreads();
         cur = nxt;
     }
-    if (odd) atomicOr(&tk->pad, 1ull);
-    if (gave_up) atomicExch(&tk->bar.err, 1);
+    if (odd) atomicOr(&tk->mark, kMarkSplit);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s_tmem), "r"(kTmemCols) : "memory");
+    if (tid == 0 && s_void) report_void(tk);
     if (arrive_last(&tk->hx_done, ctas) && tid == 0) tk->hx_next = 0ull;
 }
 
@@ -639,6 +664,7 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t s_bar[kSmallGroups];
     __shared__ uint32_t s_tmem;
+    __shared__ int s_void[kSmallGroups][2];       // a wait gave up in an item of this parity
     const RemoveArgs &A = S.r;
     const int L = A.L, H = A.H, N = A.N;
     const LayoutS lay = layout_s(KP, H, N);
@@ -664,6 +690,7 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
     }
     stage_tables<KP>(A, G, d, smem + lay.b, bin, crk, dh, dlow, 128 * kSmallGroups);
     if (gt == 0) bx[kSmallRows] = 0.0f;
+    if (gt < 2) s_void[group][gt] = 0;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // G: generic stores -> tensor core reads
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -672,7 +699,7 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
     const uint32_t trow = tmem + ((uint32_t)(warp & 3) << 21);       // this warp's 32 lanes
     const uint32_t bar = smem_u32(&s_bar[group]);
     uint32_t phase = 0;
-    bool gave_up = false, odd = false;
+    bool odd = false;
     auto sync = [&] { asm volatile("bar.sync %0, 128;\n" ::"r"(group + 1) : "memory"); };
 
     // Items in turn (sorted by class, so every group gets its share of each).
@@ -697,7 +724,7 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
     const int64_t step = (int64_t)gridDim.x * kSmallGroups;
     int64_t it = (int64_t)blockIdx.x * kSmallGroups + group;
     Item cur = fetch(it);
-    while (cur.m > 0) {
+    for (int parity = 0; cur.m > 0; parity ^= 1) {
         it += step;
         const Item nxt = fetch(it);
         const int k = cur.k, m = cur.m;
@@ -764,7 +791,7 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
                 issue_product<KP>(tmem, smem_u32(smem + lay.b), bar);
             }
             __syncwarp();
-            if (gave_up || !mbar_wait(bar, phase)) gave_up = true;
+            wait_product(bar, phase, A.polls, &s_void[group][parity]);
             phase ^= 1u;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             for_each<KP / 8>([&](auto gc) {
@@ -800,14 +827,16 @@ remove_small_kernel(const __grid_constant__ SmallArgs S, const float *__restrict
             y[bbase[i] + t] = fmaf(D, bx[r], s);
         }
         sync();
+        // (group-uniform: the flag is next written two items on)
+        if (s_void[group][parity]) break;         // once a wait has given up, no more items
         cur = nxt;
     }
-    if (odd) atomicOr(&tk->pad, 1ull);
-    if (gave_up) atomicExch(&tk->bar.err, 1);
+    if (odd) atomicOr(&tk->mark, kMarkSplit);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s_tmem), "r"(kTmemCols) : "memory");
+    if (gt == 0 && (s_void[group][0] || s_void[group][1])) report_void(tk);
 }
 
 // ---- pair addition --------------------------------------------------------------
@@ -830,10 +859,11 @@ struct AddArgs {
     int first_launch, last_launch;       // of the product
 };
 
-// one row term by term (elements that are not finite)
+// one row term by term (elements that are not finite), or NaN (void)
 __device__ __noinline__ float row_slow(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
-                                       const float *__restrict__ x, uint64_t s, float xs)
+                                       const float *__restrict__ x, uint64_t s, float xs, unsigned mark)
 {
+    if (mark & kMarkVoid) return CUDART_NAN_F;
     float D = 0.0f;
     for (int p = 0; p < A.omega; ++p)
         if (s >> p & 1ull) D += d[p];
@@ -861,7 +891,7 @@ __device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float>
         if (threadIdx.x == 0) part[blockIdx.x] = v;
     }
     if (!arrive_last(&tk->hx_done, ctas)) return;
-    if (A.last_launch && threadIdx.x == 0) tk->pad = 0ull;
+    if (A.last_launch && threadIdx.x == 0) tk->mark = 0u;
     if (!part) return;
     double s = 0.0;
     for (int i = threadIdx.x; i < (int)gridDim.x; i += kAThreads) s += __ldcg(part + i);
@@ -884,7 +914,7 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
     const int NB = A.N + 2;
     for (int i = threadIdx.x; i < A.H * NB; i += kAThreads)
         bin[i] = (uint32_t)__ldg(A.binom + (A.L + i / NB) * kBinomStride + i % NB);
-    const bool slow = *reinterpret_cast<volatile unsigned long long *>(&tk->pad) != 0ull;
+    const unsigned mark = __ldcg(&tk->mark);
     __syncthreads();
     DotAcc<float> dot;
     int c = A.c0;
@@ -908,6 +938,16 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) Dh += __shfl_xor_sync(0xffffffffu, Dh, o);
         }
+        if (mark) {                               // (in a loop of its own: the call costs the other one registers)
+#pragma unroll 1
+            for (int r = threadIdx.x; r < nk; r += kAThreads) {
+                const float xr = __ldg(x + base + r);
+                const float acc = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr, mark);
+                y[base + r] = acc;
+                if (part) dot.add(xr, acc);
+            }
+            continue;
+        }
         for (int r0 = threadIdx.x; r0 < nk; r0 += kARows * kAThreads) {
             float acc[kARows], xr[kARows];
             bool in[kARows];
@@ -915,7 +955,7 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
             for (int i = 0; i < kARows; ++i) {
                 const int r = r0 + i * kAThreads;
                 in[i] = r < nk;
-                xr[i] = in[i] && (part || k == 0 || slow) ? __ldg(x + base + r) : 0.0f;
+                xr[i] = in[i] && (part || k == 0) ? __ldg(x + base + r) : 0.0f;
                 acc[i] = k == 0 ? Dh * xr[i] : in[i] ? y[base + r] : 0.0f;
             }
             const float *zr = z + r0;
@@ -939,7 +979,6 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
             for (int i = 0; i < kARows; ++i) {
                 const int r = r0 + i * kAThreads;
                 if (!in[i]) continue;
-                if (slow) acc[i] = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr[i]);
                 y[base + r] = acc[i];
                 if (part) dot.add(xr[i], acc[i]);
             }
@@ -976,7 +1015,7 @@ add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G,
     for (int i = threadIdx.x; i < A.H * NB; i += kAThreads)
         bin[i] = (uint32_t)__ldg(A.binom + (A.L + i / NB) * kBinomStride + i % NB);
     for (int i = threadIdx.x; i < A.H; i += kAThreads) dh[i] = d[A.L + i];
-    const bool slow = *reinterpret_cast<volatile unsigned long long *>(&tk->pad) != 0ull;
+    const unsigned mark = __ldcg(&tk->mark);
     __syncthreads();
     DotAcc<float> dot;
     for (int c = A.c0; c < A.c1; ++c) {
@@ -994,12 +1033,12 @@ add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G,
                 base += bin[j * NB + ++o];
                 Dh += dh[j];
             }
-            const float xr = part || k == 0 || slow ? __ldg(x + base) : 0.0f;
+            const float xr = part || k == 0 || mark ? __ldg(x + base) : 0.0f;
             float acc = k == 0 ? Dh * xr : y[base];
             const float *z = A.scratch + A.zbase[k] + (int64_t)b * ph * nk + r;
 #pragma unroll 4
             for (int a = 0; a < ph; ++a, z += nk) acc += __ldg(z);
-            if (slow) acc = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr);
+            if (mark) acc = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr, mark);
             y[base] = acc;
             if (part) dot.add(xr, acc);
         }
@@ -1201,6 +1240,7 @@ static void fill_args(const FacPlan &p, const uint64_t *binom, WordClasses &ct, 
     A = AddArgs{};
     R.omega = A.omega = p.omega;
     R.N = A.N = N;
+    R.polls = p.polls;
     R.L = A.L = L;
     R.H = A.H = H;
     for (int k = 0; k <= kLT; ++k) {

@@ -110,6 +110,7 @@ struct FacPlan {
     bool by_class = false;               // the rows of one class (low pairs) at a time
     int64_t scratch_len = 0;             // floats of scratch
     int grid_t = 0, grid_y = 0;
+    int polls = 1 << 12;                 // of a wait, each suspended up to a millisecond
     size_t smem = 0;
     uint32_t *twords = nullptr, *ywords = nullptr;   // device
     uint16_t *low = nullptr;             // [2^L] low words
@@ -148,15 +149,18 @@ struct GridBar {                     // grid-wide barrier of a cooperative launc
     unsigned int count;              // CTAs arrived at the current barrier
     unsigned int gen;                // generation: opened by the last CTA to arrive
     int err;                         // a wait gave up (the launch's results are void)
-    int pad;
 };
 struct Tickets {
     unsigned long long hx_next;      // next block of a persistent H*x launch
     unsigned long long hx_done;      // CTAs of that launch that have finished
     unsigned long long vec_done;     // CTAs of a streaming kernel whose partial sums are written
-    unsigned long long pad;          // variant 2: an element could not be split (not finite)
+    unsigned int mark;               // variant 2, one product: kMark* bits
     GridBar bar;                     // the fused Lanczos step's barriers
+    int expired;                     // variant 2: a wait of a product gave up (stays set until a solve
+                                     // starts; follows bar.err, so that one copy reads both)
 };
+constexpr unsigned int kMarkSplit = 1;   // an element could not be split (not finite)
+constexpr unsigned int kMarkVoid = 2;    // a wait gave up: rows written from then on are NaN
 
 #ifdef __CUDACC__
 // ---- device reductions shared by the kernels ---------------------------------

@@ -91,6 +91,7 @@ _SIGNATURES = {
     "pairdiag_release_cache": (ctypes.c_int, [_P]),
     "pairdiag_set_profiling": (ctypes.c_int, [_H, ctypes.c_int]),
     "pairdiag_set_step_fusion": (ctypes.c_int, [_H, ctypes.c_int]),
+    "pairdiag_set_wait_limit": (ctypes.c_int, [_H, ctypes.c_int]),
     "pairdiag_get_profile": (ctypes.c_int, [_H, ctypes.c_int, _P, _P]),
     "pairdiag_batch_ground_state": (ctypes.c_int, [ctypes.c_int, _P, _P, _P, _P, ctypes.c_double,
                                                    ctypes.POINTER(pairdiag_options), _H, _P, _P, _P, _P]),
@@ -488,6 +489,11 @@ def pairdiag_set_profiling(h, on: bool) -> None:
 def pairdiag_set_step_fusion(h, on: bool) -> None:
     """One cooperative launch per Lanczos step (True, default) or three launches."""
     _check(lib().pairdiag_set_step_fusion(h, 1 if on else 0))
+
+
+def pairdiag_set_wait_limit(h, polls: int) -> None:
+    """Polls (of up to a millisecond) before a wait of the FP32 removal product gives up."""
+    _check(lib().pairdiag_set_wait_limit(h, polls))
 
 
 PD_PROF_STEP = 2     # record kinds PD_PROF_STEP + PD_PREC_*: the Lanczos steps' vector work
