@@ -95,9 +95,13 @@ typedef struct {
                                states or more, no or only full orbits, no room for its
                                scratch), 2-5 fall back to 1 when their shared memory does not
                                fit.  A truncated handle (pairdiag_truncate) computes its kept
-                               rows by variant 3 on x spread over the full space (2-5; 12 bytes
-                               per state of the full space), by variant 1 through the index
-                               map where 1 is asked for or that memory is missing */
+                               rows by variant 3 on x spread over the full space (2-5; 8 bytes
+                               per state of the full space, 4 more for FP32 products, 10 per
+                               kept state), by variant 1 through the index map where 1 is asked
+                               for or that memory is missing; it holds no removal scratch.
+                               That memory and the scratch are given back when the solver's
+                               own vectors do not fit beside them, unless a product of the
+                               handle has been captured in a graph */
 } pairdiag_options;
 
 typedef struct {
@@ -487,6 +491,15 @@ int pairdiag_tune_get(int omega, int n_pairs, int precision, int *low_bits, int 
  * owned by live handles are not touched.  Thread-safe; always PD_OK.
  */
 int pairdiag_release_cache(size_t *released_bytes);
+
+/*
+ * For tests of what the library does without memory: the next `count` device
+ * allocations of at least `bytes` bytes that it makes on the calling thread
+ * fail as if the device had no room (0 ends it).  What only makes products
+ * faster is given back then before the allocation is tried again: the removal's
+ * scratch (hx_variant 2) and a truncated handle's full-space vectors.
+ */
+int pairdiag_fail_alloc(size_t bytes, int count);
 
 /* ------------------------------------------------------- diagnostics ---- */
 

@@ -149,13 +149,19 @@ struct pairdiag {
     int *d_kblk_rows = nullptr;
     uint64_t *d_kfull = nullptr;     // full index and low word of every kept state
     uint16_t *d_klow = nullptr;
-    void *d_xf[2] = {nullptr, nullptr};   // x in the full space, zeros at the dropped states (per storage type)
+    // x in the full space, zeros at the dropped states, per storage type: FP64 from
+    // the truncation on, FP32 then (mixed form) or from the first FP32 product on
+    void *d_xf[2] = {nullptr, nullptr};
+    bool xf_tried[2] = {false, false};
     // the block list in the order the persistent H*x kernels take it when
     // there are few blocks per CTA: largest blocks first (ascending high word
     // within a size), so the launch does not end on one CTA's large block
     uint64_t *d_lpt_h = nullptr, *d_lpt_base = nullptr;
     Blocks B{};
-    FacPlan fac;                     // the FP32 product by pair removal
+    bool use_fac = false;            // FP32 products of the full space go by pair removal
+    int wait_polls = FacPlan{}.polls;
+    bool captured = false;           // a graph holds addresses of the optional memory
+    FacPlan fac;                     // the plan, on while its memory is there
     unsigned char *d_fac = nullptr;  // its tables and scratch
     int device = 0;
     cudaStream_t st = nullptr;
@@ -329,6 +335,13 @@ int build_tables(pairdiag *h)
 
 // The plan of the FP32 product by pair removal: its tables are made on the
 // device; h->fac.on stays false where it does not apply.
+void drop_fac(pairdiag *h)
+{
+    pool_free(h->d_fac);
+    h->d_fac = nullptr;
+    h->fac = FacPlan{};
+}
+
 int build_fac(pairdiag *h)
 {
     FacPlan &f = h->fac;
@@ -346,51 +359,114 @@ int build_fac(pairdiag *h)
                  at_low = place(sizeof(uint16_t) << f.L), at_up = place(sizeof(uint32_t) * (size_t)f.table),
                  at_z = place(sizeof(float) * fac_zeros()), at_s = place(sizeof(float) * (size_t)f.scratch_len);
     if (dalloc(&h->d_fac, off) != PD_OK) {        // no room: the kernels without scratch serve the handle
-        h->d_fac = nullptr;
-        f = FacPlan{};
+        drop_fac(h);
         return PD_OK;
     }
+    f.polls = h->wait_polls;
     f.twords = reinterpret_cast<uint32_t *>(h->d_fac + at_t);
     f.ywords = reinterpret_cast<uint32_t *>(h->d_fac + at_y);
     f.low = reinterpret_cast<uint16_t *>(h->d_fac + at_low);
     f.up = reinterpret_cast<uint32_t *>(h->d_fac + at_up);
     f.zeros = reinterpret_cast<float *>(h->d_fac + at_z);
     f.scratch = reinterpret_cast<float *>(h->d_fac + at_s);
-    // (on the legacy stream: the blocking uploads that follow in pairdiag_create
-    // are ordered after it)
     PD_CUDA(fac_build(f, h->d_binom, h->st));
+    return PD_OK;
+}
+
+// The basis blocks as the product of a precision takes them: kept rows are
+// gathered from a full-space x where there is one of that type
+Blocks blocks_of(const pairdiag *h, int precision)
+{
+    Blocks B = h->B;
+    if (precision > 1 || !h->d_xf[precision]) B.kept_low = nullptr;
+    return B;
+}
+
+void set_grids(pairdiag *h)
+{
+    for (int p = 0; p < 3; ++p) h->hxgrid[p] = hx_grid(blocks_of(h, p), p);
+}
+
+void drop_kept_lists(pairdiag *h)
+{
+    void **part[] = {(void **)&h->d_kfull, (void **)&h->d_klow, &h->d_xf[0], &h->d_xf[1]};
+    for (void **q : part) {
+        pool_free(*q);
+        *q = nullptr;
+    }
+    h->B.kept_low = nullptr;
+}
+
+// Memory that only makes products faster (the removal's scratch, the full-space
+// vectors of a truncated space) makes way for what the handle cannot do without.
+// It stays once a product has been captured: a graph then holds its addresses.
+bool give_back(pairdiag *h)
+{
+    if (h->captured || !(h->d_fac || h->d_kfull)) return false;
+    cudaStreamSynchronize(h->st);                 // no queued product may still use it
+    drop_fac(h);
+    drop_kept_lists(h);
+    set_grids(h);
+    return true;
+}
+
+// an allocation that the handle cannot do without
+template <typename T>
+int must_alloc(pairdiag *h, T **p, size_t count)
+{
+    int st = dalloc(p, count);
+    if (st == PD_ENOMEM && give_back(h)) st = dalloc(p, count);
+    return st;
+}
+
+template <typename T>
+int must_upload(pairdiag *h, T **p, const std::vector<T> &v)
+{
+    PD_TRY(must_alloc(h, p, v.size()));
+    PD_CUDA(cudaMemcpy(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
     return PD_OK;
 }
 
 int ensure_window(pairdiag *h, int dtype, int window)
 {
     const size_t es = dtype == 0 ? sizeof(double) : sizeof(float);
-    if (h->d_Q[dtype] && h->Qwin[dtype] >= window) return PD_OK;
-    if (h->d_Q[dtype]) {                          // a larger window: the old one may still be in use
-        cudaStreamSynchronize(h->st);
-        pool_free(h->d_Q[dtype]);
-        h->d_Q[dtype] = nullptr;
+    if (!h->d_Q[dtype] || h->Qwin[dtype] < window) {
+        if (h->d_Q[dtype]) {                      // a larger window: the old one may still be in use
+            cudaStreamSynchronize(h->st);
+            pool_free(h->d_Q[dtype]);
+            h->d_Q[dtype] = nullptr;
+        }
+        if (must_alloc(h, reinterpret_cast<char **>(&h->d_Q[dtype]), es * (size_t)window * (size_t)h->ldq) != PD_OK)
+            return fail(PD_ENOMEM, "Lanczos window of %d x %lld elements: no room on the device", window, (long long)h->dim);
+        h->Qwin[dtype] = window;
     }
-    void *q = nullptr;
-    cudaError_t e = pool_alloc(&q, es * (size_t)window * (size_t)h->ldq);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail(PD_ENOMEM, "Lanczos window of %d x %lld elements: %s", window, (long long)h->dim,
-                    cudaGetErrorString(e));
-    }
-    h->d_Q[dtype] = q;
-    h->Qwin[dtype] = window;
-    if (!h->d_p[dtype]) {
-        e = pool_alloc(&h->d_p[dtype], es * (size_t)h->dim);
-        if (e != cudaSuccess) { cudaGetLastError(); return fail(PD_ENOMEM, "work vector: %s", cudaGetErrorString(e)); }
-    }
+    if (!h->d_p[dtype] && must_alloc(h, reinterpret_cast<char **>(&h->d_p[dtype]), es * (size_t)h->dim) != PD_OK)
+        return fail(PD_ENOMEM, "work vector of %lld elements: no room on the device", (long long)h->dim);
     return PD_OK;
 }
 
 int ensure_fp64_pair(pairdiag *h)
 {
-    if (!h->d_v64) PD_TRY(dalloc(&h->d_v64, (size_t)h->dim));
-    if (!h->d_w64) PD_TRY(dalloc(&h->d_w64, (size_t)h->dim));
+    if (!h->d_v64) PD_TRY(must_alloc(h, &h->d_v64, (size_t)h->dim));
+    if (!h->d_w64) PD_TRY(must_alloc(h, &h->d_w64, (size_t)h->dim));
+    return PD_OK;
+}
+
+// the full-space x of storage type t of a truncated handle; without room, or
+// while the stream is captured, products of that type go through the index map
+int full_x(pairdiag *h, int t)
+{
+    if (h->xf_tried[t] || !h->d_klow) return PD_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return PD_OK;
+    }
+    h->xf_tried[t] = true;
+    const size_t bytes = (t == 0 ? sizeof(double) : sizeof(float)) * (size_t)h->full_dim;
+    if (dalloc(reinterpret_cast<char **>(&h->d_xf[t]), bytes) != PD_OK) return PD_OK;
+    PD_CUDA(cudaMemsetAsync(h->d_xf[t], 0, bytes, h->st));
+    h->hxgrid[t] = hx_grid(blocks_of(h, t), t);
     return PD_OK;
 }
 
@@ -421,7 +497,8 @@ int hx(pairdiag *h, int precision, const void *x, void *y, const int *skip = nul
     std::pair<cudaEvent_t, cudaEvent_t> *ev = nullptr;
     PD_TRY(prof_begin(h, precision == 2 ? 0 : precision, &ev));    // float-float rows count as FP64
     const HxDot dot{h->d_blkdot, dot_out};
-    Blocks B = h->B;
+    if (h->d_klow && precision < 2 && !h->d_xf[precision]) PD_TRY(full_x(h, precision));
+    Blocks B = blocks_of(h, precision);
     if (h->d_lpt_h && !B.kept_map && B.nblocks <= kLptPerCta * (int64_t)h->hxgrid[precision]) {
         B.blk_h = h->d_lpt_h;
         B.blk_base = h->d_lpt_base;
@@ -737,7 +814,7 @@ int ground_state_impl(pairdiag *h, double tol, double *e0, double *vec_dev, bool
     const int win = std::min<int64_t>(std::max(1, h->opt.window), std::min<int64_t>(dim, kMaxWindow));
     // (an earlier product whose wait gave up has left its rows NaN; it says
     // nothing about this solve)
-    if (h->fac.on) PD_CUDA(cudaMemsetAsync(&h->d_tk->expired, 0, sizeof(int), h->st));
+    if (h->use_fac) PD_CUDA(cudaMemsetAsync(&h->d_tk->expired, 0, sizeof(int), h->st));
     CycleStats cs;
     int status = PD_OK;
     int fp32_iters = 0;
@@ -879,7 +956,7 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
         int lb = 0, hv = 0;
         if (tuned_schedule(omega, n_pairs, o.precision, &lb, &hv)) { o.low_bits = lb; o.hx_variant = hv; }
     }
-    bool use_fac = o.hx_variant == 2;             // variant 2 where it serves the problem
+    bool use_fac = o.hx_variant == 2;             // where it serves the problem
     if (o.hx_variant == 0) {
         // untuned: direct gathers.  The block split follows the dimension: a CTA
         // owns a block, so few large blocks leave SMs idle or end the launch on
@@ -902,6 +979,7 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
     }
     pairdiag *h = new pairdiag();
     h->omega = omega; h->n = n_pairs; h->opt = o;
+    h->use_fac = use_fac;
     h->e.assign(e, e + omega);
     h->G.assign(G, G + (size_t)omega * omega);
     h->d.resize(omega);
@@ -914,7 +992,6 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { cudaGetLastError(); st = fail(PD_ECUDA, "no CUDA device"); break; }
         if ((st = build_tables(h)) != PD_OK) break;
-        if (use_fac && (st = build_fac(h)) != PD_OK) break;
         std::vector<float> G32(h->G.begin(), h->G.end()), d32(h->d.begin(), h->d.end());
         auto split = [](const std::vector<double> &v) {
             std::vector<float2> r(v.size());
@@ -924,25 +1001,27 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
             }
             return r;
         };
-        if ((st = upload(&h->d_G64, h->G)) != PD_OK) break;
-        if ((st = upload(&h->d_d64, h->d)) != PD_OK) break;
-        if ((st = upload(&h->d_G32, G32)) != PD_OK) break;
-        if ((st = upload(&h->d_d32, d32)) != PD_OK) break;
-        if ((st = upload(&h->d_Gff, split(h->G))) != PD_OK) break;
-        if ((st = upload(&h->d_dff, split(h->d))) != PD_OK) break;
         if ((st = dalloc(&h->d_tk, 1)) != PD_OK) break;
         if (cudaMemset(h->d_tk, 0, sizeof(Tickets)) != cudaSuccess) { st = fail(PD_ECUDA, "memset"); break; }
-        if ((st = dalloc(&h->d_blkdot, (size_t)std::max<int64_t>(h->B.nblocks, fac_partials(h->fac)))) != PD_OK) break;
+        if ((st = dalloc(&h->d_blkdot, (size_t)std::max<int64_t>(h->B.nblocks, use_fac ? fac_partials() : 0))) != PD_OK) break;
         h->ldq = (h->dim + 3) / 4 * 4;
-        h->hxgrid[0] = hx_grid(h->B, 0);
-        h->hxgrid[1] = hx_grid(h->B, 1);
-        h->hxgrid[2] = hx_grid(h->B, 2);
+        set_grids(h);
         h->rgrid = (int)std::min<int64_t>(h->B.nblocks, vec_grid());
         h->part_count = (size_t)std::max(vec_grid(), h->rgrid) * kMaxWindow;
         if ((st = dalloc(&h->d_part, h->part_count)) != PD_OK) break;
         if ((st = dalloc(&h->d_S, 1)) != PD_OK) break;
         if ((st = dalloc(&h->d_small, 8)) != PD_OK) break;
         if (cudaMemset(h->d_S, 0, sizeof(LanczosScalars)) != cudaSuccess) { st = fail(PD_ECUDA, "memset"); break; }
+        if ((st = upload(&h->d_G64, h->G)) != PD_OK) break;
+        if ((st = upload(&h->d_d64, h->d)) != PD_OK) break;
+        if ((st = upload(&h->d_G32, G32)) != PD_OK) break;
+        if ((st = upload(&h->d_d32, d32)) != PD_OK) break;
+        if ((st = upload(&h->d_Gff, split(h->G))) != PD_OK) break;
+        if ((st = upload(&h->d_dff, split(h->d))) != PD_OK) break;
+        // the removal's scratch last, after all that the handle cannot do without
+        if (use_fac && (st = build_fac(h)) != PD_OK) break;
+        // (the caller may go on with a stream that does not follow this one)
+        if (cudaStreamSynchronize(h->st) != cudaSuccess) { st = fail(PD_ECUDA, "tables"); break; }
     } while (0);
     if (st != PD_OK) {
         free_all(h);
@@ -981,7 +1060,7 @@ int pairdiag_set_wait_limit(pairdiag_t *h, int polls)
 {
     if (!h) return fail(PD_EINVAL, "null handle");
     if (polls < 0 || polls > 1 << 20) return fail(PD_EINVAL, "polls outside 0..2^20");
-    h->fac.polls = polls;
+    h->wait_polls = h->fac.polls = polls;
     return PD_OK;
 }
 
@@ -1035,7 +1114,7 @@ int pairdiag_basis(const pairdiag_t *h, uint64_t *out)
 {
     if (!h || !out) return fail(PD_EINVAL, "null argument");
     uint64_t *d = nullptr;
-    PD_TRY(dalloc(&d, (size_t)h->full_dim));
+    PD_TRY(must_alloc(const_cast<pairdiag *>(h), &d, (size_t)h->full_dim));
     int st = pairdiag_basis_dev(h, 0, h->full_dim, d);
     if (st == PD_OK) {
         cudaError_t e1 = cudaMemcpyAsync(out, d, sizeof(uint64_t) * h->full_dim, cudaMemcpyDeviceToHost, h->st);
@@ -1062,6 +1141,11 @@ int pairdiag_hx_dev(pairdiag_t *h, int precision, const void *x_dev, void *y_dev
     if (x_dev == y_dev) return fail(PD_EINVAL, "x and y must not overlap");
     if (precision == PD_HX_FLOATFLOAT && h->hxgrid[2] < 1)
         return fail(PD_ENOTSUP, "no float-float product for this handle (truncated space or shared memory)");
+    if (!h->captured && (h->d_fac || h->d_kfull)) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(h->st, &cs) == cudaSuccess) h->captured = cs != cudaStreamCaptureStatusNone;
+        else cudaGetLastError();
+    }
     return hx(h, precision, x_dev, y_dev);
 }
 
@@ -1163,8 +1247,8 @@ int pairdiag_lowest_states_dev(pairdiag_t *h, int k, double tol, double *energie
         h->d_L64 = nullptr;
         h->d_L32 = nullptr;
         h->lock_cap = 0;
-        PD_TRY(dalloc(&h->d_L64, (size_t)k * (size_t)ld));
-        if (mixed) PD_TRY(dalloc(&h->d_L32, (size_t)k * (size_t)ld));
+        PD_TRY(must_alloc(h, &h->d_L64, (size_t)k * (size_t)ld));
+        if (mixed) PD_TRY(must_alloc(h, &h->d_L32, (size_t)k * (size_t)ld));
         h->lock_cap = k;
     }
     if (!h->d_lockc) PD_TRY(dalloc(&h->d_lockc, (size_t)kMaxWindow));
@@ -1224,12 +1308,13 @@ void drop_space(pairdiag *h)
     cudaStreamSynchronize(h->st);
     void **vecs[] = {&h->d_Q[0], &h->d_Q[1], &h->d_p[0], &h->d_p[1], (void **)&h->d_v64, (void **)&h->d_w64,
                      (void **)&h->d_L64, (void **)&h->d_L32, (void **)&h->d_kmap, (void **)&h->d_kblk_h,
-                     (void **)&h->d_kblk_base, (void **)&h->d_kblk_first, (void **)&h->d_kblk_rows,
-                     (void **)&h->d_kfull, (void **)&h->d_klow, &h->d_xf[0], &h->d_xf[1]};
+                     (void **)&h->d_kblk_base, (void **)&h->d_kblk_first, (void **)&h->d_kblk_rows};
     for (void **v : vecs) {
         pool_free(*v);
         *v = nullptr;
     }
+    drop_kept_lists(h);
+    h->xf_tried[0] = h->xf_tried[1] = false;
     h->Qwin[0] = h->Qwin[1] = 0;
     h->lock_cap = 0;
     h->n_locked = 0;
@@ -1239,13 +1324,19 @@ void drop_space(pairdiag *h)
     h->B.kept_nblocks = 0;
     h->B.kept_blk_first = nullptr;
     h->B.kept_blk_rows = nullptr;
-    h->B.kept_low = nullptr;
     h->dim = h->full_dim;
     h->nnz = h->full_nnz;
     h->ldq = (h->dim + 3) / 4 * 4;
-    h->hxgrid[0] = hx_grid(h->B, 0);
-    h->hxgrid[1] = hx_grid(h->B, 1);
-    h->hxgrid[2] = hx_grid(h->B, 2);
+    set_grids(h);
+}
+
+// the removal's memory of a handle that has come back to the full space
+int restore_fac(pairdiag *h)
+{
+    if (h->d_kmap || !h->use_fac || h->d_fac) return PD_OK;
+    PD_TRY(build_fac(h));
+    PD_CUDA(cudaStreamSynchronize(h->st));        // (the caller may go on with another stream)
+    return PD_OK;
 }
 
 // The kept states of Sec. 3.5 and the map full index -> kept index.  Returns
@@ -1268,11 +1359,8 @@ int build_truncation(pairdiag *h, int64_t limit, int64_t bins, int64_t *kept)
         for (void *p : tmp) pool_free(p);
     };
     auto talloc = [&](void **p, size_t bytes) -> int {
-        const cudaError_t e = pool_alloc(p, bytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(PD_ENOMEM, "truncation: %zu bytes: %s", bytes, cudaGetErrorString(e));
-        }
+        if (must_alloc(h, reinterpret_cast<char **>(p), bytes) != PD_OK)
+            return fail(PD_ENOMEM, "truncation: no room for %zu bytes", bytes);
         tmp.push_back(*p);
         return PD_OK;
     };
@@ -1325,7 +1413,13 @@ int build_truncation(pairdiag *h, int64_t limit, int64_t bins, int64_t *kept)
         int64_t *d_first = nullptr;
         PD_TRY(talloc((void **)&d_first, sizeof(int64_t) * first.size()));
         PD_CUDA(cudaMemcpyAsync(d_first, first.data(), sizeof(int64_t) * first.size(), cudaMemcpyHostToDevice, st));
-        PD_TRY(dalloc(&h->d_kmap, (size_t)full));
+        // products of the truncated space take no removal scratch (a graph of a
+        // full-space product may still hold its addresses)
+        if (!h->captured) {
+            PD_CUDA(cudaStreamSynchronize(st));
+            drop_fac(h);
+        }
+        PD_TRY(must_alloc(h, &h->d_kmap, (size_t)full));
         PD_CUDA(trunc_map_launch(B, h->d_d64, lo, hi, bins, cut, d_first, h->d_kmap, grid, st));
         // the blocks that hold kept states, for the truncated H*x to walk
         std::vector<uint64_t> bh(cnt.size()), bb(cnt.size());
@@ -1347,24 +1441,19 @@ int build_truncation(pairdiag *h, int64_t limit, int64_t bins, int64_t *kept)
             kf.push_back(first[b]);
             kr.push_back(cnt[b]);
         }
-        PD_TRY(upload(&h->d_kblk_h, kh));
-        PD_TRY(upload(&h->d_kblk_base, kb));
-        PD_TRY(upload(&h->d_kblk_first, kf));
-        PD_TRY(upload(&h->d_kblk_rows, kr));
+        PD_TRY(must_upload(h, &h->d_kblk_h, kh));
+        PD_TRY(must_upload(h, &h->d_kblk_base, kb));
+        PD_TRY(must_upload(h, &h->d_kblk_first, kf));
+        PD_TRY(must_upload(h, &h->d_kblk_rows, kr));
         // lists of the kept states, and x in the full space: without room for
         // them the product looks every state up in the map
-        const bool room = dalloc(&h->d_kfull, (size_t)total) == PD_OK && dalloc(&h->d_klow, (size_t)total) == PD_OK &&
-                          dalloc((double **)&h->d_xf[0], (size_t)full) == PD_OK &&
-                          dalloc((float **)&h->d_xf[1], (size_t)full) == PD_OK;
-        if (room) {
-            PD_CUDA(kept_list_launch(B, h->d_kmap, h->d_kfull, h->d_klow, grid, st));
-            PD_CUDA(cudaMemsetAsync(h->d_xf[0], 0, sizeof(double) * (size_t)full, st));
-            PD_CUDA(cudaMemsetAsync(h->d_xf[1], 0, sizeof(float) * (size_t)full, st));
-        } else {
-            void **part[] = {(void **)&h->d_kfull, (void **)&h->d_klow, &h->d_xf[0], &h->d_xf[1]};
-            for (void **q : part) {
-                pool_free(*q);
-                *q = nullptr;
+        if (h->B.variant != 1) {
+            if (dalloc(&h->d_kfull, (size_t)total) == PD_OK && dalloc(&h->d_klow, (size_t)total) == PD_OK) {
+                PD_CUDA(kept_list_launch(B, h->d_kmap, h->d_kfull, h->d_klow, grid, st));
+                PD_TRY(full_x(h, 0));
+                if (h->opt.precision == PD_PREC_MIXED) PD_TRY(full_x(h, 1));
+            } else {
+                drop_kept_lists(h);
             }
         }
         h->B.kept_nblocks = (int64_t)kh.size();
@@ -1385,7 +1474,7 @@ int pairdiag_truncate(pairdiag_t *h, int64_t dimension_limit, int64_t bins, int6
     PD_CUDA(cudaSetDevice(h->device));
     drop_space(h);
     *kept_dim = h->dim;
-    if (dimension_limit == 0) return PD_OK;
+    if (dimension_limit == 0) return restore_fac(h);
     int64_t kept = 0;
     int rc = build_truncation(h, dimension_limit, bins, &kept);
     if (rc == PD_OK && h->d_kmap) {
@@ -1396,10 +1485,8 @@ int pairdiag_truncate(pairdiag_t *h, int64_t dimension_limit, int64_t bins, int6
         h->B.kept_blk_base = h->d_kblk_base;
         h->B.kept_blk_first = h->d_kblk_first;
         h->B.kept_blk_rows = h->d_kblk_rows;
-        h->B.kept_low = h->d_xf[0] && h->d_xf[1] ? h->d_klow : nullptr;
-        h->hxgrid[0] = hx_grid(h->B, 0);
-        h->hxgrid[1] = hx_grid(h->B, 1);
-        h->hxgrid[2] = hx_grid(h->B, 2);
+        h->B.kept_low = h->d_klow;
+        set_grids(h);
         // off-diagonal nonzeros of the truncated matrix: H x with every G_ij = 1
         // and d = 0 on x = 1 counts each row's kept targets (exact in FP64)
         rc = [&]() -> int {
@@ -1413,11 +1500,12 @@ int pairdiag_truncate(pairdiag_t *h, int64_t dimension_limit, int64_t bins, int6
             if (r == PD_OK && cudaStreamSynchronize(h->st) != cudaSuccess) r = fail(PD_ECUDA, "product start");
             if (r == PD_OK) {
                 const HxProblem P1{g1, d0, nullptr, nullptr};
-                const bool direct = hx_kept_direct(h->B, 0);
+                const Blocks B = blocks_of(h, 0);
+                const bool direct = hx_kept_direct(B, 0);
                 cudaError_t ce = direct ? kept_scatter_launch(0, h->d_kfull, kept, h->d_v64, h->d_xf[0], h->st, nullptr)
                                         : cudaSuccess;
                 if (ce == cudaSuccess)
-                    ce = hx_launch(h->B, P1, 0, direct ? (const void *)h->d_xf[0] : (const void *)h->d_v64, h->d_w64,
+                    ce = hx_launch(B, P1, 0, direct ? (const void *)h->d_xf[0] : (const void *)h->d_v64, h->d_w64,
                                    h->d_tk, h->hxgrid[0], h->st);
                 if (ce == cudaSuccess)
                     ce = multidot_launch(0, h->d_w64, kept, 1, h->d_v64, kept, h->d_part, &h->d_S->dots[0], h->st,
@@ -1435,11 +1523,14 @@ int pairdiag_truncate(pairdiag_t *h, int64_t dimension_limit, int64_t bins, int6
         }();
     }
     if (rc != PD_OK) {
+        const std::string why = g_last_error;
         drop_space(h);
+        restore_fac(h);
+        g_last_error = why;
         return rc;
     }
     *kept_dim = h->dim;
-    return PD_OK;
+    return restore_fac(h);
 }
 
 int pairdiag_kept_map_dev(const pairdiag_t *h, int32_t *map_dev)

@@ -1228,7 +1228,7 @@ cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st)
     return cudaSuccess;
 }
 
-int64_t fac_partials(const FacPlan &p) { return p.grid_y; }
+int64_t fac_partials() { return (int64_t)kACtas * sm_count(); }
 
 
 static void fill_args(const FacPlan &p, const uint64_t *binom, WordClasses &ct, WordClasses &cy, RemoveArgs &R, AddArgs &A)

@@ -363,7 +363,7 @@ bool fac_pays(int omega, int n, int64_t dim);
 void fac_sizes(int omega, int n, FacPlan &p);
 size_t fac_zeros();
 cudaError_t fac_build(FacPlan &p, const uint64_t *binom, cudaStream_t st);
-int64_t fac_partials(const FacPlan &p);
+int64_t fac_partials();
 cudaError_t fac_launch(const FacPlan &p, const uint64_t *binom, const float *G, const float *d, const float *x, float *y,
                        Tickets *tk, cudaStream_t st, const int *skip, const HxDot *dot);
 // Many problems in one launch each of the two kernels: fac_item writes the

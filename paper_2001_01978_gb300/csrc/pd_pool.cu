@@ -54,11 +54,19 @@ void release_locked(Pool &P)
     cudaSetDevice(cur);
 }
 
+// pairdiag_fail_alloc: allocations of this thread that are to fail
+thread_local size_t t_fail_bytes = 0;
+thread_local int t_fail_count = 0;
+
 }  // namespace
 
 cudaError_t pool_alloc(void **p, size_t bytes)
 {
     *p = nullptr;
+    if (t_fail_count > 0 && bytes >= t_fail_bytes) {
+        --t_fail_count;
+        return cudaErrorMemoryAllocation;
+    }
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -110,6 +118,14 @@ size_t pool_cached_bytes()
 }
 
 }  // namespace pd
+
+extern "C" int pairdiag_fail_alloc(size_t bytes, int count)
+{
+    if (count < 0) return pd::fail(PD_EINVAL, "count < 0");
+    pd::t_fail_bytes = bytes;
+    pd::t_fail_count = count;
+    return PD_OK;
+}
 
 extern "C" int pairdiag_release_cache(size_t *released_bytes)
 {

@@ -89,6 +89,7 @@ _SIGNATURES = {
     "pairdiag_tridiag_lowest": (ctypes.c_int, [_H, ctypes.c_int, _P, _P, _P, _P]),
     "pairdiag_kernel_launches": (ctypes.c_int64, []),
     "pairdiag_release_cache": (ctypes.c_int, [_P]),
+    "pairdiag_fail_alloc": (ctypes.c_int, [ctypes.c_size_t, ctypes.c_int]),
     "pairdiag_set_profiling": (ctypes.c_int, [_H, ctypes.c_int]),
     "pairdiag_set_step_fusion": (ctypes.c_int, [_H, ctypes.c_int]),
     "pairdiag_set_wait_limit": (ctypes.c_int, [_H, ctypes.c_int]),
@@ -489,6 +490,11 @@ def pairdiag_set_profiling(h, on: bool) -> None:
 def pairdiag_set_step_fusion(h, on: bool) -> None:
     """One cooperative launch per Lanczos step (True, default) or three launches."""
     _check(lib().pairdiag_set_step_fusion(h, 1 if on else 0))
+
+
+def pairdiag_fail_alloc(nbytes: int, count: int) -> None:
+    """The next `count` library allocations of at least `nbytes` on this thread fail (for tests)."""
+    _check(lib().pairdiag_fail_alloc(nbytes, count))
 
 
 def pairdiag_set_wait_limit(h, polls: int) -> None:
