@@ -72,6 +72,11 @@ struct DevBuf {
         *p = static_cast<T *>(q);
         return PD_OK;
     }
+    void release(void *p)                // (its stream has finished with it)
+    {
+        ptrs.erase(std::remove(ptrs.begin(), ptrs.end(), p), ptrs.end());
+        pool_free(p);
+    }
     template <typename T>
     int upload(T **p, const std::vector<T> &v)
     {
@@ -135,7 +140,11 @@ struct ClassRun {
     int *ctl = nullptr;                  // [0] running problems, [1] cycle number, [2] reopened
     std::vector<FacProblem> fac;
     std::vector<FacBatch> fac_batch;     // one launch per tile width
+    char *fac_mem = nullptr;             // their tables, scratch and counters
     Tickets *fac_tk = nullptr;           // [fac.size()]
+    bool fac_expired = false;            // a wait inside a product gave up
+    std::vector<BatchDesc> desc;
+    const uint64_t *binom = nullptr;
     int64_t rest_blocks = 0;             // blocks of the other problems, first in the list
     unsigned long long *counter = nullptr;   // [0] next block, [1] finished CTAs of the batched H*x
     char *Q32 = nullptr, *p32 = nullptr, *Q64 = nullptr, *p64 = nullptr;
@@ -158,11 +167,34 @@ bool fac_take(ClassRun &c, int p, int om, int n, int64_t dim, int64_t off, bool 
     return true;
 }
 
+// Reads the removal's wait flags; after a synchronisation of the class's stream.
+int read_expired(ClassRun &c)
+{
+    if (!c.fac_mem) return PD_OK;
+    std::vector<Tickets> tk(c.fac.size());
+    PD_CUDA(cudaMemcpy(tk.data(), c.fac_tk, sizeof(Tickets) * tk.size(), cudaMemcpyDeviceToHost));
+    for (const Tickets &t : tk)
+        if (t.expired) c.fac_expired = true;
+    return PD_OK;
+}
+
+// The removal's memory of a class whose FP32 cycles are over
+int give_back(ClassRun &c)
+{
+    if (!c.fac_mem) return PD_OK;
+    PD_CUDA(cudaStreamSynchronize(c.st));
+    PD_TRY(read_expired(c));
+    c.buf.release(c.fac_mem);
+    c.fac_mem = nullptr;
+    return PD_OK;
+}
+
 // Tables and scratch of the class's products by pair removal.  Without room for
 // them every problem goes through the batched row-by-row kernel.
-int setup_removal(ClassRun &c, const uint64_t *binom, const std::vector<BatchDesc> &desc)
+int setup_removal(ClassRun &c)
 {
     if (c.fac.empty()) return PD_OK;
+    const uint64_t *binom = c.binom;
     // by tile width, the largest problems first
     std::stable_sort(c.fac.begin(), c.fac.end(), [](const FacProblem &a, const FacProblem &b) {
         const int ka = fac_columns(a.plan.omega), kb = fac_columns(b.plan.omega);
@@ -210,12 +242,12 @@ int setup_removal(ClassRun &c, const uint64_t *binom, const std::vector<BatchDes
         at_s[i] = place(sizeof(float) * (size_t)c.fac[i].plan.scratch_len);
         at_w[i] = place(sizeof(uint32_t) * (size_t)(c.fac[i].plan.nt + c.fac[i].plan.ny));
     }
-    char *mem = nullptr;
-    if (c.buf.alloc(&mem, bytes) != PD_OK) {
+    if (c.buf.alloc(&c.fac_mem, bytes) != PD_OK) {
         c.fac.clear();
         c.fac_batch.clear();
         return PD_OK;
     }
+    char *const mem = c.fac_mem;
     c.fac_tk = reinterpret_cast<Tickets *>(mem + at_tk);
     std::vector<char> items(item * count);
     // the uploads of binom, G and d ran on the default stream, whose order c.st
@@ -230,7 +262,7 @@ int setup_removal(ClassRun &c, const uint64_t *binom, const std::vector<BatchDes
         f.twords = reinterpret_cast<uint32_t *>(mem + at_w[i]);
         f.ywords = f.twords + f.nt;
         PD_CUDA(fac_build(f, binom, c.st));
-        const BatchDesc &D = desc[c.fac[i].p];
+        const BatchDesc &D = c.desc[c.fac[i].p];
         fac_item(f, binom, c.P.G32 + D.g_off, c.P.d32 + D.d_off, c.fac[i].off, c.fac[i].p, c.fac_tk + i, nt[i], ny[i],
                  items.data() + item * i);
     }
@@ -255,7 +287,8 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
                 const double *G_all)
 {
     const int count = c.count;
-    std::vector<BatchDesc> desc(count);
+    std::vector<BatchDesc> &desc = c.desc;
+    desc.resize(count);
     std::vector<uint32_t> blk_prob;
     std::vector<uint64_t> blk_h, blk_base;
     std::vector<uint32_t> fblk_prob;     // of the problems in c.fac
@@ -416,7 +449,7 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
     V.prob_chunk0 = d_pc0; V.prob_nchunk = d_pnc; V.prob_off = d_po;
     c.P = HxProblem{d_G64, d_d64, d_G32, d_d32, d_Gff, d_dff};
     c.total = total;
-    PD_TRY(setup_removal(c, d_binom, desc));
+    c.binom = d_binom;
 
     PD_TRY(buf.alloc(&c.part, (size_t)V.nchunks * kMaxWindow));
     PD_TRY(buf.alloc(&c.S, (size_t)count));
@@ -549,25 +582,32 @@ int build_phase_graph(ClassRun &c, int dt, int window, char *Q, char *pvc, doubl
     return rc;
 }
 
-// Buffers, start vectors and the first phase's graph of one class.  Done for
+// Vectors of one class, for every class before the removal's scratch of any.
+int alloc_vectors(ClassRun &c, const pairdiag_options &opt)
+{
+    const int m = std::min(opt.window, kMaxWindow);
+    const bool mixed = opt.precision == PD_PREC_MIXED;
+    const int64_t total = c.total;
+    const size_t es = mixed ? 4 : 8;
+    PD_TRY(c.buf.alloc(mixed ? &c.Q32 : &c.Q64, es * (size_t)m * (size_t)total));
+    PD_TRY(c.buf.alloc(mixed ? &c.p32 : &c.p64, es * (size_t)total));
+    if (mixed) {
+        PD_TRY(c.buf.alloc(&c.v64, (size_t)total));
+        PD_TRY(c.buf.alloc(&c.w64, (size_t)total));
+    }
+    return PD_OK;
+}
+
+// Start vectors and the first phase's graph of one class.  Done for
 // every class before any graph runs: the network pass of the learned start
 // frees memory, which would wait for work already running on the device.
 int prepare_class(ClassRun &c, const pairdiag_options &opt, pairdiag_mlp *mlp, double tol)
 {
     const int m = std::min(opt.window, kMaxWindow);
     const int dtype = opt.precision == PD_PREC_MIXED ? 1 : 0;
-    const int64_t total = c.total;
     cudaStream_t st = c.st;
-    DevBuf &buf = c.buf;
-    char *&Q = dtype == 1 ? c.Q32 : c.Q64;
-    char *&pv = dtype == 1 ? c.p32 : c.p64;
-    const size_t es = dtype == 1 ? 4 : 8;
-    PD_TRY(buf.alloc(&Q, es * (size_t)m * (size_t)total));
-    PD_TRY(buf.alloc(&pv, es * (size_t)total));
-    if (dtype == 1) {
-        PD_TRY(buf.alloc(&c.v64, (size_t)total));
-        PD_TRY(buf.alloc(&c.w64, (size_t)total));
-    }
+    char *Q = dtype == 1 ? c.Q32 : c.Q64;
+    char *pv = dtype == 1 ? c.p32 : c.p64;
     if (opt.start == PD_START_MLP)
         PD_TRY(batch_mlp_start(mlp, c.BB, c.count, c.omega.data(), c.n_pairs.data(), c.e_all.data(), c.G_all.data(),
                                dtype, Q, st));
@@ -610,7 +650,10 @@ int launch_class(ClassRun &c, const pairdiag_options &opt, double tol)
 }
 
 // Mixed form, after the refinement: FP64 cycles for the reopened problems.
-int continue_class(ClassRun &c, const pairdiag_options &opt, double tol)
+// make_room gives the removal's memory of every class back (all FP32 cycles are
+// enqueued by then).
+template <class F>
+int continue_class(ClassRun &c, const pairdiag_options &opt, double tol, F &&make_room)
 {
     int ctl[3] = {0, 0, 0};
     PD_CUDA(cudaMemcpyAsync(ctl, c.ctl, sizeof ctl, cudaMemcpyDeviceToHost, c.st));
@@ -618,8 +661,13 @@ int continue_class(ClassRun &c, const pairdiag_options &opt, double tol)
     c.reopened = ctl[2];
     if (c.reopened == 0) return PD_OK;
     const int m = std::min(opt.window, kMaxWindow);
-    PD_TRY(c.buf.alloc(&c.Q64, 8 * (size_t)m * (size_t)c.total));
-    PD_TRY(c.buf.alloc(&c.p64, 8 * (size_t)c.total));
+    auto alloc = [&](char **p, size_t bytes) -> int {
+        if (c.buf.alloc(p, bytes) == PD_OK) return PD_OK;
+        PD_TRY(make_room());
+        return c.buf.alloc(p, bytes);
+    };
+    PD_TRY(alloc(&c.Q64, 8 * (size_t)m * (size_t)c.total));
+    PD_TRY(alloc(&c.p64, 8 * (size_t)c.total));
     PD_CUDA(cudaMemcpyAsync(c.Q64, c.v64, 8 * (size_t)c.total, cudaMemcpyDeviceToDevice, c.st));
     const int left = std::max(0, opt.max_restarts - ctl[1]);
     PD_TRY(build_phase_graph(c, 0, m, c.Q64, c.p64, tol, 0, left, c.phase[1]));
@@ -716,10 +764,16 @@ extern "C" int pairdiag_batch_ground_state(int count, const int *omega, const in
             }
             PD_TRY(setup_class(c, opt, omega, n_pairs, e_off, g_off, e_all, G_all));
         }
+        for (auto &c : cls) PD_TRY(alloc_vectors(*c, opt));
+        for (auto &c : cls) PD_TRY(setup_removal(*c));
         for (auto &c : cls) PD_TRY(prepare_class(*c, opt, mlp, tol));
         for (auto &c : cls) PD_TRY(launch_class(*c, opt, tol));
+        auto make_room = [&]() -> int {
+            for (auto &c : cls) PD_TRY(give_back(*c));
+            return PD_OK;
+        };
         if (opt.precision == PD_PREC_MIXED)
-            for (auto &c : cls) PD_TRY(continue_class(*c, opt, tol));
+            for (auto &c : cls) PD_TRY(continue_class(*c, opt, tol, make_room));
         for (auto &c : cls) PD_CUDA(cudaStreamSynchronize(c->st));
         return PD_OK;
     }();
@@ -739,16 +793,13 @@ extern "C" int pairdiag_batch_ground_state(int count, const int *omega, const in
         int ctl[3] = {0, 0, 0};
         cudaError_t e1 = cudaMemcpyAsync(hs.data(), c.S, sizeof(BatchState) * c.count, cudaMemcpyDeviceToHost, c.st);
         if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(ctl, c.ctl, sizeof ctl, cudaMemcpyDeviceToHost, c.st);
-        std::vector<Tickets> tk(c.fac_batch.empty() ? 0 : c.fac.size());
-        if (e1 == cudaSuccess && !tk.empty())
-            e1 = cudaMemcpyAsync(tk.data(), c.fac_tk, sizeof(Tickets) * tk.size(), cudaMemcpyDeviceToHost, c.st);
         if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(c.st);
         if (e1 != cudaSuccess) {
             rc = fail(PD_ECUDA, "batch: result copy failed: %s", cudaGetErrorString(e1));
             break;
         }
-        for (const Tickets &t : tk)
-            if (t.expired) rc = fail(PD_ETIMEOUT, "batch: a wait inside a product ran out");
+        rc = read_expired(c);
+        if (rc == PD_OK && c.fac_expired) rc = fail(PD_ETIMEOUT, "batch: a wait inside a product ran out");
         if (rc != PD_OK) break;
         // kernels that ran: both graphs' prologues and every executed loop body
         // (ctl[1] counts the cycle heads: one in each prologue, one per body)

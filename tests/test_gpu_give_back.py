@@ -134,3 +134,44 @@ def test_fp32_product_of_a_truncated_fp64_handle():
         pd.pairdiag_fail_alloc(4 * DIM, 1)
         assert torch.equal(product(t), product(by_map))
         assert torch.equal(product(t), product(by_map))
+
+
+def batch(sizes, tol, **kw):
+    ps = [(o, n, *pd_inputs.separable_noise(o, seed=5 + o)) for o, n in sizes]
+    before = pd.pairdiag_kernel_launches()
+    r = pd.pairdiag_batch_ground_state(ps, tol, pd.pairdiag_default_options(precision=pd.PD_PREC_MIXED, **kw))
+    return list(r["e0"]), pd.pairdiag_kernel_launches() - before
+
+
+def scratch_bytes(sizes):
+    return 4 * sum(math.comb(o - 12, p) * p * math.comb(12, n - p) for o, n in sizes for p in range(o - 11) if p <= n)
+
+
+def vector_elements(sizes):
+    return sum((math.comb(o, n) + 3) // 4 * 4 for o, n in sizes)
+
+
+def test_batch_takes_its_vectors_before_the_scratch():
+    """The first allocation of the scratch's size or more is the FP32 window: its
+    failure is the call's.  The failure of the FP64 window makes the scratch go,
+    and the call ends as without it."""
+    sizes = [(17, 8), (18, 9), (19, 8)]
+    assert scratch_bytes(sizes) < 4 * 20 * vector_elements(sizes)
+    ref = batch(sizes, 1e-9)
+    assert ref[1] != batch(sizes, 1e-9, hx_variant=3)[1]      # two launches per FP32 product
+    pd.pairdiag_fail_alloc(scratch_bytes(sizes), 1)
+    with pytest.raises(pd.PairDiagError) as err:
+        batch(sizes, 1e-9)
+    assert err.value.code == pd.PD_ENOMEM
+    pd.pairdiag_fail_alloc(8 * 20 * vector_elements(sizes), 1)
+    assert batch(sizes, 1e-9) == ref
+
+
+def test_batch_without_the_scratch_goes_row_by_row():
+    """A window of four vectors is smaller than the scratch of C(22, 11)."""
+    sizes = [(22, 11)]
+    assert scratch_bytes(sizes) > 4 * 4 * vector_elements(sizes)
+    rows = batch(sizes, 1e-5, window=4, hx_variant=3)
+    assert batch(sizes, 1e-5, window=4)[1] != rows[1]
+    pd.pairdiag_fail_alloc(scratch_bytes(sizes), 1)
+    assert batch(sizes, 1e-5, window=4) == rows
