@@ -141,6 +141,8 @@ struct ClassRun {
     std::vector<FacProblem> fac;
     std::vector<FacBatch> fac_batch;     // one launch per tile width
     char *fac_mem = nullptr;             // their tables, scratch and counters
+    std::vector<char> fac_items;         // sources of asynchronous copies into it
+    std::vector<int2> fac_ctas_t, fac_ctas_y;
     Tickets *fac_tk = nullptr;           // [fac.size()]
     bool fac_expired = false;            // a wait inside a product gave up
     std::vector<BatchDesc> desc;
@@ -206,7 +208,7 @@ int setup_removal(ClassRun &c)
     auto share = [&](int64_t blocks, int per_cta, int64_t fill) {
         return (int)std::min<int64_t>(blocks, std::max<int64_t>((blocks + per_cta - 1) / per_cta, (fill + count - 1) / count));
     };
-    std::vector<int2> ctas_t, ctas_y;
+    std::vector<int2> &ctas_t = c.fac_ctas_t, &ctas_y = c.fac_ctas_y;
     std::vector<int> nt(count), ny(count);
     std::vector<size_t> first_t, first_y;
     c.fac_batch.clear();
@@ -249,7 +251,8 @@ int setup_removal(ClassRun &c)
     }
     char *const mem = c.fac_mem;
     c.fac_tk = reinterpret_cast<Tickets *>(mem + at_tk);
-    std::vector<char> items(item * count);
+    std::vector<char> &items = c.fac_items;
+    items.resize(item * count);
     // the uploads of binom, G and d ran on the default stream, whose order c.st
     // does not follow
     PD_CUDA(cudaStreamSynchronize(nullptr));
