@@ -13,9 +13,16 @@
 //
 // Precision.  tcgen05.mma kind::tf32 keeps 11 significant bits of an operand, so
 // V and G are split in two, v = v_hi + v_lo with v_hi = v rounded to TF32 (the
-// difference is exact), and Z = V_hi G_hi + V_lo G_hi + V_hi G_lo accumulates in
-// FP32: what is dropped is below 2^-23 of a term, and a row sum is a tree of
-// depth two instead of a chain of N (Omega - N) additions.  Elements that are
+// difference is exact), and Z = V_hi G_lo + V_lo G_hi + V_hi G_hi accumulates in
+// FP32, the small products first (the accumulator truncates: mean row error 0.189
+// -> 0.170 x 2^-23 at C(24,12) against V_hi G_hi first).  Of a term at most 4 x
+// 2^-23 is dropped: V_lo G_lo (2^-22: a low part is at most 2^-11), the last bit of
+// V_lo, which the unit cuts off, and the rounding of G_lo (2^-23 each).  A row sum
+// is a tree of depth two instead of a chain of N (Omega - N) additions, so rows are
+// more exact than row by row (norm of the error at C(24,12) 1.34e-7 / 3.23e-7,
+// C(14,7) 0.73e-7 / 1.95e-7), but not a row with one dominant hop (1.0e-7 / 0.34e-7).
+// Measured and not kept: V_lo G_lo as a fourth product, 0.56 to 0.82e-7 for such a
+// row, the same 1.34e-7 for the others, and C(30,15) 6.55 -> 6.80 ms.  Elements that are
 // not finite (or that overflow when rounded to TF32) cannot be split; a tile
 // that meets one sets a flag, and the second kernel then forms its rows term by
 // term.
@@ -381,11 +388,11 @@ __device__ __forceinline__ void issue_product(const uint32_t tmem, const uint32_
         (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(C::kN >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
     const uint64_t b0 = g_desc<KP>(g_smem);
 #pragma unroll
-    for (int s = 0; s < 3; ++s)
+    for (int s = 0; s < 3; ++s)                   // V_hi G_lo, V_lo G_hi, V_hi G_hi
 #pragma unroll
         for (int kk = 0; kk < KP / 8; ++kk) {
             const uint32_t a = tmem + (s == 1 ? KP : 0) + 8 * kk;
-            const uint64_t db = b0 + (uint64_t)(((s == 2 ? 4 * C::kN * KP : 0) + kk * 256) >> 4);
+            const uint64_t db = b0 + (uint64_t)(((s == 0 ? 4 * C::kN * KP : 0) + kk * 256) >> 4);
             const uint32_t accum = (s || kk) ? 1u : 0u;
             asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                          "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem + 2 * KP),

@@ -93,3 +93,24 @@ def test_class_by_class_vs_float_float():
         pd.pairdiag_hx_dev(a.h, pd.PD_HX_FLOATFLOAT, x.abs(), scale)
         torch.cuda.synchronize()
         assert bool(((y.double() - ref).abs() <= removal_eps(omega, n) * scale).all())
+
+
+@pytest.mark.parametrize("omega,n,i,j", [(12, 6, 1, 2), (14, 7, 12, 3), (18, 9, 16, 15), (24, 12, 1, 2), (30, 4, 29, 0)])
+def test_rows_with_one_dominant_hop(omega, n, i, j):
+    """Every other coefficient 1e-12 times smaller: the row is one term, of which
+    the split may drop 4 x 2^-23 and the FP32 rounding of G 2^-24; each of the K / 8
+    steps after the term is in the accumulator, the alignment in its own step and the
+    two additions that follow (rows, high orbits) may cut one unit in the last place,
+    2^-23, of which at most 40 / 8 + 1 + 2 are."""
+    e, G = pd_inputs.separable_noise(omega, seed=omega)
+    e, G = e * 1e-12, G * 1e-12
+    G[i, j] = G[j, i] = 0.3331111
+    b = oracle.basis(omega, n)
+    x32 = pd_inputs.random_vector(len(b), omega + n).astype(np.float32)
+    x = x32.astype(np.float64)
+    rows = ((b >> np.uint64(i)) ^ (b >> np.uint64(j))) & np.uint64(1) == 1
+    with pd.Solver(omega, n, e, G, precision=pd.PD_PREC_MIXED, hx_variant=2) as s:
+        got = product32(s, x32)
+    err = np.abs(got - oracle.hx(omega, n, e, G, x, b))[rows]
+    scale = abs_row_scale(omega, n, e, G, x, basis=b)[rows]
+    assert np.all(err <= (4.5 + 40 / 8 + 1 + 2) * 2.0 ** -23 * scale), np.max(err / scale) * 2 ** 23
