@@ -24,8 +24,8 @@
 // Measured and not kept: V_lo G_lo as a fourth product, 0.56 to 0.82e-7 for such a
 // row, the same 1.34e-7 for the others, and C(30,15) 6.55 -> 6.80 ms.  Elements that are
 // not finite (or that overflow when rounded to TF32) cannot be split; a tile
-// that meets one sets a flag, and the second kernel then forms its rows term by
-// term.
+// that meets one sets a flag, and the second kernel then forms the rows that it
+// reaches term by term.
 //
 // Layout.  Low orbits: the L <= 12 lowest; high word h, block as in
 // pd_internal.h.  remove_kernel takes one high word at a time (a block of t):
@@ -866,26 +866,31 @@ struct AddArgs {
     int first_launch, last_launch;       // of the product
 };
 
-// one row term by term (elements that are not finite), or NaN (void)
-__device__ __noinline__ float row_slow(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
-                                       const float *__restrict__ x, uint64_t s, float xs, unsigned mark)
+// One row term by term, by a warp (its hops over the lanes)
+__device__ float row_slow(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
+                          const float *__restrict__ x, uint64_t s, float xs)
 {
-    if (mark & kMarkVoid) return CUDART_NAN_F;
+    if (xs != xs) return xs;                      // NaN stays
+    const int lane = threadIdx.x & 31, M = A.omega - A.N;
     float D = 0.0f;
-    for (int p = 0; p < A.omega; ++p)
+    for (int p = lane; p < A.omega; p += 32)
         if (s >> p & 1ull) D += d[p];
-    float acc = D * xs;
-    for (int o = 0; o < A.omega; ++o) {
-        if (!(s >> o & 1ull)) continue;
-        for (int e = 0; e < A.omega; ++e) {
-            if (s >> e & 1ull) continue;
-            uint64_t t = s ^ (1ull << o) ^ (1ull << e), idx = 0;
-            int c = 0;
-            for (uint64_t w = t; w; w &= w - 1)
-                idx += __ldg(A.binom + (__ffsll((long long)w) - 1) * kBinomStride + ++c);
-            acc = fmaf(G[e * A.omega + o], x[idx], acc);
-        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
+    float acc = lane == 0 ? D * xs : 0.0f;
+    for (int i = lane; i < A.N * M; i += 32) {
+        uint64_t wo = s, we = ~s;
+        for (int j = i / M; j > 0; --j) wo &= wo - 1;
+        for (int j = i % M; j > 0; --j) we &= we - 1;
+        const int o = __ffsll((long long)wo) - 1, e = __ffsll((long long)we) - 1;
+        uint64_t idx = 0;
+        int c = 0;
+        for (uint64_t w = s ^ (1ull << o) ^ (1ull << e); w; w &= w - 1)
+            idx += __ldg(A.binom + (__ffsll((long long)w) - 1) * kBinomStride + ++c);
+        acc = fmaf(G[e * A.omega + o], x[idx], acc);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     return acc;
 }
 
@@ -906,6 +911,59 @@ __device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float>
     if (threadIdx.x == 0) *dot_out = A.first_launch ? s : *dot_out + s;
 }
 
+// The addition after a marked product (a function and a loop of its own, so that
+// the usual ones keep their registers).  An element that cannot be split makes its
+// tiles' rows of Z NaN, so exactly the rows that it reaches are not finite (and
+// those that overflow anyway): they are formed term by term, the others are as
+// usual.  C(24,12) with one such element: 12.3 ms when every row was formed that way.
+__device__ __noinline__ void add_marked(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
+                                        const float *__restrict__ x, float *__restrict__ y, Tickets *tk, double *part,
+                                        double *dot_out, const int cta, const int ctas, const uint32_t *bin, double *sred,
+                                        const unsigned mark)
+{
+    const int lane = threadIdx.x & 31, NB = A.N + 2;
+    DotAcc<float> dot;
+    int c = A.c0;
+    for (int64_t b = A.first[A.c0] + cta; b < A.first[A.c1]; b += ctas) {
+        while (b >= A.first[c + 1]) ++c;
+        const int ph = A.ph[c], k = A.N - ph;
+        const int lo_k = A.lo_off[k], nk = A.lo_off[k + 1] - lo_k;
+        const uint32_t h = __ldg(A.words + b);
+        uint32_t base = 0;
+        float Dh = 0.0f;
+        int o = k;
+        for (uint32_t w = h; w; w &= w - 1) {
+            const int j = __ffs(w) - 1;
+            base += bin[j * NB + ++o];
+            Dh += d[A.L + j];
+        }
+        const float *z = A.scratch + A.zbase[k] + (b - A.first[c]) * (int64_t)ph * nk;
+#pragma unroll 1
+        for (int r0 = threadIdx.x & ~31; r0 < nk; r0 += kAThreads) {      // whole warps
+            const bool in = r0 + lane < nk;
+            const int r = in ? r0 + lane : nk - 1;
+            const float xr = __ldg(x + base + r);
+            float acc = k == 0 ? Dh * xr : y[base + r];                   // (no pair removal writes rows with k = 0)
+            const float *zr = z + r;
+#pragma unroll 4
+            for (int a = 0; a < ph; ++a, zr += nk) acc += __ldcs(zr);
+            if (mark & kMarkVoid) acc = CUDART_NAN_F;
+            const uint64_t s = (uint64_t)h << A.L | __ldg(A.low + lo_k + r);
+            const bool again = in && !(mark & kMarkVoid) && !isfinite(acc);
+            for (unsigned m = __ballot_sync(0xffffffffu, again); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const float v = row_slow(A, G, d, x, __shfl_sync(0xffffffffu, s, src), __shfl_sync(0xffffffffu, xr, src));
+                if (lane == src) acc = v;
+            }
+            __syncwarp();
+            if (!in) continue;
+            y[base + r] = acc;
+            dot.add(xr, acc);
+        }
+    }
+    finish_add(A, dot, tk, part, dot_out, sred, ctas);
+}
+
 // y(h, l) += sum over the pairs a of h of scratch(h, a, l); fused x^T y.  Bound
 // by the latency of streaming reads: 16 loads per thread in flight, small CTAs
 // so that blocks of very different sizes balance.  Omega=24 (65 MB of scratch,
@@ -923,6 +981,10 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
         bin[i] = (uint32_t)__ldg(A.binom + (A.L + i / NB) * kBinomStride + i % NB);
     const unsigned mark = __ldcg(&tk->mark);
     __syncthreads();
+    if (mark) {
+        add_marked(A, G, d, x, y, tk, part, dot_out, cta, ctas, bin, sred, mark);
+        return;
+    }
     DotAcc<float> dot;
     int c = A.c0;
     int64_t b = A.first[A.c0] + cta;
@@ -944,16 +1006,6 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
             Dh = occ ? d[A.L + lane] : 0.0f;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) Dh += __shfl_xor_sync(0xffffffffu, Dh, o);
-        }
-        if (mark) {                               // (in a loop of its own: the call costs the other one registers)
-#pragma unroll 1
-            for (int r = threadIdx.x; r < nk; r += kAThreads) {
-                const float xr = __ldg(x + base + r);
-                const float acc = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr, mark);
-                y[base + r] = acc;
-                if (part) dot.add(xr, acc);
-            }
-            continue;
         }
         for (int r0 = threadIdx.x; r0 < nk; r0 += kARows * kAThreads) {
             float acc[kARows], xr[kARows];
@@ -1024,6 +1076,10 @@ add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G,
     for (int i = threadIdx.x; i < A.H; i += kAThreads) dh[i] = d[A.L + i];
     const unsigned mark = __ldcg(&tk->mark);
     __syncthreads();
+    if (mark) {
+        add_marked(A, G, d, x, y, tk, part, dot_out, blockIdx.x, gridDim.x, bin, sred, mark);
+        return;
+    }
     DotAcc<float> dot;
     for (int c = A.c0; c < A.c1; ++c) {
         const int ph = A.ph[c], k = A.N - ph;
@@ -1040,12 +1096,11 @@ add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G,
                 base += bin[j * NB + ++o];
                 Dh += dh[j];
             }
-            const float xr = part || k == 0 || mark ? __ldg(x + base) : 0.0f;
+            const float xr = part || k == 0 ? __ldg(x + base) : 0.0f;
             float acc = k == 0 ? Dh * xr : y[base];
             const float *z = A.scratch + A.zbase[k] + (int64_t)b * ph * nk + r;
 #pragma unroll 4
             for (int a = 0; a < ph; ++a, z += nk) acc += __ldg(z);
-            if (mark) acc = row_slow(A, G, d, x, (uint64_t)h << A.L | __ldg(A.low + lo_k + r), xr, mark);
             y[base] = acc;
             if (part) dot.add(xr, acc);
         }
