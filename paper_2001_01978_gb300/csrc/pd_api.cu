@@ -1652,8 +1652,10 @@ int pairdiag_autotune(int omega, int n_pairs, const double *e, const double *G, 
             pairdiag_t *h = nullptr;
             if ((rc = pairdiag_create(omega, n_pairs, e, G, &o, &h)) != PD_OK) break;
             // the variant does not fit: the launch would run another one; variant 2
-            // has a block split of its own, so it is timed once
-            const bool same = variant == 2 ? precision != PD_PREC_MIXED || !h->fac.on || L != h->fac.L
+            // has a block split of its own, so it is timed once, and only where its
+            // rows are no less exact than the others'
+            const bool same = variant == 2 ? precision != PD_PREC_MIXED || !h->fac.on || L != h->fac.L ||
+                                                 !fac_exact(omega, n_pairs, dim)
                                            : variant > 1 && hx_variant(h->B, precision == PD_PREC_FP64 ? 0 : 1) != variant;
             if (same) {
                 pairdiag_destroy(h);

@@ -1196,12 +1196,24 @@ bool fac_fits(int omega, int n, int64_t dim)
            layout_r(padded(omega), H, n).total <= kSmemMax;
 }
 
-// Where variant 2 is the faster one and no less exact (variant 3 / variant 2,
-// FP32, back to back): C(17,6) 15.7 / 18.5 us, C(18,9) = 48620 18.7 / 20.6 us,
-// C(20,10) = 184756 31 / 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 6.5 ms,
-// C(34,9) 12.8 / 1.7 ms.  Far above half filling there are more words t than
-// states and their rows are longer: C(24,16) 94 / 64 us, C(24,18) 48 / 41 us,
-// C(28,22) 141 / 211 us, and C(20,17) loses accuracy (2.2e-7 / 2.6e-7).
+// Where the rows of variant 2 have been at least as exact as row by row in every
+// draw (norm of the error against 64-bit rows, removal / rows).  Up to two thirds of
+// the orbits occupied (rounded up) everywhere: C(14,7) 0.7 / 2.0e-7, C(24,12) 1.3 /
+// 3.2e-7.  Above that from 30000 states on: means of six draws C(24,19) 2.0 / 3.1e-7,
+// C(34,30) 2.4 / 3.8e-7; in smaller spaces the mean is lower too (C(22,19) 2.0 /
+// 2.6e-7, C(24,20) 2.2 / 2.9e-7, C(30,26) 2.5 / 2.7e-7), but one or two of the six
+// draws were higher.
+bool fac_exact(int omega, int n, int64_t dim)
+{
+    return dim >= 30000 || 3 * n <= 2 * omega + 2;
+}
+
+// Where variant 2 is taken unasked (FP32, rows / removal, a cold L2 before each):
+// C(17,6) 15.7 / 18.5 us, C(18,9) = 48620 18.7 / 20.6 us, C(20,10) = 184756 31 /
+// 22.6 us, C(24,12) 215 / 96 us, C(30,15) 16.5 / 6.5 ms, C(34,9) 12.8 / 1.7 ms.  Up
+// to two thirds filling (rounded up); above, it is taken on request and by the
+// autotuner, which finds it the faster one in large spaces there too: C(22,16) 46 /
+// 31 us, C(24,17) 134 / 64 us, C(24,18) 54 / 54 us, C(28,22) 146 / 97 us.
 bool fac_pays(int omega, int n, int64_t dim)
 {
     return dim >= 60000 && 3 * n <= 2 * omega + 2 && fac_fits(omega, n, dim);

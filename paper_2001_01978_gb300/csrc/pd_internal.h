@@ -353,12 +353,14 @@ cudaError_t kept_scatter_launch(int dtype, const uint64_t *full, int64_t n, cons
                                 const int *skip);
 cudaError_t kept_list_launch(const Blocks &B, const int32_t *map, uint64_t *full, uint16_t *low, int grid,
                              cudaStream_t st);
-// variant 2 (pd_hxf.cu).  fac_fits: whether it serves a problem; fac_sizes: the
+// variant 2 (pd_hxf.cu).  fac_fits: whether it serves a problem, fac_exact: with rows
+// no less exact than row by row, fac_pays: faster as well; fac_sizes: the
 // lengths of the device arrays, which the caller allocates; fac_build fills them.
 // fac_partials: doubles that a fused dot needs in blk_part.  fac_launch: as
 // hx_launch for FP32.
 int fac_low(int omega);
 bool fac_fits(int omega, int n, int64_t dim);
+bool fac_exact(int omega, int n, int64_t dim);
 bool fac_pays(int omega, int n, int64_t dim);
 void fac_sizes(int omega, int n, FacPlan &p);
 size_t fac_zeros();
