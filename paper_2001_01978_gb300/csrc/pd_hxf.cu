@@ -919,7 +919,7 @@ __device__ __forceinline__ void finish_add(const AddArgs &A, const DotAcc<float>
 __device__ __noinline__ void add_marked(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
                                         const float *__restrict__ x, float *__restrict__ y, Tickets *tk, double *part,
                                         double *dot_out, const int cta, const int ctas, const uint32_t *bin, double *sred,
-                                        const unsigned mark)
+                                        const unsigned mark, const bool tree)
 {
     const int lane = threadIdx.x & 31, NB = A.N + 2;
     DotAcc<float> dot;
@@ -936,6 +936,11 @@ __device__ __noinline__ void add_marked(const AddArgs &A, const float *__restric
             const int j = __ffs(w) - 1;
             base += bin[j * NB + ++o];
             Dh += d[A.L + j];
+        }
+        if (tree) {                               // (in the order of the kernel that this one stands in for)
+            Dh = h >> lane & 1u ? d[A.L + lane] : 0.0f;
+#pragma unroll
+            for (int p = 16; p > 0; p >>= 1) Dh += __shfl_xor_sync(0xffffffffu, Dh, p);
         }
         const float *z = A.scratch + A.zbase[k] + (b - A.first[c]) * (int64_t)ph * nk;
 #pragma unroll 1
@@ -982,7 +987,7 @@ __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__rest
     const unsigned mark = __ldcg(&tk->mark);
     __syncthreads();
     if (mark) {
-        add_marked(A, G, d, x, y, tk, part, dot_out, cta, ctas, bin, sred, mark);
+        add_marked(A, G, d, x, y, tk, part, dot_out, cta, ctas, bin, sred, mark, true);
         return;
     }
     DotAcc<float> dot;
@@ -1077,7 +1082,7 @@ add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G,
     const unsigned mark = __ldcg(&tk->mark);
     __syncthreads();
     if (mark) {
-        add_marked(A, G, d, x, y, tk, part, dot_out, blockIdx.x, gridDim.x, bin, sred, mark);
+        add_marked(A, G, d, x, y, tk, part, dot_out, blockIdx.x, gridDim.x, bin, sred, mark, false);
         return;
     }
     DotAcc<float> dot;

@@ -21,8 +21,8 @@ def neighbours(omega, n, index):
     return np.array([bin(int(v)).count("1") <= 2 for v in w])
 
 
-# one set of blocks; the kernels of small blocks
-@pytest.mark.parametrize("omega,n", [(18, 9), (30, 4)])
+# one set of blocks, without and with rows of no low pairs; the kernels of small blocks
+@pytest.mark.parametrize("omega,n", [(18, 9), (22, 5), (30, 4)])
 @pytest.mark.parametrize("value", [np.inf, np.nan])
 def test_rows_it_does_not_reach(omega, n, value):
     e, G = pd_inputs.separable_noise(omega, seed=1)
