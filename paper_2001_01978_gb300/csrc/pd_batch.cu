@@ -464,6 +464,30 @@ int setup_class(ClassRun &c, const pairdiag_options &opt, const int *omega, cons
     return PD_OK;
 }
 
+// One product of every problem whose skip flag is not set.  FP32: the larger
+// problems by pair removal, the others row by row.
+struct Product {
+    int dt;
+    bool removal;
+    BatchBlocks rest;
+    int rest_grid;
+    Product(const ClassRun &c, int dtype) : dt(dtype), removal(dtype == 1 && !c.fac_batch.empty()), rest(c.BB)
+    {
+        if (removal) rest.nblocks = c.rest_blocks;
+        rest_grid = rest.nblocks > 0 ? hx_batch_grid(rest, dt) : 0;
+    }
+    int launch(const ClassRun &c, const void *x, void *y, cudaStream_t st) const
+    {
+        const int *skip = &c.S[0].skip;
+        const int stride = (int)(sizeof(BatchState) / sizeof(int));
+        if (removal)
+            for (const FacBatch &b : c.fac_batch)
+                PD_CUDA(fac_batch_launch(b, (const float *)x, (float *)y, st, skip, stride));
+        if (rest.nblocks > 0) PD_CUDA(hx_batch_launch(rest, c.P, dt, x, y, c.counter, rest_grid, st, skip, stride));
+        return PD_OK;
+    }
+};
+
 // Restarted Lanczos of every problem of the class that is not done, on storage
 // type dt, as one graph: prologue + WHILE(cycle).  Q_0 of the window holds the
 // start vectors.  The graph is built here and launched on the class's stream.
@@ -475,30 +499,15 @@ int build_phase_graph(ClassRun &c, int dt, int window, char *Q, char *pvc, doubl
     const size_t es = dt == 0 ? 8 : 4;
     const int64_t total = c.total;
     const BatchVec &V = c.V;
-    const BatchBlocks &BB = c.BB;
     BatchState *S = c.S;
     double *part = c.part;
     void *pv = pvc;
-    const int *skip = &S[0].skip;
-    const int skip_stride = (int)(sizeof(BatchState) / sizeof(int));
     const int sd = (int)(sizeof(BatchState) / sizeof(double));
     auto q = [&](int j) { return (void *)(Q + es * (size_t)j * (size_t)total); };
     cudaStream_t cs = nullptr;                    // the capturing stream
-    // FP32: the larger problems' products by pair removal, the others' row by row
-    const bool removal = dt == 1 && !c.fac_batch.empty();
-    BatchBlocks rest = BB;
-    if (removal) rest.nblocks = c.rest_blocks;
-    const int rest_grid = rest.nblocks > 0 ? hx_batch_grid(rest, dt) : 0;
-    auto product = [&](int i) -> int {
-        if (removal)
-            for (const FacBatch &b : c.fac_batch)
-                PD_CUDA(fac_batch_launch(b, (const float *)q(i), (float *)pv, cs, skip, skip_stride));
-        if (rest.nblocks > 0)
-            PD_CUDA(hx_batch_launch(rest, c.P, dt, q(i), pv, c.counter, rest_grid, cs, skip, skip_stride));
-        return PD_OK;
-    };
+    const Product product(c, dt);
     auto step = [&](int i) -> int {
-        PD_TRY(product(i));
+        PD_TRY(product.launch(c, q(i), pv, cs));
         PD_CUDA(seg_dots_launch(dt, V, q(i), total, 1, pv, S, part, &S[0].c1, sd, cs));
         PD_CUDA(seg_recur_project_launch(dt, V, Q, total, i, pv, S, part, cs));
         PD_CUDA(seg_update_launch(dt, V, Q, total, i + 1, pv, S, part, cs));
@@ -679,6 +688,46 @@ int continue_class(ClassRun &c, const pairdiag_options &opt, double tol, F &&mak
 }
 
 }  // namespace
+
+// For the tests (not in the header): `reps` FP32 products y = H x of every problem
+// as the batched solver launches them.  x, y: host, the problems one after the
+// other, each on a 4-element boundary; skip: host [count], problems to leave out;
+// by_removal: how many go by pair removal.
+extern "C" int pairdiag_batch_product_for_tests(int count, const int *omega, const int *n_pairs, const double *e_all,
+                                                const double *G_all, const pairdiag_options *opt, int reps,
+                                                const float *x, float *y, const int *skip, int *by_removal)
+{
+    std::vector<int64_t> e_off(count), g_off(count);
+    int64_t eo = 0, go = 0;
+    ClassRun c;
+    c.count = count;
+    for (int p = 0; p < count; ++p) {
+        c.prob.push_back(p);
+        e_off[p] = eo;
+        g_off[p] = go;
+        eo += omega[p];
+        go += (int64_t)omega[p] * omega[p];
+    }
+    PD_TRY(setup_class(c, *opt, omega, n_pairs, e_off, g_off, e_all, G_all));
+    PD_TRY(setup_removal(c));
+    *by_removal = (int)c.fac.size();
+    float *dx = nullptr, *dy = nullptr;
+    PD_TRY(c.buf.alloc(&dx, (size_t)c.total));
+    PD_TRY(c.buf.alloc(&dy, (size_t)c.total));
+    std::vector<BatchState> S(count);
+    memset(S.data(), 0, sizeof(BatchState) * S.size());
+    for (int p = 0; p < count; ++p) S[p].skip = skip[p];
+    PD_CUDA(cudaMemcpy(c.S, S.data(), sizeof(BatchState) * S.size(), cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemcpy(dx, x, sizeof(float) * (size_t)c.total, cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemset(dy, 0xff, sizeof(float) * (size_t)c.total));       // NaN
+    const Product product(c, 1);
+    for (int r = 0; r < reps; ++r) PD_TRY(product.launch(c, dx, dy, c.st));
+    PD_CUDA(cudaStreamSynchronize(c.st));
+    PD_TRY(read_expired(c));
+    if (c.fac_expired) return fail(PD_ETIMEOUT, "batch: a wait inside a product ran out");
+    PD_CUDA(cudaMemcpy(y, dy, sizeof(float) * (size_t)c.total, cudaMemcpyDeviceToHost));
+    return PD_OK;
+}
 
 extern "C" int pairdiag_batch_ground_state(int count, const int *omega, const int *n_pairs, const double *e_all,
                                            const double *G_all, double tol, const pairdiag_options *opt_in,

@@ -114,3 +114,27 @@ def test_rows_with_one_dominant_hop(omega, n, i, j):
     err = np.abs(got - oracle.hx(omega, n, e, G, x, b))[rows]
     scale = abs_row_scale(omega, n, e, G, x, basis=b)[rows]
     assert np.all(err <= (4.5 + 40 / 8 + 1 + 2) * 2.0 ** -23 * scale), np.max(err / scale) * 2 ** 23
+
+
+def test_class_by_class_40_columns():
+    """C(38, 10), 4.7e8 states: tiles of 40 columns, one set of partial results,
+    classes with small blocks in launches of their own; every row against the
+    float-float product."""
+    omega, n = 38, 10
+    e, G = pd_inputs.separable_noise(omega, seed=4)
+    d = 2.0 * e + np.diag(G)
+    with pd.Solver(omega, n, e, G, precision=pd.PD_PREC_MIXED) as s, \
+            pd.Solver(omega, n, (np.abs(d) - np.abs(np.diag(G))) / 2.0, np.abs(G)) as a:
+        gen = torch.Generator(device="cuda").manual_seed(7)
+        x = torch.randn(s.dim, dtype=torch.float32, device="cuda", generator=gen)
+        y = torch.full_like(x, float("nan"))
+        pd.pairdiag_hx_dev(s.h, pd.PD_PREC_MIXED, x, y)
+        err = torch.empty(s.dim, dtype=torch.float64, device="cuda")
+        pd.pairdiag_hx_dev(s.h, pd.PD_HX_FLOATFLOAT, x, err)
+        torch.cuda.synchronize()
+        err.sub_(y).abs_()
+        del y
+        scale = torch.empty_like(err)
+        pd.pairdiag_hx_dev(a.h, pd.PD_HX_FLOATFLOAT, x.abs_(), scale)
+        torch.cuda.synchronize()
+        assert bool((err <= scale.mul_(removal_eps(omega, n))).all())
