@@ -93,7 +93,8 @@ typedef struct {
                                CTAs per SM (fewer registers, more warps).  Variant 2 falls
                                back to 3 where it does not apply (more than 40 orbits, 2^32
                                states or more, no or only full orbits, no room for its
-                               scratch), 2-5 fall back to 1 when their shared memory does not
+                               scratch, or its tables beyond shared memory: 32 orbits with
+                               27 to 31 pairs), 2-5 fall back to 1 when their shared memory does not
                                fit.  A truncated handle (pairdiag_truncate) computes its kept
                                rows by variant 3 on x spread over the full space (2-5; 8 bytes
                                per state of the full space, 4 more for FP32 products, 10 per

@@ -1314,11 +1314,6 @@ cudaError_t launch_ff(const Blocks &B, const FF *G, const FF *d, const float *x,
 
 }  // namespace
 
-size_t hx_smem_bytes(const Blocks &B, int precision)
-{
-    return precision == 0 ? kernel_smem<double, double>(B) : kernel_smem<float, float>(B);
-}
-
 int hx_variant(const Blocks &B, int precision)
 {
     if (precision == 0 ? use_v3<double, double>(B) : use_v3<float, float>(B)) return B.variant == 2 ? 3 : B.variant;

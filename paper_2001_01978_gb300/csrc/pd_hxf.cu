@@ -57,8 +57,8 @@ constexpr int kRows = 924;               // most rows of a block: C(12,6)
 constexpr int kSpare = kRows;            // slot of hops that do not exist (reads 0, writes ignored)
 constexpr int kStride = 928;             // floats per orbit of the partial results
 // Scratch (floats): all rows at once up to 2 GiB, else class by class (the rows
-// with k low pairs, k ascending), which bounds it at the largest class: 1.2 GB
-// instead of 5.2 GB at Omega=30, 5 GB instead of 22 GB at Omega=32.  Measured,
+// with k low pairs, k ascending), which bounds it at the largest class: 1.62 GB
+// instead of 5.58 GB at Omega=30, 6.83 GB instead of 24.0 GB at Omega=32.  Measured,
 // when the line was drawn, at once / by class: Omega=24 0.096 / 0.28 ms (26 short launches), Omega=28
 // 1.79 / 1.97 ms, Omega=30 7.45 / 7.36 ms.
 constexpr int64_t kScratchAll = (int64_t)2048 << 18;
@@ -854,7 +854,6 @@ constexpr int kACtas = 10;               // CTAs per SM
 struct AddArgs {
     int omega, N, L, H;
     int lo_off[kLT + 2];
-    int nclass;
     int ph[kLT + 1];
     int64_t first[kLT + 2];              // number of the class's first word in words
     int c0, c1;                          // classes of this launch
@@ -1334,7 +1333,6 @@ static void fill_args(const FacPlan &p, const uint64_t *binom, WordClasses &ct, 
     R.zeros = p.zeros;
     A.scratch = p.scratch;
     A.words = p.ywords;
-    A.nclass = cy.n;
     for (int i = 0; i < cy.n; ++i) A.ph[i] = cy.ph[i];
     for (int i = 0; i <= cy.n; ++i) A.first[i] = cy.first[i];
     int64_t z = 0;

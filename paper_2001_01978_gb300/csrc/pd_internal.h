@@ -331,7 +331,6 @@ struct HxProblem {
 cudaError_t hx_batch_launch(const BatchBlocks &BB, const HxProblem &P, int precision, const void *x, void *y,
                             unsigned long long *counter, int grid, cudaStream_t st, const int *skip, int skip_stride);
 int hx_batch_grid(const BatchBlocks &BB, int precision);
-size_t hx_smem_bytes(const Blocks &B, int precision);
 int hx_variant(const Blocks &B, int precision);   // kernel variant hx_launch will use
 // y = H x (Eq. 2 in the pair basis) over the persistent grid.
 // skip (nullable, device): when *skip != 0 the launched kernels return at once.
