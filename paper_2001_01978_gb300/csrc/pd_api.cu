@@ -169,7 +169,7 @@ struct pairdiag {
     unsigned char *d_fac = nullptr;  // its tables and scratch
     int device = 0;
     cudaStream_t st = nullptr;
-    // tables, one allocation
+    // tables, counters and partial sums, one allocation
     unsigned char *d_tables = nullptr;
     uint64_t *d_blk_h = nullptr, *d_blk_base = nullptr, *d_binom = nullptr;
     uint16_t *d_lowword = nullptr, *d_rankL = nullptr;
@@ -222,8 +222,7 @@ void free_all(pairdiag *h)
         cudaEventDestroy(ev.second);
     }
     h->hx_events.clear();
-    void *ptrs[] = {h->d_tables, h->d_tk, h->d_blkdot, h->d_part, h->d_S, h->d_small,
-                    h->d_Q[0], h->d_Q[1], h->d_p[0], h->d_p[1], h->d_v64, h->d_w64,
+    void *ptrs[] = {h->d_tables, h->d_Q[0], h->d_Q[1], h->d_p[0], h->d_p[1], h->d_v64, h->d_w64,
                     h->d_L64, h->d_L32, h->d_lockc, h->d_kmap, h->d_kblk_h, h->d_kblk_base, h->d_kblk_first,
                     h->d_kblk_rows, h->d_kfull, h->d_klow, h->d_xf[0], h->d_xf[1],
                     h->d_fac};
@@ -305,7 +304,16 @@ int build_tables(pairdiag *h)
                  at_lw = place(2 * nL), at_rk = place(2 * nL), at_bin = place(8 * 64 * 64), at_G = place(8 * no * no),
                  at_d = place(8 * no), at_G32 = place(4 * no * no), at_d32 = place(4 * no), at_Gff = place(8 * no * no),
                  at_dff = place(8 * no);
-    std::unique_ptr<unsigned char[]> host(new unsigned char[bytes]);
+    const size_t host_bytes = bytes;
+    // Counters and partial sums beside them: with an allocation each, the products
+    // inside FP64 solves of C(18,8) took 25 to 32 us by where these happened to lie
+    // (nine handles, mean 28.4), in one block 24.4 to 28 (25.7)
+    h->rgrid = (int)std::min<int64_t>(nblocks, vec_grid());
+    h->part_count = (size_t)std::max(vec_grid(), h->rgrid) * kMaxWindow;
+    const size_t at_tk = place(sizeof(Tickets)), at_S = place(sizeof(LanczosScalars)), at_small = place(8 * 8),
+                 at_dot = place(8 * std::max<size_t>(nb, h->use_fac ? (size_t)fac_partials() : 0)),
+                 at_part = place(8 * h->part_count);
+    std::unique_ptr<unsigned char[]> host(new unsigned char[host_bytes]);
     auto at = [&](auto *type, size_t off) { return reinterpret_cast<decltype(type)>(host.get() + off); };
     uint64_t *hw = at((uint64_t *)nullptr, at_h), *base = at((uint64_t *)nullptr, at_b);
     // blocks by ascending high word, each starting where the last one ends
@@ -369,7 +377,8 @@ int build_tables(pairdiag *h)
     coefficients(h->d, at_d, at_d32, at_dff);
 
     PD_TRY(dalloc(&h->d_tables, bytes));
-    PD_CUDA(cudaMemcpy(h->d_tables, host.get(), bytes, cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemcpy(h->d_tables, host.get(), host_bytes, cudaMemcpyHostToDevice));
+    PD_CUDA(cudaMemsetAsync(h->d_tables + at_tk, 0, at_small - at_tk, h->st));
     auto dev = [&](auto *&p, size_t o) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(h->d_tables + o); };
     dev(h->d_blk_h, at_h);
     dev(h->d_blk_base, at_b);
@@ -386,6 +395,11 @@ int build_tables(pairdiag *h)
     dev(h->d_d32, at_d32);
     dev(h->d_Gff, at_Gff);
     dev(h->d_dff, at_dff);
+    dev(h->d_tk, at_tk);
+    dev(h->d_S, at_S);
+    dev(h->d_small, at_small);
+    dev(h->d_blkdot, at_dot);
+    dev(h->d_part, at_part);
 
     Blocks &B = h->B;
     B.omega = omega; B.n = N; B.L = L; B.H = H;
@@ -1058,17 +1072,8 @@ int pairdiag_create(int omega, int n_pairs, const double *e, const double *G,
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { cudaGetLastError(); st = fail(PD_ECUDA, "no CUDA device"); break; }
         if ((st = build_tables(h)) != PD_OK) break;
-        if ((st = dalloc(&h->d_tk, 1)) != PD_OK) break;
-        if (cudaMemset(h->d_tk, 0, sizeof(Tickets)) != cudaSuccess) { st = fail(PD_ECUDA, "memset"); break; }
-        if ((st = dalloc(&h->d_blkdot, (size_t)std::max<int64_t>(h->B.nblocks, use_fac ? fac_partials() : 0))) != PD_OK) break;
         h->ldq = (h->dim + 3) / 4 * 4;
         set_grids(h);
-        h->rgrid = (int)std::min<int64_t>(h->B.nblocks, vec_grid());
-        h->part_count = (size_t)std::max(vec_grid(), h->rgrid) * kMaxWindow;
-        if ((st = dalloc(&h->d_part, h->part_count)) != PD_OK) break;
-        if ((st = dalloc(&h->d_S, 1)) != PD_OK) break;
-        if ((st = dalloc(&h->d_small, 8)) != PD_OK) break;
-        if (cudaMemset(h->d_S, 0, sizeof(LanczosScalars)) != cudaSuccess) { st = fail(PD_ECUDA, "memset"); break; }
         // the removal's scratch last, after all that the handle cannot do without
         if (use_fac && (st = build_fac(h)) != PD_OK) break;
         // (the caller may go on with a stream that does not follow this one)

@@ -155,7 +155,7 @@ struct Tickets {
     unsigned long long hx_done;      // CTAs of that launch that have finished
     unsigned long long vec_done;     // CTAs of a streaming kernel whose partial sums are written
     unsigned int mark;               // variant 2, one product: kMark* bits
-    GridBar bar;                     // the fused Lanczos step's barriers
+    alignas(32) GridBar bar;         // the fused Lanczos step's barriers (one sector)
     int expired;                     // variant 2: a wait of a product gave up (stays set until a solve
                                      // starts; follows bar.err, so that one copy reads both)
 };
