@@ -407,9 +407,9 @@ __device__ __forceinline__ void issue_product(const uint32_t tmem, const uint32_
 // share an SM's tensor memory, so that one group's gathers overlap another's
 // product; the high orbits of the next tile are loaded while the product runs;
 // the ninth (thirteenth) warp prepares the next block's pointers.  Omega=24:
-// 75 us alone with a cold cache for 3.9e8 hops (46e6 warp instructions, 0.55 of
+// 78 us alone with a cold cache for 3.9e8 hops (47e6 warp instructions, 0.54 of
 // the issue slots), where the row-by-row kernel (pd_hx.cu, variant 3) took
-// 215 us; both kernels together 0.0945 ms.  Measured and not kept: FP32
+// 215 us; both kernels together 0.0964 ms.  Measured and not kept: FP32
 // multiply-adds instead of the tensor cores (packed pairs, coefficients from
 // shared memory or the constant bank, 8, 10 or 12 low orbits, hops between high
 // orbits in registers): 0.127 to 0.18 ms.
@@ -656,8 +656,8 @@ __host__ __device__ inline LayoutS layout_s(int KP, int H, int N)
 
 // What bounds it: the latency of an item's chain (starts of the blocks, gather,
 // product, scatter, rows: about 8 us), of which only four overlap per SM, because
-// the operands of four tiles fill its tensor memory.  Omega=34, N=9: 0.73 ms for
-// these blocks and 0.57 ms for the others, against 5.1 ms for both in
+// the operands of four tiles fill its tensor memory.  Omega=34, N=9: 0.72 ms for
+// these blocks and 0.51 ms for the others, against 5.1 ms for both in
 // remove_kernel.  Measured and not kept: the rows' sums over the set bits of a
 // low word instead of twelve predicated loads, 0.76 ms.
 template <int KP>
@@ -971,8 +971,8 @@ __device__ __noinline__ void add_marked(const AddArgs &A, const float *__restric
 // y(h, l) += sum over the pairs a of h of scratch(h, a, l); fused x^T y.  Bound
 // by the latency of streaming reads: 16 loads per thread in flight, small CTAs
 // so that blocks of very different sizes balance.  Omega=24 (65 MB of scratch,
-// mostly in L2): 25 us alone with a cold cache, against 32 us with 256 threads
-// and 40 us with two rows per thread.
+// mostly in L2): 23 us alone with a cold cache; 25 us before the rows of marked
+// products left its loop, 32 us then with 256 threads, 40 us with two rows per thread.
 __device__ __forceinline__ void add_blocks(const AddArgs &A, const float *__restrict__ G, const float *__restrict__ d,
                                            const float *__restrict__ x, float *__restrict__ y, Tickets *tk, double *part,
                                            double *dot_out, const int cta, const int ctas)
@@ -1062,8 +1062,8 @@ add_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const
 // The rows of classes with small blocks (at most kAddSmall rows): one thread per
 // row, numbered through the class, where add_kernel has one block per CTA and
 // pass.  Omega=34, N=9 (990,000 blocks of 1, 12 and 66 rows): 0.18 ms for these
-// rows and 0.26 ms for the others, against 1.68 ms for both in add_kernel; 445 us
-// for 1.6 GB is 0.55 of the measured copy rate, the scattered y rows included.
+// rows and 0.22 ms for the others, against 1.68 ms for both in add_kernel; 396 us
+// for 1.6 GB is 0.61 of the measured copy rate, the scattered y rows included.
 constexpr int kAddSmall = 66;
 __global__ void __launch_bounds__(kAThreads, kACtas)
 add_small_kernel(const __grid_constant__ AddArgs A, const float *__restrict__ G, const float *__restrict__ d,
