@@ -540,7 +540,7 @@ int pairdiag_set_step_fusion(pairdiag_t *h, int on);
 
 /*
  * Bound of each wait inside the handle's FP32 product by pair removal, in polls
- * of up to a millisecond (default 2^12; at most 2^20).  When one runs out, a
+ * of up to a millisecond (default 2^14; at most 2^20).  When one runs out, a
  * solve returns PD_ETIMEOUT and a single product leaves NaN in y; a solve after
  * that starts afresh.  0: the first wait gives up at once (a test of that path).
  */

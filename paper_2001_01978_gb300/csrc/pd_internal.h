@@ -110,7 +110,7 @@ struct FacPlan {
     bool by_class = false;               // the rows of one class (low pairs) at a time
     int64_t scratch_len = 0;             // floats of scratch
     int grid_t = 0, grid_y = 0;
-    int polls = 1 << 12;                 // of a wait, each suspended up to a millisecond
+    int polls = 1 << 14;                 // of a wait, each suspended up to a millisecond
     size_t smem = 0;
     uint32_t *twords = nullptr, *ywords = nullptr;   // device
     uint16_t *low = nullptr;             // [2^L] low words

@@ -27,7 +27,7 @@ def test_rows_of_an_expired_product_are_nan(omega, n):
         pd.pairdiag_hx_dev(s.h, pd.PD_PREC_MIXED, x, y)
         torch.cuda.synchronize()
         assert bool(torch.isnan(y).all())
-        pd.pairdiag_set_wait_limit(s.h, 1 << 12)
+        pd.pairdiag_set_wait_limit(s.h, 1 << 14)
         pd.pairdiag_hx_dev(s.h, pd.PD_PREC_MIXED, x, y)
         torch.cuda.synchronize()
         assert torch.equal(y, good)
@@ -40,13 +40,13 @@ def test_a_solve_reports_its_own_waits_only():
         x = torch.ones(math.comb(omega, n), dtype=torch.float32, device="cuda")
         pd.pairdiag_set_wait_limit(s.h, 0)
         pd.pairdiag_hx_dev(s.h, pd.PD_PREC_MIXED, x, torch.empty_like(x))
-        pd.pairdiag_set_wait_limit(s.h, 1 << 12)
+        pd.pairdiag_set_wait_limit(s.h, 1 << 14)
         first = pd.pairdiag_ground_state_dev(s.h, 1e-6)       # not failed by the product before it
         pd.pairdiag_set_wait_limit(s.h, 0)
         with pytest.raises(pd.PairDiagError, match="pair removal") as err:
             pd.pairdiag_ground_state_dev(s.h, 1e-6)
         assert err.value.code == pd.PD_ETIMEOUT
-        pd.pairdiag_set_wait_limit(s.h, 1 << 12)
+        pd.pairdiag_set_wait_limit(s.h, 1 << 14)
         assert pd.pairdiag_ground_state_dev(s.h, 1e-6)["e0"] == first["e0"]
 
 
